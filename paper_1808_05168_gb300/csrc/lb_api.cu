@@ -114,7 +114,7 @@ struct lb_ctx {
   bool tma = false;                // d_tmaps holds maps for the current tile
   int* d_err = nullptr;
   double* d_scratch = nullptr;  // 18 * max_lattice_sites doubles (populations I/O)
-  double* d_mass = nullptr;
+  double* d_mass = nullptr;     // lb_mass (MASS_BUF doubles)
   size_t bytes = 0;
 
   std::vector<DiagLattice> diag;
@@ -922,14 +922,15 @@ int create_impl(lb_ctx** out, int n, const lb_params* ps, int flags, lb_alloc_fn
   if (!rc) rc = dev_alloc(c, &c->d_t, sizeof(int64_t));
   if (!rc) rc = dev_alloc(c, &c->d_barrier, 4 * sizeof(unsigned));
   if (!rc) rc = dev_alloc(c, &c->d_err, sizeof(int));
-  if (!rc) rc = dev_alloc(c, &c->d_mass, 2 * sizeof(double));
+  if (!rc) rc = dev_alloc(c, &c->d_mass, MASS_BUF * sizeof(double));
   if (!rc && cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking) != cudaSuccess) rc = LB_ERR_CUDA;
   c->stream = c->own_stream;
   if (!rc) rc = c->dev32 ? upload_tables<float>(c) : upload_tables<double>(c);
   if (!rc && (c->dev32 ? prepare_step<float>(256) : prepare_step<double>(256)) != cudaSuccess) rc = LB_ERR_CUDA;
   if (!rc && (cudaMemset(c->stats, 0, n * sizeof(DiagStats)) != cudaSuccess ||
               cudaMemset(c->d_t, 0, sizeof(int64_t)) != cudaSuccess ||
-              cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess))
+              cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess ||
+              cudaMemset(c->d_mass, 0, MASS_BUF * sizeof(double)) != cudaSuccess))
     rc = LB_ERR_CUDA;
   if (!rc) {
     // default tile: 128 columns; rows per item chosen so that the grid has a few waves, down to

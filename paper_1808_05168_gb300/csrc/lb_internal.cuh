@@ -573,8 +573,11 @@ cudaError_t launch_profiles(const DiagLattice* lat, const int* row_lat, int n_ro
 cudaError_t launch_finalize(const DiagLattice* d_lat, int n_lat, const double* partials, DiagStats* stats,
                             cudaStream_t s);
 
+// The two masses into out[0], out[1]; out holds MASS_BUF doubles (the masses, a block counter that is
+// zero between calls, and the block sums).
+constexpr int MASS_BLOCKS = 8 * 152, MASS_BUF = 4 + 2 * MASS_BLOCKS;
 template <class real>
-cudaError_t launch_mass(const real* f, const BgParams& bp, double* out2, cudaStream_t s);
+cudaError_t launch_mass(const real* f, const BgParams& bp, double* out, cudaStream_t s);
 template <class real>
 cudaError_t launch_to_absolute(const real* f, const BgParams& bp, double* out, cudaStream_t s);
 template <class real>
