@@ -161,32 +161,16 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// The fourteen normals of a site.  FP32: exactly those of the forward FP32 kernel.  FP64: the
-// library Box-Muller; the forward FP64 kernel's table-driven normals agree with it to a few units
-// in the last place, far below what the gradient resolves.
+// The fourteen normals of a site, exactly those of the forward kernel of the state's precision.
 template <class real>
-__device__ __forceinline__ void normals14(uint32_t site, uint32_t step, const LatticeDev<real>& L, real n[14]);
-template <>
-__device__ __forceinline__ void normals14<double>(uint32_t site, uint32_t step, const LatticeDev<double>& L,
-                                                  double n[14]) {
-  U4 w[4];
-  philox_site(site, step, L.lattice_id, L.key0, L.key1, w);
-  box_muller<double>(w[0].x, w[0].y, n[0], n[1]);
-  box_muller<double>(w[0].z, w[0].w, n[2], n[3]);
-  box_muller<double>(w[1].x, w[1].y, n[4], n[5]);
-  box_muller<double>(w[1].z, w[1].w, n[6], n[7]);
-  box_muller<double>(w[2].x, w[2].y, n[8], n[9]);
-  box_muller<double>(w[2].z, w[2].w, n[10], n[11]);
-  box_muller<double>(w[3].x, w[3].y, n[12], n[13]);
-}
-template <>
-__device__ __forceinline__ void normals14<float>(uint32_t site, uint32_t step, const LatticeDev<float>& L, float n[14]) {
+__device__ __forceinline__ void normals14(uint32_t site, uint32_t step, const LatticeDev<real>& L,
+                                          const NormalTables* tab, real n[14]) {
   U4 w[4];
   philox_site(site, step, L.lattice_id, L.key0, L.key1, w);
   const uint32_t k[16] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w,
                           w[2].x, w[2].y, w[2].z, w[2].w, w[3].x, w[3].y, w[3].z, w[3].w};
 #pragma unroll
-  for (int p = 0; p < 7; ++p) normal_pair<float>(k[2 * p], k[2 * p + 1], n[2 * p], n[2 * p + 1], nullptr);
+  for (int p = 0; p < 7; ++p) normal_pair<real>(k[2 * p], k[2 * p + 1], n[2 * p], n[2 * p + 1], tab);
 }
 
 // The local part of the transposed step at every site of every lattice (see the file comment).
@@ -202,7 +186,7 @@ __global__ void adj_local_kernel(const real* __restrict__ f, const double* __res
                                  const LatticeDev<real>* lat, const RowConst<real>* rows,
                                  const AdjConst* __restrict__ kcs, const AdjMap map, const double* __restrict__ rho,
                                  uint32_t step, double sign, double* __restrict__ fl, double* __restrict__ sb,
-                                 double* __restrict__ partials) {
+                                 double* __restrict__ partials, const NormalTables* tab) {
   using real_s = real;
   const int li = adj_lattice(map);
   const LatticeDev<real_s> L = lat[li];
@@ -265,7 +249,7 @@ __global__ void adj_local_kernel(const real* __restrict__ f, const double* __res
     double n[14];
     if (NOISE) {
       real_s nn[14];
-      normals14<real_s>((uint32_t)i, step, L, nn);
+      normals14<real_s>((uint32_t)i, step, L, tab, nn);
 #pragma unroll
       for (int q = 0; q < 14; ++q) n[q] = (double)nn[q];
     }
@@ -541,12 +525,12 @@ cudaError_t launch_adjoint_step(const real* f_prev, const real* f_next, const do
                                 const LatticeDev<real>* lat, const RowConst<real>* rows, const AdjConst* kcs,
                                 bool options, const AdjMap& map, uint32_t step, bool noise, double sign,
                                 bool rho_ready, double* rho, double* rho_next, double* fl, double* sb,
-                                double* partials, cudaStream_t s) {
+                                double* partials, const NormalTables* tab, cudaStream_t s) {
   const int nb = map.n_blocks;
   if (!rho_ready) adj_rho_kernel<real><<<nb, kAdjBlock, 0, s>>>(f_prev, lat, rows, map, rho);
   auto local = [&](auto noise_c, auto opts_c) {
     adj_local_kernel<real, decltype(noise_c)::value, decltype(opts_c)::value>
-        <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, rows, kcs, map, rho, step, sign, fl, sb, partials);
+        <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, rows, kcs, map, rho, step, sign, fl, sb, partials, tab);
   };
   using T = std::true_type;
   using F = std::false_type;
@@ -565,10 +549,10 @@ cudaError_t launch_adjoint_gradient(const double* partials, const AdjMap& map, d
 template cudaError_t launch_adjoint_step<float>(const float*, const float*, const double*, double*,
                                                 const LatticeDev<float>*, const RowConst<float>*, const AdjConst*,
                                                 bool, const AdjMap&, uint32_t, bool, double, bool, double*, double*,
-                                                double*, double*, double*, cudaStream_t);
+                                                double*, double*, double*, const NormalTables*, cudaStream_t);
 template cudaError_t launch_adjoint_step<double>(const double*, const double*, const double*, double*,
                                                  const LatticeDev<double>*, const RowConst<double>*, const AdjConst*,
                                                  bool, const AdjMap&, uint32_t, bool, double, bool, double*, double*,
-                                                 double*, double*, double*, cudaStream_t);
+                                                 double*, double*, double*, const NormalTables*, cudaStream_t);
 
 }  // namespace lbk

@@ -72,7 +72,7 @@ cudaError_t launch_adjoint_step(const real* f_prev, const real* f_next, const do
                                 const LatticeDev<real>* lat, const RowConst<real>* rows, const AdjConst* kcs,
                                 bool options, const AdjMap& map, uint32_t step, bool noise, double sign,
                                 bool rho_ready, double* rho, double* rho_next, double* fl, double* sb,
-                                double* partials, cudaStream_t s);
+                                double* partials, const NormalTables* tab, cudaStream_t s);
 cudaError_t launch_adjoint_gradient(const double* partials, const AdjMap& map, double* grads, cudaStream_t s);
 
 }  // namespace lbk

@@ -113,6 +113,7 @@ struct lb_ctx {
   CUtensorMap* d_tmaps = nullptr;  // bulk staging: 3-d tensor maps [buffer][lattice][run of 1, 2 links]
   bool tma = false;                // d_tmaps holds maps for the current tile
   int* d_err = nullptr;
+  const NormalTables* normals = nullptr;  // FP64 noise: the device's tables (normal_tables)
   double* d_scratch = nullptr;  // 18 * max_lattice_sites doubles (populations I/O)
   double* d_mass = nullptr;     // lb_mass (MASS_BUF doubles)
   size_t bytes = 0;
@@ -605,6 +606,7 @@ StepArgs<real> step_args(lb_ctx* c, int cur, int t_offset) {
   a.pfield = (real*)c->pfield;
   a.partials = c->partials;
   a.err = c->d_err;
+  a.normals = c->normals;
   a.tmaps = c->tma ? c->d_tmaps : nullptr;
   a.n_lat = c->n_lat;
   a.src_buf = cur;
@@ -927,6 +929,7 @@ int create_impl(lb_ctx** out, int n, const lb_params* ps, int flags, lb_alloc_fn
   c->stream = c->own_stream;
   if (!rc) rc = c->dev32 ? upload_tables<float>(c) : upload_tables<double>(c);
   if (!rc && (c->dev32 ? prepare_step<float>(256) : prepare_step<double>(256)) != cudaSuccess) rc = LB_ERR_CUDA;
+  if (!rc && !c->dev32 && normal_tables(&c->normals) != cudaSuccess) rc = LB_ERR_CUDA;
   if (!rc && (cudaMemset(c->stats, 0, n * sizeof(DiagStats)) != cudaSuccess ||
               cudaMemset(c->d_t, 0, sizeof(int64_t)) != cudaSuccess ||
               cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess ||
@@ -1198,7 +1201,7 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
                                        R.fb + R.fcur * S, R.fb + (1 - R.fcur) * S, (const LatticeDev<real>*)c->d_lat,
                                        (const RowConst<real>*)c->d_rows, d_kcs, options, map, (uint32_t)k,
                                        R.noise != NOISE_OFF, R.sign, k < c0 + len - 1, rho_k, rho_n, R.fl, R.sb,
-                                       R.gpart, R.s));
+                                       R.gpart, c->normals, R.s));
           R.fcur = 1 - R.fcur;
         }
         rcur = 1 - rcur;
@@ -1989,8 +1992,11 @@ int lb_debug_box_muller(int precision, const uint32_t* host_words, int64_t n_pai
   if (cudaMemcpy(dw, host_words, (size_t)n_pairs * 2 * sizeof(uint32_t), cudaMemcpyHostToDevice) != cudaSuccess)
     rc = LB_ERR_CUDA;
   if (!rc) {
-    cudaError_t e = precision == LB_PREC_FP64 ? launch_debug_normals<double>(dw, n_pairs, dout, nullptr)
-                                              : launch_debug_normals<float>(dw, n_pairs, dout, nullptr);
+    const NormalTables* tab = nullptr;
+    cudaError_t e = precision == LB_PREC_FP64 ? normal_tables(&tab) : cudaSuccess;
+    if (e == cudaSuccess)
+      e = precision == LB_PREC_FP64 ? launch_debug_normals<double>(dw, n_pairs, dout, tab, nullptr)
+                                    : launch_debug_normals<float>(dw, n_pairs, dout, nullptr, nullptr);
     if (e == cudaSuccess) e = cudaMemcpy(host_out, dout, (size_t)n_pairs * 2 * sizeof(double), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) rc = LB_ERR_CUDA;
   }

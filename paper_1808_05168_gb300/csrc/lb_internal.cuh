@@ -12,6 +12,7 @@
 #include <stdint.h>
 
 #include "lb.h"
+#include "lb_normals64.cuh"
 
 namespace lbk {
 
@@ -162,41 +163,10 @@ __device__ __forceinline__ void philox_site(uint32_t c0, uint32_t c1, uint32_t c
   for (int i = 0; i < 4; ++i) out[i] = U4{s0[i], s1[i], s2[i], s3[i]};
 }
 
-// Uniform in (0, 1) from the low 23 bits, u = (2 (k mod 2^23) + 1) 2^-24, exact in float and
-// double: the bits form x = 1 + (k mod 2^23) 2^-23 in [1, 2) and u = x - (1 - 2^-24) exactly.
+// Uniform in (0, 1) from the low 23 bits, u = (2 (k mod 2^23) + 1) 2^-24, exact in float: the bits form x = 1 + (k mod 2^23) 2^-23 in [1, 2) and u = x - (1 - 2^-24) exactly.
 __device__ __forceinline__ float unit_interval_bits(uint32_t k) { return __uint_as_float(0x3F800000u | (k & 0x7FFFFFu)); }
-template <class real>
-__device__ __forceinline__ real uniform01(uint32_t k);
-template <>
-__device__ __forceinline__ float uniform01<float>(uint32_t k) {
+__device__ __forceinline__ float uniform01(uint32_t k) {
   return unit_interval_bits(k) - 0.999999940395355224609375f;
-}
-template <>
-__device__ __forceinline__ double uniform01<double>(uint32_t k) {
-  return __longlong_as_double((long long)(0x3FF0000000000000ull | ((unsigned long long)(k & 0x7FFFFFu) << 29))) -
-         0.999999940395355224609375;
-}
-
-// Box-Muller: (r cos 2 pi u2, r sin 2 pi u2) with r = sqrt(-2 ln u1).
-template <class real>
-__device__ __forceinline__ void box_muller(uint32_t a, uint32_t b, real& n0, real& n1);
-template <>
-__device__ __forceinline__ void box_muller<float>(uint32_t a, uint32_t b, float& n0, float& n1) {
-  const float u1 = uniform01<float>(a), u2 = uniform01<float>(b);
-  const float r = sqrtf(-2.0f * logf(u1));
-  float s, c;
-  sincospif(2.0f * u2, &s, &c);
-  n0 = r * c;
-  n1 = r * s;
-}
-template <>
-__device__ __forceinline__ void box_muller<double>(uint32_t a, uint32_t b, double& n0, double& n1) {
-  const double u1 = uniform01<double>(a), u2 = uniform01<double>(b);
-  const double r = sqrt(-2.0 * log(u1));
-  double s, c;
-  sincospi(2.0 * u2, &s, &c);
-  n0 = r * c;
-  n1 = r * s;
 }
 
 // ---- normals of the step kernels ----------------------------------------------------------
@@ -234,42 +204,6 @@ __device__ __forceinline__ double site_reciprocal(double x) {
   return fma(y, fma(-x, y, 1.0), y);
 }
 
-// Tables of the double-precision Box-Muller (the table-driven method of P. T. P. Tang for the
-// logarithm and for sine/cosine): cs[j] = (cos, sin)(2 pi j / 1024), ln[j] = (-2 ln y_j, 1 / y_j)
-// with y_j = 3/4 + j/256, j = 0 .. 192, and the exponent's share ex[k] = (-2 n ln2_hi,
-// -2 n ln2_lo) for n = k - 24, k = 0 .. 24 (ln 2 = ln2_hi + ln2_lo, ln2_hi rounded to 24 bits, so
-// the first product is exact).  The single-precision path needs none.
-template <class real>
-struct BmTables {};
-template <>
-struct BmTables<double> {
-  double2 cs[1024];
-  double2 ln[193];
-  double2 ex[25];
-};
-constexpr double kLn2Hi = 0.693147182464599609375, kLn2Lo = -1.904654299957768e-09;
-
-// All threads of the block fill the tables (from the correctly rounded library functions); the
-// caller synchronises the block before use.
-template <class real>
-__device__ __forceinline__ void fill_bm_tables(BmTables<real>* T) {
-  if constexpr (sizeof(real) == 8) {
-    for (int j = threadIdx.x; j < 1024; j += blockDim.x) {
-      double sn, cs;
-      sincospi((double)j / 512.0, &sn, &cs);
-      T->cs[j] = make_double2(cs, sn);
-    }
-    for (int j = threadIdx.x; j < 193; j += blockDim.x) {
-      const double y = 0.75 + (double)j / 256.0;
-      T->ln[j] = make_double2(-2.0 * log(y), 1.0 / y);  // -2 ln y_j (an exact scaling), 1 / y_j
-    }
-    for (int k = threadIdx.x; k < 25; k += blockDim.x) {
-      const double n = (double)(k - 24);
-      T->ex[k] = make_double2(n * (-2.0 * kLn2Hi), n * (-2.0 * kLn2Lo));
-    }
-  }
-}
-
 // Box-Muller pair of the working precision, (r cos 2 pi u2, r sin 2 pi u2) with r = sqrt(-2 ln u1).
 // FP32: t = -2 ln u1 from the hardware base-2 logarithm, whose absolute error (~2^-22) the square
 // root would magnify where t is small; there (v = 1 - u1 < 2^-6, v exact) the series
@@ -277,20 +211,12 @@ __device__ __forceinline__ void fill_bm_tables(BmTables<real>* T) {
 // is t / sqrt(t) through the reciprocal square root, and the angle is reduced to (-pi, pi) for
 // the fast sine/cosine: cos 2 pi u2 = -cos phi and sin 2 pi u2 = -sin phi with
 // phi = 2 pi u2 - pi.  Absolute error below 3e-6 on a normal.
-// FP64, table-driven: u = m 2^-24 with m = 2 (k mod 2^23) + 1.  ln u1 = (e - 24) ln 2 + ln y with
-// m = 2^e y, y in [3/4, 3/2); ln y = ln y_j + ln(1 + t), y_j the table point nearest y and
-// t = y (1 / y_j) - 1 (one fused multiply-add; exact where y_j = 1, i.e. wherever u1 is near 1
-// and -2 ln u1 small), |t| <= 2^-9 / (3/4), from its series to t^6; (e - 24) times the two parts
-// of -2 ln 2 comes from a table.  The angle 2 pi m 2^-24 is
-// the table angle 2 pi (m >> 14) / 1024 plus d = 2 pi (m mod 2^14) 2^-24 < 6.2e-3, whose sine and
-// cosine come from their series (to d^5 and d^6) and the addition theorems.  Within a few units
-// in the last place of the library functions.
+// FP64: in integer arithmetic from the tables `tab` (normal_pair_fixed); FP32 takes none.
 template <class real>
-__device__ __forceinline__ void normal_pair(uint32_t a, uint32_t b, real& n0, real& n1, const BmTables<real>* T);
+__device__ __forceinline__ void normal_pair(uint32_t a, uint32_t b, real& n0, real& n1, const NormalTables* tab);
 template <>
-__device__ __forceinline__ void normal_pair<float>(uint32_t a, uint32_t b, float& n0, float& n1,
-                                                   const BmTables<float>*) {
-  const float u1 = uniform01<float>(a);
+__device__ __forceinline__ void normal_pair<float>(uint32_t a, uint32_t b, float& n0, float& n1, const NormalTables*) {
+  const float u1 = uniform01(a);
   const float v = 1.0f - u1;
   const float t_log = -1.38629436111989061f * lg2_ftz(u1);
   const float t_ser = v * fmaf(v, fmaf(v, 0.666666666666666667f, 1.0f), 2.0f);
@@ -305,41 +231,8 @@ __device__ __forceinline__ void normal_pair<float>(uint32_t a, uint32_t b, float
 }
 template <>
 __device__ __forceinline__ void normal_pair<double>(uint32_t a, uint32_t b, double& n0, double& n1,
-                                                    const BmTables<double>* T) {
-  const uint32_t m1 = 2u * (a & 0x7FFFFFu) + 1u;
-  const unsigned long long bits = (unsigned long long)__double_as_longlong((double)m1);
-  int e = (int)(bits >> 52) - 1023;
-  unsigned long long mant = bits & 0xFFFFFFFFFFFFFull;
-  int j;
-  double y;
-  if (mant >= (1ull << 51)) {  // y0 = m1 / 2^e in [3/2, 2): y = y0 / 2 in [3/4, 1)
-    e += 1;
-    y = __longlong_as_double((long long)(0x3FE0000000000000ull | mant));
-    j = (int)(((mant - (1ull << 51)) + (1ull << 44)) >> 45);
-  } else {  // y in [1, 3/2)
-    y = __longlong_as_double((long long)(0x3FF0000000000000ull | mant));
-    j = 64 + (int)((mant + (1ull << 43)) >> 44);
-  }
-  const double2 L = T->ln[j];
-  const double t = fma(y, L.y, -1.0);
-  // -2 ln u1 directly: every term and coefficient scaled by -2, a power of two, so the result is
-  // bit for bit -2 times the logarithm formed term by term
-  const double p2 =
-      fma(t, fma(t, fma(t, fma(t, fma(t, 1.0 / 3.0, -0.4), 0.5), -2.0 / 3.0), 1.0), -2.0);  // -2 p(t)
-  const double2 E = T->ex[e];  // e - 24 in -24 .. 0
-  const double m2lnu = E.x + (L.x + fma(t, p2, E.y));
-  const double r = sqrt(m2lnu);
-  // angle
-  const uint32_t m2 = 2u * (b & 0x7FFFFFu) + 1u;
-  const double2 CS = T->cs[m2 >> 14];
-  const double d = (double)(m2 & 0x3FFFu) * (6.283185307179586476925286766559 * 5.9604644775390625e-08);
-  const double d2 = d * d;
-  const double sd = fma(d * d2, fma(d2, 1.0 / 120.0, -1.0 / 6.0), d);
-  const double cm1 = d2 * fma(d2, fma(d2, -1.0 / 720.0, 1.0 / 24.0), -0.5);  // cos d - 1
-  const double cs = fma(-CS.y, sd, fma(CS.x, cm1, CS.x));
-  const double sn = fma(CS.x, sd, fma(CS.y, cm1, CS.y));
-  n0 = r * cs;
-  n1 = r * sn;
+                                                    const NormalTables* tab) {
+  normal_pair_fixed(a, b, n0, n1, tab);
 }
 
 // Two Box-Muller pairs at once, (a0, b0) and (a1, b1): normal_pair's arithmetic with its FP32
@@ -347,13 +240,13 @@ __device__ __forceinline__ void normal_pair<double>(uint32_t a, uint32_t b, doub
 // likewise.  FP64: two normal_pair calls.
 template <class real>
 __device__ __forceinline__ void normal_pair2(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1, real& n00,
-                                             real& n01, real& n10, real& n11, const BmTables<real>* T) {
-  normal_pair<real>(a0, b0, n00, n01, T);
-  normal_pair<real>(a1, b1, n10, n11, T);
+                                             real& n01, real& n10, real& n11, const NormalTables* tab) {
+  normal_pair<real>(a0, b0, n00, n01, tab);
+  normal_pair<real>(a1, b1, n10, n11, tab);
 }
 template <>
 __device__ __forceinline__ void normal_pair2<float>(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1, float& n00,
-                                                    float& n01, float& n10, float& n11, const BmTables<float>*) {
+                                                    float& n01, float& n10, float& n11, const NormalTables*) {
   const float2 x1 = make_float2(unit_interval_bits(a0), unit_interval_bits(a1));
   const float2 u1 = __fadd2_rn(x1, make_float2(-0.999999940395355224609375f, -0.999999940395355224609375f));
   const float2 v = __ffma2_rn(u1, make_float2(-1.0f, -1.0f), make_float2(1.0f, 1.0f));
@@ -400,6 +293,7 @@ struct StepArgs {
                        // deviation mode (sample steps only)
   double* partials;    // per item: pressure deviation sum, mass deviation A, B
   int* err;            // set to 1 by a device-side wait that gave up
+  const NormalTables* normals;  // FP64 noise (null in FP32)
   // bulk path (FP32 state): 3-d tensor maps [x][z][link] of the (A, B) pairs as 8-byte elements,
   // per state buffer and lattice, for runs of one and of two links (index (buffer n_lat +
   // lattice) 2 + run length - 1), or null; src_buf: the state buffer src points to
@@ -606,7 +500,8 @@ int prepare_power_spectrum_current_device();
 cudaError_t measure_fma_rate(bool fp64, double* flops_per_s);
 
 template <class real>
-cudaError_t launch_debug_normals(const uint32_t* words, int64_t n_pairs, double* out, cudaStream_t s);
+cudaError_t launch_debug_normals(const uint32_t* words, int64_t n_pairs, double* out, const NormalTables* tab,
+                                 cudaStream_t s);
 
 // Test hook of the bounded waits of the persistent launch: `blocks` co-resident blocks each set
 // done[b] and wait until done[list[0 .. expected)] are set.

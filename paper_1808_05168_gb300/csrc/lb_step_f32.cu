@@ -14,7 +14,7 @@ namespace lbk {
   template int persistent_grid<real>(int, int, bool);                                                              \
   template cudaError_t launch_step_persistent<real>(const StepArgs<real>&, int, int, int, bool, const PersistArgs&, \
                                                     int, cudaStream_t);                                         \
-  template cudaError_t launch_debug_normals<real>(const uint32_t*, int64_t, double*, cudaStream_t);
+  template cudaError_t launch_debug_normals<real>(const uint32_t*, int64_t, double*, const NormalTables*, cudaStream_t);
 LB_STEP_INST(float)
 
 }  // namespace lbk

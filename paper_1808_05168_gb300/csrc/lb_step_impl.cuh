@@ -380,7 +380,7 @@ __device__ __forceinline__ void site_update(const SiteK<real>& K, const RowConst
                                             const Pr<real>* ring, int bc, int bu, int bd, uint32_t site,
                                             uint32_t step, real* fl, real* pl, int LzLx, double& acc_p,
                                             double& acc_a, double& acc_b, Pr<real>* out, int ostride, int flags,
-                                            const BmTables<real>* bm) {
+                                            const NormalTables* bm) {
   using P = Pr<real>;
   const P c9 = pr(real(1) / 9), c36 = pr(real(1) / 36);
   const P d = ring[bc];
@@ -486,25 +486,18 @@ __device__ __forceinline__ void block_partials(double acc_p, double acc_a, doubl
 // Generic: reduction scratch, lattice constants, density ring (4 rows of TX + 2 pairs), stage
 // (NS rows x 9 links x (TX + 2) pairs).
 template <class real>
-struct BmBytes {
-  static constexpr size_t value = sizeof(real) == 8 ? sizeof(BmTables<double>) : 0;
-};
-
-template <class real>
 struct Smem {
   static constexpr size_t red = 0;
   static constexpr size_t lat = 8 * 3 * sizeof(double);
   static constexpr size_t ring = lat + ((sizeof(LatticeDev<real>) + 15) / 16) * 16;
   __host__ __device__ static size_t stage(int tx) { return ring + (size_t)8 * (tx + 2) * sizeof(real); }
-  __host__ __device__ static size_t bm(int tx) {
+  __host__ __device__ static size_t bytes(int tx) {
     return ((stage(tx) + (size_t)NS * 9 * (tx + 2) * sizeof(Pr<real>) + 15) / 16) * 16;
   }
-  __host__ __device__ static size_t bytes(int tx) { return bm(tx) + BmBytes<real>::value; }
 };
 
 // Bulk: as generic, then input slots (NSI slots of SlotLayout, 128-byte aligned: the dynamic
-// shared memory is declared 128-byte aligned), NSI mbarriers and an abort flag.  Both end with
-// the double-precision Box-Muller tables (FP64 kernels only).
+// shared memory is declared 128-byte aligned), NSI mbarriers and an abort flag.
 template <class real, int TX>
 struct SmemBulk {
   // halo columns on each side: the densities of the columns next to the strip pull from two
@@ -522,9 +515,8 @@ struct SmemBulk {
   // per-link and per-run copy descriptors (int4 each), filled once per launch by bulk_init
   static constexpr size_t ptab = ((tmap + 8 + 15) / 16) * 16;
   static constexpr size_t rtab = ptab + 9 * 16;
-  static constexpr size_t bm = rtab + 6 * 16;  // 16-byte entries
-  static constexpr size_t bytes = bm + BmBytes<real>::value;
-  static_assert(in % 128 == 0 && bars % 8 == 0 && tmap % 8 == 0 && ptab % 16 == 0 && bm % 16 == 0,
+  static constexpr size_t bytes = rtab + 6 * 16;
+  static_assert(in % 128 == 0 && bars % 8 == 0 && tmap % 8 == 0 && ptab % 16 == 0,
                 "shared-memory regions must stay aligned");
 };
 
@@ -536,7 +528,6 @@ __device__ __forceinline__ void process_item(const StepArgs<real>& a, const real
                                              real* __restrict__ dst, int item_index, uint32_t step,
                                              unsigned char* smem) {
   double* red = reinterpret_cast<double*>(smem + Smem<real>::red);
-  const BmTables<real>* bm = reinterpret_cast<const BmTables<real>*>(smem + Smem<real>::bm(blockDim.x));
   LatticeDev<real>* Ls = reinterpret_cast<LatticeDev<real>*>(smem + Smem<real>::lat);
   const int TX = blockDim.x, W = TX + 2;
   Pr<real>* ring = reinterpret_cast<Pr<real>*>(smem + Smem<real>::ring);
@@ -640,7 +631,7 @@ __device__ __forceinline__ void process_item(const StepArgs<real>& a, const real
         if (below && above) m.m2 = add2(m.m2, interior_m2_shift(k9, k36));
         site_update<real, SAMPLE, NOISE, decltype(unit)::value, decltype(astar)::value>(
             K, rows[z], m, ring, bc, bu, bd, site, step, a.fields + 4 * L.site_off + r0, a.pfield + L.site_off + r0,
-            LzLx, acc_p, acc_a, acc_b, g + r0, LzLx, flags, bm);
+            LzLx, acc_p, acc_a, acc_b, g + r0, LzLx, flags, a.normals);
       };
       if (flags & DF_UNIT) {
         if (flags & DF_ASTAR) site_at(BoolC<true>(), BoolC<true>());
@@ -694,7 +685,6 @@ __device__ __forceinline__ bool process_item_bulk(const StepArgs<real>& a, const
   using LAY = typename SM::LAY;
   constexpr int PAD = SM::PAD, SW = SM::SW, W = TX + 2;
   double* red = reinterpret_cast<double*>(smem + SM::red);
-  const BmTables<real>* bm = reinterpret_cast<const BmTables<real>*>(smem + SM::bm);
   LatticeDev<real>* Ls = reinterpret_cast<LatticeDev<real>*>(smem + SM::lat);
   Pr<real>* ring = reinterpret_cast<Pr<real>*>(smem + SM::ring);
   Pr<real>* instage = reinterpret_cast<Pr<real>*>(smem + SM::in);
@@ -875,7 +865,7 @@ __device__ __forceinline__ bool process_item_bulk(const StepArgs<real>& a, const
         if (IN) m.m2 = add2(m.m2, interior_m2_shift(k9, k36));
         site_update<real, SAMPLE, NOISE, decltype(unit)::value, decltype(astar)::value>(
             K, rows[z], m, ring, bc, bu, bd, site, step, a.fields + 4 * L.site_off + r0, a.pfield + L.site_off + r0,
-            LzLx, acc_p, acc_a, acc_b, g + r0, LzLx, flags, bm);
+            LzLx, acc_p, acc_a, acc_b, g + r0, LzLx, flags, a.normals);
       };
       auto rates = [&](auto inner) {
         if (flags & DF_UNIT) {
@@ -913,15 +903,6 @@ __device__ __forceinline__ bool process_item_bulk(const StepArgs<real>& a, const
 // ======================================================================================
 // Kernels.
 // ======================================================================================
-// The FP64 noise tables of the block (before its first item; none in FP32 or without noise).
-template <class real, int NOISE>
-__device__ __forceinline__ void prepare_bm(unsigned char* p) {
-  if constexpr (sizeof(real) == 8 && NOISE != NOISE_OFF) {
-    fill_bm_tables<real>(reinterpret_cast<BmTables<real>*>(p));
-    __syncthreads();
-  }
-}
-
 template <class real>
 struct MinBlocks {
   static constexpr int value = sizeof(real) == 4 ? 2 : 1;
@@ -931,7 +912,6 @@ template <class real, bool SAMPLE, int NOISE>
 __global__ void __launch_bounds__(256, MinBlocks<real>::value) step_kernel(StepArgs<real> a) {
   extern __shared__ __align__(128) unsigned char smem[];
   const uint32_t step = (uint32_t)(*a.d_t + a.t_offset);
-  prepare_bm<real, NOISE>(smem + Smem<real>::bm(blockDim.x));
   process_item<real, SAMPLE, NOISE>(a, a.src, a.dst, blockIdx.x, step, smem);
 }
 
@@ -952,7 +932,6 @@ __global__ void __launch_bounds__(TX, BulkBlocks<real>::value * 128 / TX) step_k
   extern __shared__ __align__(128) unsigned char smem[];
   const uint32_t step = (uint32_t)(*a.d_t + a.t_offset);
   bulk_init<real, TX>(smem);
-  prepare_bm<real, NOISE>(smem + SmemBulk<real, TX>::bm);
   uint32_t ph = 0;
   process_item_bulk<real, TX, SAMPLE, NOISE>(a, a.src, a.dst, blockIdx.x, step, smem, ph, a.src_buf);
 }
@@ -1034,7 +1013,6 @@ __global__ void __launch_bounds__(256, MinBlocks<real>::value)
     persistent_kernel(StepArgs<real> a, int nsteps, PersistArgs p) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int64_t t0 = *a.d_t + a.t_offset;
-  prepare_bm<real, NOISE>(smem + Smem<real>::bm(blockDim.x));
   const unsigned long long n = (unsigned)a.n_items, total = (unsigned long long)nsteps * n;
   for (unsigned long long t; (t = next_ticket(p.counter)) < total;) {
     const int k = (int)(t / n), i = (int)(t - (unsigned long long)k * n);
@@ -1055,7 +1033,6 @@ __global__ void __launch_bounds__(TX, PersistentBlocks<real>::value * 128 / TX)
   extern __shared__ __align__(128) unsigned char smem[];
   const int64_t t0 = *a.d_t + a.t_offset;
   bulk_init<real, TX>(smem);
-  prepare_bm<real, NOISE>(smem + SmemBulk<real, TX>::bm);
   uint32_t ph = 0;
   const unsigned long long n = (unsigned)a.n_items, total = (unsigned long long)nsteps * n;
   for (unsigned long long t; (t = next_ticket(p.counter)) < total;) {
@@ -1219,35 +1196,28 @@ cudaError_t launch_step_persistent(const StepArgs<real>& a, int tile_x, int nste
 // The normals of the step kernels for given Philox word pairs (test hook): thread j forms pairs
 // 2j and 2j + 1 together as the step kernels do, a trailing odd pair alone.
 template <class real>
-__global__ void debug_normals_kernel(const uint32_t* __restrict__ words, int64_t n_pairs, double* __restrict__ out) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  prepare_bm<real, NOISE_HOM>(smem);
-  const BmTables<real>* bm = reinterpret_cast<const BmTables<real>*>(smem);
+__global__ void debug_normals_kernel(const uint32_t* __restrict__ words, int64_t n_pairs, double* __restrict__ out,
+                                     const NormalTables* __restrict__ tab) {
   const int64_t i = 2 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   if (i + 1 < n_pairs) {
     real n[4];
     normal_pair2<real>(words[2 * i], words[2 * i + 1], words[2 * i + 2], words[2 * i + 3], n[0], n[1], n[2], n[3],
-                       bm);
+                       tab);
     for (int k = 0; k < 4; ++k) out[2 * i + k] = (double)n[k];
   } else if (i < n_pairs) {
     real n0, n1;
-    normal_pair<real>(words[2 * i], words[2 * i + 1], n0, n1, bm);
+    normal_pair<real>(words[2 * i], words[2 * i + 1], n0, n1, tab);
     out[2 * i] = (double)n0;
     out[2 * i + 1] = (double)n1;
   }
 }
 
 template <class real>
-cudaError_t launch_debug_normals(const uint32_t* words, int64_t n_pairs, double* out, cudaStream_t s) {
+cudaError_t launch_debug_normals(const uint32_t* words, int64_t n_pairs, double* out, const NormalTables* tab,
+                                 cudaStream_t s) {
   if (n_pairs <= 0) return cudaSuccess;
   const int64_t blocks = ((n_pairs + 1) / 2 + 255) / 256;
-  const size_t smem = BmBytes<real>::value;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(debug_normals_kernel<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  debug_normals_kernel<real><<<(unsigned)blocks, 256, smem, s>>>(words, n_pairs, out);
+  debug_normals_kernel<real><<<(unsigned)blocks, 256, 0, s>>>(words, n_pairs, out, tab);
   return cudaGetLastError();
 }
 
