@@ -1035,114 +1035,158 @@ int prepare_power_spectrum_current_device() {
 namespace {
 
 // ---- adjoint sweep for the gradient of the mean-pressure shift -----------------------------
+// The noiseless companion of a batch: the same lattices with kT = 0 and two columns.  From the rest
+// state without noise every column of a lattice stays the same, bit for bit (each site's arithmetic
+// does not depend on its x), so the spatial means of the loss and of the gradient are those of any
+// number of columns; two is the least that the bulk staging takes.  With the full width the noiseless
+// run cost as much as the noisy one (256 x 128, 500 steps: 97 -> 68 ms in FP64; eight seeds, 300 steps
+// from FP32 state: 237 -> 133 ms).
+int create_noiseless(lb_ctx** out, const lb_ctx* c) {
+  std::vector<lb_params> ps(c->params);
+  for (lb_params& p : ps) {
+    p.Lx = 2;
+    p.kT = 0.0;
+  }
+  int rc = create_impl(out, c->n_lat, ps.data(), c->flags & ~(LB_GRAPH | LB_PERSISTENT | LB_AUTOTUNE), c->alloc_fn,
+                       c->free_fn, c->alloc_user);
+  // one shape of items whatever the batch, so that a lattice's sums are those of the lattice alone
+  if (!rc && (rc = lb_set_tile(*out, 32, 2)) != LB_OK) {
+    lb_destroy(*out);
+    *out = nullptr;
+  }
+  return rc;
+}
+
 // Every lattice of the context at once: losses[i] and grads[3 i ..] per lattice (either may be
 // null; grads null: the loss alone).
 template <class real>
 int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* losses) {
   NvtxRange r("lb_pressure_shift_gradient");
   const int n = c->n_lat;
-  const size_t S = c->n_f;         // reals per state: every lattice at its f_off
-  const size_t NS = c->n_sites;    // sites of the batch: every lattice at its site_off
   const int64_t nck = (T + C - 1) / C;
   const bool want_grad = grads != nullptr;
-  cudaStream_t st = c->stream;
-  // the adjoint's blocks, lattice by lattice, and the lattices' constants of the transposed step
-  std::vector<int> first(n + 1, 0), lat_of;
-  std::vector<AdjConst> kcs(n);
-  bool options = false;
-  for (int i = 0; i < n; ++i) {
-    const int nb = adjoint_blocks(c->params[i].Lx * c->params[i].Lz);
-    first[i + 1] = first[i] + nb;
-    lat_of.insert(lat_of.end(), nb, i);
-    kcs[i] = adjoint_constants(
-        make_lattice<real>(c->params[i], c->flags, c->dev32, c->f_off[i], c->site_off[i], c->row_off[i]));
-    kcs[i].w_loss = 1.0 / ((double)T * (double)(c->params[i].Lx * c->params[i].Lz));
-    options = options || kcs[i].options;
-  }
-  const int nblk = first[n];
-  std::vector<void*> owned;
-  auto alloc = [&](size_t bytes) -> void* {
-    void* q = ctx_malloc(c, bytes);
-    if (q) owned.push_back(q);
-    return q;
-  };
-  // the noisy run (index 0) and the noiseless run (1) are independent until their losses and
-  // gradients are combined: each has its own buffers and its own stream, so that their small
-  // kernels overlap on the GPU
+  // the noisy run (index 0, on the context's lattices) and the noiseless run (1, on its narrow
+  // companion) are independent until their losses and gradients are combined: each has its own
+  // buffers and its own stream, so that their small kernels overlap on the GPU
   struct Run {
+    lb_ctx* x = nullptr;  // whose lattices, tables and items
     cudaStream_t s = nullptr;
+    size_t S = 0, NS = 0;  // reals per state; sites of the batch
     real *ck = nullptr, *ring = nullptr, *cur = nullptr, *fields = nullptr, *pfield = nullptr;
     double *fb = nullptr, *rho = nullptr, *fl = nullptr, *sb = nullptr, *partials = nullptr, *gpart = nullptr;
     DiagStats* stats = nullptr;
+    AdjConst* kcs = nullptr;
+    int* map_buf = nullptr;
+    AdjMap map{nullptr, nullptr, 0, 0};
+    std::vector<int> first, lat_of;  // the adjoint's blocks, lattice by lattice
+    std::vector<AdjConst> hkcs;      // the lattices' constants of the transposed step
+    bool options = false;
     int noise = NOISE_OFF;
     double sign = 1.0;
     int fcur = 0;
   } runs[2];
-  cudaStream_t s1 = nullptr;
+  char* arena = nullptr;
+  double* d_grad = nullptr;  // 3 n per run
+  int64_t* zero_t = nullptr;
+  cudaStream_t st = c->stream, s1 = nullptr;
   cudaEvent_t ev[2] = {nullptr, nullptr};
   auto release = [&]() {
     cudaStreamSynchronize(st);
     if (s1) cudaStreamSynchronize(s1);
-    for (void* q : owned) dev_free(c, q);
+    dev_free(c, arena);
     if (s1) cudaStreamDestroy(s1);
     for (cudaEvent_t x : ev)
       if (x) cudaEventDestroy(x);
+    if (runs[1].x) lb_destroy(runs[1].x);
   };
-  bool got = cudaStreamCreateWithFlags(&s1, cudaStreamNonBlocking) == cudaSuccess &&
-             cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming) == cudaSuccess &&
-             cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming) == cudaSuccess;
-  if (!got) {
+  if (cudaStreamCreateWithFlags(&s1, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming) != cudaSuccess) {
     release();
     return LB_ERR_CUDA;
   }
+  runs[0].x = c;
+  const int rc = create_noiseless(&runs[1].x, c);
+  if (rc) {
+    release();
+    return rc;
+  }
+  // one allocation for the call, cut into 256-byte aligned pieces (the first pass only adds them up)
+  size_t bytes = 0;
+  auto piece = [&](size_t count, size_t size) -> char* {
+    char* q = arena ? arena + bytes : nullptr;
+    bytes += (std::max<size_t>(count * size, 16) + 255) & ~(size_t)255;
+    return q;
+  };
   for (int q = 0; q < 2; ++q) {
     Run& R = runs[q];
     R.s = q == 0 ? st : s1;
     R.noise = q == 0 ? c->noise_mode : NOISE_OFF;
     R.sign = q == 0 ? 1.0 : -1.0;
-    R.ck = (real*)alloc(nck * S * sizeof(real));
-    R.cur = (real*)alloc(2 * S * sizeof(real));
-    R.fields = (real*)alloc(4 * NS * sizeof(real));
-    R.pfield = (real*)alloc(NS * sizeof(real));
-    R.partials = (double*)alloc((size_t)3 * c->items.size() * sizeof(double));
-    R.stats = (DiagStats*)alloc((size_t)n * sizeof(DiagStats));
-    got = got && R.ck && R.cur && R.fields && R.pfield && R.partials && R.stats;
-    if (want_grad) {
-      R.ring = (real*)alloc(C * S * sizeof(real));
-      R.fb = (double*)alloc(2 * S * sizeof(double));
-      R.rho = (double*)alloc(4 * NS * sizeof(double));  // two density sets
-      R.fl = (double*)alloc(S * sizeof(double));
-      R.sb = (double*)alloc(4 * NS * sizeof(double));
-      R.gpart = (double*)alloc((size_t)3 * nblk * sizeof(double));
-      got = got && R.ring && R.fb && R.rho && R.fl && R.sb && R.gpart;
+    R.S = R.x->n_f;
+    R.NS = R.x->n_sites;
+    R.first.assign(n + 1, 0);
+    R.hkcs.resize(n);
+    for (int i = 0; i < n; ++i) {
+      const lb_params& p = R.x->params[i];
+      const int nb = adjoint_blocks(p.Lx * p.Lz);
+      R.first[i + 1] = R.first[i] + nb;
+      R.lat_of.insert(R.lat_of.end(), nb, i);
+      R.hkcs[i] = adjoint_constants(
+          make_lattice<real>(p, c->flags, c->dev32, R.x->f_off[i], R.x->site_off[i], R.x->row_off[i]));
+      R.hkcs[i].w_loss = 1.0 / ((double)T * (double)(p.Lx * p.Lz));
+      R.options = R.options || R.hkcs[i].options;
     }
   }
-  double* d_grad = (double*)alloc((size_t)6 * n * sizeof(double));  // per run
-  int64_t* zero_t = (int64_t*)alloc(sizeof(int64_t));
-  int* d_map = want_grad ? (int*)alloc((size_t)(nblk + n + 1) * sizeof(int)) : nullptr;
-  AdjConst* d_kcs = want_grad ? (AdjConst*)alloc((size_t)n * sizeof(AdjConst)) : nullptr;
-  if (!got || !d_grad || !zero_t || (want_grad && (!d_map || !d_kcs))) {
-    release();
-    return LB_ERR_OOM;
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass == 1) {
+      arena = (char*)ctx_malloc(c, bytes);
+      if (!arena) {
+        release();
+        return LB_ERR_OOM;
+      }
+      bytes = 0;
+    }
+    for (Run& R : runs) {
+      const int nblk = R.first[n];
+      R.ck = (real*)piece(nck * R.S, sizeof(real));
+      R.cur = (real*)piece(2 * R.S, sizeof(real));
+      R.fields = (real*)piece(4 * R.NS, sizeof(real));
+      R.pfield = (real*)piece(R.NS, sizeof(real));
+      R.partials = (double*)piece(3 * R.x->items.size(), sizeof(double));
+      R.stats = (DiagStats*)piece(n, sizeof(DiagStats));
+      if (want_grad) {
+        R.ring = (real*)piece(C * R.S, sizeof(real));
+        R.fb = (double*)piece(2 * R.S, sizeof(double));
+        R.rho = (double*)piece(4 * R.NS, sizeof(double));  // two density sets
+        R.fl = (double*)piece(R.S, sizeof(double));
+        R.sb = (double*)piece(4 * R.NS, sizeof(double));
+        R.gpart = (double*)piece((size_t)3 * nblk, sizeof(double));
+        R.map_buf = (int*)piece((size_t)nblk + n + 1, sizeof(int));
+        R.kcs = (AdjConst*)piece(n, sizeof(AdjConst));
+      }
+    }
+    d_grad = (double*)piece((size_t)6 * n, sizeof(double));
+    zero_t = (int64_t*)piece(1, sizeof(int64_t));
   }
   cudaError_t e = cudaSuccess;
   auto ok = [&](cudaError_t r) {
     if (e == cudaSuccess && r != cudaSuccess) e = r;
   };
-  AdjMap map{nullptr, nullptr, nblk, n};
-  if (want_grad) {
-    ok(cudaMemcpy(d_map, lat_of.data(), (size_t)nblk * sizeof(int), cudaMemcpyHostToDevice));
-    ok(cudaMemcpy(d_map + nblk, first.data(), (size_t)(n + 1) * sizeof(int), cudaMemcpyHostToDevice));
-    ok(cudaMemcpy(d_kcs, kcs.data(), (size_t)n * sizeof(AdjConst), cudaMemcpyHostToDevice));
-    map.lat_of = d_map;
-    map.first = d_map + nblk;
-  }
+  if (want_grad)
+    for (Run& R : runs) {
+      const int nblk = R.first[n];
+      ok(cudaMemcpy(R.map_buf, R.lat_of.data(), (size_t)nblk * sizeof(int), cudaMemcpyHostToDevice));
+      ok(cudaMemcpy(R.map_buf + nblk, R.first.data(), (size_t)(n + 1) * sizeof(int), cudaMemcpyHostToDevice));
+      ok(cudaMemcpy(R.kcs, R.hkcs.data(), (size_t)n * sizeof(AdjConst), cudaMemcpyHostToDevice));
+      R.map = AdjMap{R.map_buf, R.map_buf + nblk, nblk, n};
+    }
   ok(cudaMemsetAsync(zero_t, 0, sizeof(int64_t), st));
   ok(cudaMemsetAsync(d_grad, 0, (size_t)6 * n * sizeof(double), st));
   ok(cudaEventRecord(ev[0], st));  // the second run's stream starts after the set-up
   ok(cudaStreamWaitEvent(s1, ev[0], 0));
   auto args = [&](const Run& R, const real* src, real* dst, int64_t k) {
-    StepArgs<real> a = step_args<real>(c, 0, 0);
+    StepArgs<real> a = step_args<real>(R.x, 0, 0);
     a.src = src;
     a.dst = dst;
     a.tmaps = nullptr;  // the context's tensor maps describe its own state buffers, not these
@@ -1151,6 +1195,7 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
     a.fields = R.fields;
     a.pfield = R.pfield;
     a.partials = R.partials;
+    a.err = c->d_err;
     return a;
   };
   // forward runs from rest, step by step in both streams: checkpoints f*_{c-1} before every C-th
@@ -1158,22 +1203,22 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
   {
     NvtxRange rr("lb adjoint: forward runs");
     for (Run& R : runs) {
-      if (want_grad) ok(cudaMemsetAsync(R.gpart, 0, (size_t)3 * nblk * sizeof(double), R.s));
+      if (want_grad) ok(cudaMemsetAsync(R.gpart, 0, (size_t)3 * R.map.n_blocks * sizeof(double), R.s));
       for (int i = 0; i < n; ++i) {
-        const lb_params& p = c->params[i];
+        const lb_params& p = R.x->params[i];
         const BgParams bp{p.Lx, p.Lz, c->dev32 ? 1 : 0, kRhoBar, p.grad_c0};
-        ok(launch_init_rest<real>(R.cur + c->f_off[i], bp, R.s));
+        ok(launch_init_rest<real>(R.cur + R.x->f_off[i], bp, R.s));
       }
       ok(cudaMemsetAsync(R.stats, 0, (size_t)n * sizeof(DiagStats), R.s));
     }
     for (int64_t k = 0; k < T && e == cudaSuccess; ++k)
       for (Run& R : runs) {
-        real* src = R.cur + (k & 1) * S;
-        real* dst = R.cur + ((k + 1) & 1) * S;
+        real* src = R.cur + (k & 1) * R.S;
+        real* dst = R.cur + ((k + 1) & 1) * R.S;
         if (k % C == 0)
-          ok(cudaMemcpyAsync(R.ck + (k / C) * S, src, S * sizeof(real), cudaMemcpyDeviceToDevice, R.s));
-        ok(launch_step<real>(args(R, src, dst, k), c->tile_x, true, R.noise, c->bulk_ok, R.s));
-        ok(launch_finalize(c->d_diag, n, R.partials, R.stats, R.s));
+          ok(cudaMemcpyAsync(R.ck + (k / C) * R.S, src, R.S * sizeof(real), cudaMemcpyDeviceToDevice, R.s));
+        ok(launch_step<real>(args(R, src, dst, k), R.x->tile_x, true, R.noise, R.x->bulk_ok, R.s));
+        ok(launch_finalize(R.x->d_diag, n, R.partials, R.stats, R.s));
       }
   }
   // reverse sweeps, one checkpoint segment at a time in both streams; a run's sign (+ noisy,
@@ -1181,34 +1226,34 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
   // whole sweep is linear
   if (want_grad && e == cudaSuccess) {
     NvtxRange rr("lb adjoint: reverse sweeps");
-    for (Run& R : runs) ok(cudaMemsetAsync(R.fb, 0, S * sizeof(double), R.s));
+    for (Run& R : runs) ok(cudaMemsetAsync(R.fb, 0, R.S * sizeof(double), R.s));
     for (int64_t seg = nck - 1; seg >= 0 && e == cudaSuccess; --seg) {
       const int64_t c0 = seg * C, len = std::min<int64_t>(C, T - c0);
-      for (Run& R : runs) {
-        ok(cudaMemcpyAsync(R.ring, R.ck + seg * S, S * sizeof(real), cudaMemcpyDeviceToDevice, R.s));
-        for (int64_t i = 1; i < len; ++i)
-          ok(launch_step<real>(args(R, R.ring + (i - 1) * S, R.ring + i * S, c0 + i - 1), c->tile_x, false, R.noise,
-                               c->bulk_ok, R.s));
-      }
+      for (Run& R : runs)
+        ok(cudaMemcpyAsync(R.ring, R.ck + seg * R.S, R.S * sizeof(real), cudaMemcpyDeviceToDevice, R.s));
+      for (int64_t i = 1; i < len; ++i)
+        for (Run& R : runs)
+          ok(launch_step<real>(args(R, R.ring + (i - 1) * R.S, R.ring + i * R.S, c0 + i - 1), R.x->tile_x, false,
+                               R.noise, R.x->bulk_ok, R.s));
       // the densities of each step's state come with the previous step's gather (within a
       // segment; at its top they are computed on their own)
       int rcur = 0;
       for (int64_t k = c0 + len - 1; k >= c0 && e == cudaSuccess; --k) {
         for (Run& R : runs) {
-          double* rho_k = R.rho + (size_t)rcur * 2 * NS;
-          double* rho_n = R.rho + (size_t)(1 - rcur) * 2 * NS;
-          ok(launch_adjoint_step<real>(R.ring + (k - c0) * S, k > c0 ? R.ring + (k - 1 - c0) * S : nullptr,
-                                       R.fb + R.fcur * S, R.fb + (1 - R.fcur) * S, (const LatticeDev<real>*)c->d_lat,
-                                       (const RowConst<real>*)c->d_rows, d_kcs, options, map, (uint32_t)k,
-                                       R.noise != NOISE_OFF, R.sign, k < c0 + len - 1, rho_k, rho_n, R.fl, R.sb,
-                                       R.gpart, c->normals, R.s));
+          double* rho_k = R.rho + (size_t)rcur * 2 * R.NS;
+          double* rho_n = R.rho + (size_t)(1 - rcur) * 2 * R.NS;
+          ok(launch_adjoint_step<real>(R.ring + (k - c0) * R.S, k > c0 ? R.ring + (k - 1 - c0) * R.S : nullptr,
+                                       R.fb + R.fcur * R.S, R.fb + (1 - R.fcur) * R.S,
+                                       (const LatticeDev<real>*)R.x->d_lat, (const RowConst<real>*)R.x->d_rows, R.kcs,
+                                       R.options, R.map, (uint32_t)k, R.noise != NOISE_OFF, R.sign, k < c0 + len - 1,
+                                       rho_k, rho_n, R.fl, R.sb, R.gpart, c->normals, R.s));
           R.fcur = 1 - R.fcur;
         }
         rcur = 1 - rcur;
       }
     }
     for (int q = 0; q < 2 && e == cudaSuccess; ++q)
-      ok(launch_adjoint_gradient(runs[q].gpart, map, d_grad + (size_t)3 * n * q, runs[q].s));
+      ok(launch_adjoint_gradient(runs[q].gpart, runs[q].map, d_grad + (size_t)3 * n * q, runs[q].s));
   }
   // join the second stream, then read the results
   ok(cudaEventRecord(ev[1], s1));
@@ -1224,9 +1269,13 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
   for (const DiagStats& x : hs)
     if (x.nonfinite) return LB_ERR_NONFINITE;
   for (int i = 0; i < n; ++i) {
-    if (losses) losses[i] = (hs[i].P_sum + hs[i].P_comp) / (double)T - (hs[n + i].P_sum + hs[n + i].P_comp) / (double)T;
+    const bool same = c->params[i].kT == 0.0;  // both runs are the same run: the shift is exactly zero
+    if (losses)
+      losses[i] = same ? 0.0
+                       : (hs[i].P_sum + hs[i].P_comp) / (double)T - (hs[n + i].P_sum + hs[n + i].P_comp) / (double)T;
     if (want_grad)
-      for (int k = 0; k < 3; ++k) grads[3 * i + k] = hg[3 * i + k] + hg[(size_t)3 * n + 3 * i + k];
+      for (int k = 0; k < 3; ++k)
+        grads[3 * i + k] = same ? 0.0 : hg[3 * i + k] + hg[(size_t)3 * n + 3 * i + k];
   }
   int err = 0;
   if (cudaMemcpy(&err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess && err) {
