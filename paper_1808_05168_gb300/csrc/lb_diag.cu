@@ -40,31 +40,8 @@ __device__ __forceinline__ void twiddle<double>(int k, int n, double& c, double&
   sincospi(-2.0 * (double)k / (double)n, &s, &c);
 }
 
-// In-place iterative radix-2 transform X_k = sum_j x_j exp(-2 pi i j k / n) of n = 2^logn
-// points held in bit-reversed order in shared memory; tw holds exp(-2 pi i k / n), k < n/2.
-template <class real>
-__device__ void fft_inplace(Cplx<real>* s, const Cplx<real>* tw, int n, int logn) {
-  for (int lg = 1; lg <= logn; ++lg) {
-    const int half = 1 << (lg - 1);
-    const int stride = n >> lg;  // twiddle index step for this stage
-    for (int j = threadIdx.x; j < (n >> 1); j += blockDim.x) {
-      const int pos = j & (half - 1);
-      const int i0 = ((j >> (lg - 1)) << lg) + pos, i1 = i0 + half;
-      const Cplx<real> w = tw[pos * stride];
-      const Cplx<real> b = s[i1], a = s[i0];
-      const real tr = w.re * b.re - w.im * b.im;
-      const real ti = w.re * b.im + w.im * b.re;
-      s[i0] = Cplx<real>{a.re + tr, a.im + ti};
-      s[i1] = Cplx<real>{a.re - tr, a.im - ti};
-    }
-    __syncthreads();
-  }
-}
-
-__device__ __forceinline__ int ilog2(int n) { return 31 - __clz(n); }
-
 // Twiddle tables of the sample-step transforms, exp(-2 pi i k / n) for k < n/2, every power of
-// two n = 2 .. 8192 at offset n/2 - 1; filled once per device by prepare_sf.
+// two n = 2 .. 8192 at offset n/2 - 1; filled by prepare_sf and prepare_power_spectrum.
 constexpr int TW_TABLE = 8192;
 __device__ Cplx<float> g_tw_f[TW_TABLE];
 __device__ Cplx<double> g_tw_d[TW_TABLE];
@@ -91,15 +68,6 @@ template <class real>
 __device__ void load_twiddles(Cplx<real>* tw, int n) {
   const Cplx<real>* t = tw_table<real>() + (n / 2 - 1);
   for (int k = threadIdx.x; k < (n >> 1); k += blockDim.x) tw[k] = t[k];
-}
-
-template <class real>
-__device__ void fill_twiddles(Cplx<real>* tw, int n) {
-  for (int k = threadIdx.x; k < (n >> 1); k += blockDim.x) {
-    real c, s;
-    twiddle<real>(k, n, c, s);
-    tw[k] = Cplx<real>{c, s};
-  }
 }
 
 __device__ __forceinline__ void neumaier_add(double& sum, double& comp, double v) {
@@ -244,23 +212,15 @@ struct SfBatch {
   static constexpr int rows = sizeof(real) == 4 ? 8 : 4, cols = sizeof(real) == 4 ? 4 : 2;
 };
 
-// Row pass: one block per (lattice, field * Lz + z0), rows z0 .. z0 + R - 1 with
-// R = sf_row_group(Lx, Lz, cap).  Rows 2c and 2c + 1 of the group enter as the real and imaginary
-// parts of sequence c, so one complex transform gives both: with Z = DFT(a + i b),
-// A_q = (Z_q + conj Z_{n-q}) / 2 and B_q = (Z_q - conj Z_{n-q}) / (2 i).  q_x = 0 .. Lx/2 of every
-// row goes to tmp; the q_x = 0 bin is the row sum, whose mean goes to the profile.
+// R real rows of n points at src (contiguous) to the q_x = 0 .. n/2 bins of their transforms at out
+// (n/2 + 1 per row).  Rows 2c and 2c + 1 enter as the real and imaginary parts of sequence c, so one
+// complex transform gives both: with Z = DFT(a + i b), A_q = (Z_q + conj Z_{n-q}) / 2 and
+// B_q = (Z_q - conj Z_{n-q}) / (2 i).  The sequences stay in s.
 template <class real>
-__global__ void __launch_bounds__(512) sf_rows_kernel(const DiagLattice* lat, const int2* tasks, const real* fields, Cplx<real>* tmp,
-                               double* prof_sum, double* prof_comp, int n_rows, int cap) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int2 task = tasks[blockIdx.x];
-  const DiagLattice L = lat[task.x];
-  const int n = L.Lx, logn = 31 - __clz(n), H = sf_half(n), SS = sf_seq_stride(n);
-  const int R = sf_row_group(n, L.Lz, cap), seqs = (R + 1) >> 1;
-  Cplx<real>* tw = reinterpret_cast<Cplx<real>*>(smem);
-  Cplx<real>* s = tw + ((n >> 1) + 1);
+__device__ __forceinline__ void transform_rows(const real* __restrict__ src, int n, int R, Cplx<real>* out,
+                                               Cplx<real>* tw, Cplx<real>* s) {
+  const int logn = 31 - __clz(n), H = sf_half(n), SS = sf_seq_stride(n), seqs = (R + 1) >> 1;
   load_twiddles<real>(tw, n);
-  const real* src = fields + 4 * L.site_off + (int64_t)task.y * n;
   const int total = seqs * n, T = blockDim.x;
   // loads in batches of SfBatch<real>::rows per thread, all issued before their shared-memory stores
   for (int base = threadIdx.x; base < total; base += SfBatch<real>::rows * T) {
@@ -285,24 +245,37 @@ __global__ void __launch_bounds__(512) sf_rows_kernel(const DiagLattice* lat, co
   }
   __syncthreads();
   stockham_fft<real>(s, tw, n, seqs);
-  Cplx<real>* out = tmp + 4 * L.site_off + (int64_t)task.y * H;
-  {
-    const int dc = T / H, dq = T - dc * H;
-    int c = threadIdx.x / H, q = threadIdx.x - c * H;
-    for (int idx = threadIdx.x; idx < seqs * H; idx += T) {
-      const int qm = (n - q) & (n - 1);
-      const Cplx<real> Z = s[c * SS + q + (q >> 4)], M = s[c * SS + qm + (qm >> 4)];
-      const real hf = real(0.5);
-      out[(int64_t)(2 * c) * H + q] = Cplx<real>{hf * (Z.re + M.re), hf * (Z.im - M.im)};
-      if (2 * c + 1 < R) out[(int64_t)(2 * c + 1) * H + q] = Cplx<real>{hf * (Z.im + M.im), hf * (M.re - Z.re)};
-      c += dc;
-      q += dq;
-      if (q >= H) {
-        q -= H;
-        ++c;
-      }
+  const int dc = T / H, dq = T - dc * H;
+  int c = threadIdx.x / H, q = threadIdx.x - c * H;
+  for (int idx = threadIdx.x; idx < seqs * H; idx += T) {
+    const int qm = (n - q) & (n - 1);
+    const Cplx<real> Z = s[c * SS + q + (q >> 4)], M = s[c * SS + qm + (qm >> 4)];
+    const real hf = real(0.5);
+    out[(int64_t)(2 * c) * H + q] = Cplx<real>{hf * (Z.re + M.re), hf * (Z.im - M.im)};
+    if (2 * c + 1 < R) out[(int64_t)(2 * c + 1) * H + q] = Cplx<real>{hf * (Z.im + M.im), hf * (M.re - Z.re)};
+    c += dc;
+    q += dq;
+    if (q >= H) {
+      q -= H;
+      ++c;
     }
   }
+}
+
+// Row pass: one block per (lattice, field * Lz + z0), rows z0 .. z0 + R - 1 with
+// R = sf_row_group(Lx, Lz, cap).  q_x = 0 .. Lx/2 of every row goes to tmp; the q_x = 0 bin is the row
+// sum, whose mean goes to the profile.
+template <class real>
+__global__ void __launch_bounds__(512) sf_rows_kernel(const DiagLattice* lat, const int2* tasks, const real* fields, Cplx<real>* tmp,
+                               double* prof_sum, double* prof_comp, int n_rows, int cap) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int2 task = tasks[blockIdx.x];
+  const DiagLattice L = lat[task.x];
+  const int n = L.Lx, SS = sf_seq_stride(n), R = sf_row_group(n, L.Lz, cap);
+  Cplx<real>* tw = reinterpret_cast<Cplx<real>*>(smem);
+  Cplx<real>* s = tw + ((n >> 1) + 1);
+  transform_rows<real>(fields + 4 * L.site_off + (int64_t)task.y * n, n, R,
+                       tmp + 4 * L.site_off + (int64_t)task.y * sf_half(n), tw, s);
   const int fld = task.y / L.Lz, z0 = task.y - fld * L.Lz;
   for (int r = threadIdx.x; r < R; r += blockDim.x) {
     const Cplx<real> Z0 = s[(r >> 1) * SS];
@@ -317,6 +290,50 @@ __device__ __forceinline__ void kahan_add(double& sum, double& comp, double v) {
   const double t = sum + y;
   comp = (t - sum) - y;
   sum = t;
+}
+
+// Walk of a block's threads over the points idx = j w + c of a strip (row j, column c) in steps of T.
+struct StripWalk {
+  int j, c, dj, dc, w;
+  __device__ __forceinline__ StripWalk(int w_, int T) : w(w_) {
+    dj = T / w;
+    dc = T - dj * w;
+    j = threadIdx.x / w;
+    c = threadIdx.x - j * w;
+  }
+  __device__ __forceinline__ void advance() {
+    j += dj;
+    c += dc;
+    if (c >= w) {
+      c -= w;
+      ++j;
+    }
+  }
+};
+
+// The DFTs along z of w adjacent columns (n points, row stride H) of `in`, left in s (sequence c:
+// column c).
+template <class real>
+__device__ __forceinline__ void transform_columns(const Cplx<real>* __restrict__ in, int H, int n, int w,
+                                                  Cplx<real>* tw, Cplx<real>* s) {
+  load_twiddles<real>(tw, n);
+  const int T = blockDim.x, total = w * n, SS = sf_seq_stride(n);
+  StripWalk k(w, T);
+  for (int b0 = threadIdx.x; b0 < total; b0 += SfBatch<real>::cols * T) {
+    Cplx<real> x[SfBatch<real>::cols];
+    int at[SfBatch<real>::cols];
+#pragma unroll
+    for (int i = 0; i < SfBatch<real>::cols; ++i) {
+      if (b0 + i * T < total) x[i] = in[(int64_t)k.j * H + k.c];
+      at[i] = k.c * SS + k.j + (k.j >> 4);
+      k.advance();
+    }
+#pragma unroll
+    for (int i = 0; i < SfBatch<real>::cols; ++i)
+      if (b0 + i * T < total) s[at[i]] = x[i];
+  }
+  __syncthreads();
+  stockham_fft<real>(s, tw, n, w);
 }
 
 // Column pass: one block per (lattice, field * Lx + q_x0), the strip of cq = sf_col_strip(Lx, Lz,
@@ -335,41 +352,11 @@ __global__ void __launch_bounds__(512) sf_cols_kernel(const DiagLattice* lat, co
   const int cq = sf_col_strip(Lx, n, cap), w = min(cq, H - qx0);
   Cplx<real>* tw = reinterpret_cast<Cplx<real>*>(smem);
   Cplx<real>* s = tw + ((n >> 1) + 1);
-  load_twiddles<real>(tw, n);
-  const Cplx<real>* in = tmp + 4 * L.site_off + (int64_t)fld * H * n + qx0;  // compact row transforms
-  const int64_t base = 4 * L.site_off + (int64_t)fld * Lx * n + qx0;     // accumulators
-  // point idx = j w + c of the strip (row j, column c); threads step idx by T, so (j, c) advance
-  // by (dj, dc) with a carry
-  const int T = blockDim.x, total = w * n, dj = T / w, dc = T - dj * w;
-  const int j0 = threadIdx.x / w, c0 = threadIdx.x - j0 * w;
-  auto advance = [&](int& j, int& c) {
-    j += dj;
-    c += dc;
-    if (c >= w) {
-      c -= w;
-      ++j;
-    }
-  };
-  {
-    int j = j0, c = c0;
-    for (int b0 = threadIdx.x; b0 < total; b0 += SfBatch<real>::cols * T) {
-      Cplx<real> x[SfBatch<real>::cols];
-      int at[SfBatch<real>::cols];
-#pragma unroll
-      for (int i = 0; i < SfBatch<real>::cols; ++i) {
-        if (b0 + i * T < total) x[i] = in[(int64_t)j * H + c];
-        at[i] = c * SS + j + (j >> 4);
-        advance(j, c);
-      }
-#pragma unroll
-      for (int i = 0; i < SfBatch<real>::cols; ++i)
-        if (b0 + i * T < total) s[at[i]] = x[i];
-    }
-  }
-  __syncthreads();
-  stockham_fft<real>(s, tw, n, w);
+  transform_columns<real>(tmp + 4 * L.site_off + (int64_t)fld * H * n + qx0, H, n, w, tw, s);
+  const int64_t base = 4 * L.site_off + (int64_t)fld * Lx * n + qx0;  // accumulators
+  const int T = blockDim.x, total = w * n;
   const real scale = real(1) / ((real)Lx * (real)n);
-  int j = j0, c = c0;
+  StripWalk k(w, T);
   for (int b0 = threadIdx.x; b0 < total; b0 += SfBatch<real>::cols * T) {
     double sm[SfBatch<real>::cols], cp[SfBatch<real>::cols];
     real pw[SfBatch<real>::cols];
@@ -377,13 +364,13 @@ __global__ void __launch_bounds__(512) sf_cols_kernel(const DiagLattice* lat, co
 #pragma unroll
     for (int i = 0; i < SfBatch<real>::cols; ++i) {
       if (b0 + i * T < total) {
-        const Cplx<real> v = s[c * SS + j + (j >> 4)];
+        const Cplx<real> v = s[k.c * SS + k.j + (k.j >> 4)];
         pw[i] = (v.re * v.re + v.im * v.im) * scale;
-        o[i] = base + (int64_t)j * Lx + c;
+        o[i] = base + (int64_t)k.j * Lx + k.c;
         sm[i] = acc_sum[o[i]];
         cp[i] = acc_comp[o[i]];
       }
-      advance(j, c);
+      k.advance();
     }
 #pragma unroll
     for (int i = 0; i < SfBatch<real>::cols; ++i) {
@@ -397,54 +384,34 @@ __global__ void __launch_bounds__(512) sf_cols_kernel(const DiagLattice* lat, co
 }
 
 // ---- power spectrum of one real field (one snapshot, written out, nothing accumulated) -----
-// Row pass: block z transforms row z of phi along x into tmp.
-__global__ void ps_rows_kernel(const double* __restrict__ phi, int Lx, int Lz, Cplx<double>* __restrict__ tmp) {
+// The sample step's transforms on one double-precision field, bound by the FP64 pipe (about 40
+// instructions per point and dimension): two real rows per complex transform, so that only
+// q_x = 0 .. Lx/2 goes through tmp and the column pass, which writes S(-q) = S(q) beside S(q).
+// 2048 x 1024: 158 us (448 us with radix-2 passes over all Lx complex columns).
+__global__ void __launch_bounds__(512) ps_rows_kernel(const double* __restrict__ phi, int Lx, int R,
+                                                      Cplx<double>* __restrict__ tmp) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int z = blockIdx.x, n = Lx, logn = ilog2(n);
-  Cplx<double>* s = reinterpret_cast<Cplx<double>*>(smem);
-  Cplx<double>* tw = s + n;
-  fill_twiddles<double>(tw, n);
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    const int r = (int)(__brev((unsigned)j) >> (32 - logn));
-    s[r] = Cplx<double>{phi[(int64_t)z * Lx + j], 0.0};
-  }
-  __syncthreads();
-  fft_inplace<double>(s, tw, n, logn);
-  for (int j = threadIdx.x; j < n; j += blockDim.x) tmp[(int64_t)z * Lx + j] = s[j];
+  Cplx<double>* tw = reinterpret_cast<Cplx<double>*>(smem);
+  const int64_t z0 = (int64_t)blockIdx.x * R;
+  transform_rows<double>(phi + z0 * Lx, Lx, R, tmp + z0 * sf_half(Lx), tw, tw + ((Lx >> 1) + 1));
 }
 
-// Column pass: block b transforms columns [b cq, (b + 1) cq) along z and writes |X|^2 / (Lx Lz).
-__global__ void ps_cols_kernel(const Cplx<double>* __restrict__ tmp, int Lx, int Lz, int cq, double* __restrict__ out) {
+__global__ void __launch_bounds__(512) ps_cols_kernel(const Cplx<double>* __restrict__ tmp, int Lx, int Lz, int cq,
+                                                      double* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int n = Lz, logn = ilog2(n), half = n >> 1, lcq = ilog2(cq), q0 = blockIdx.x * cq;
+  const int n = Lz, H = sf_half(Lx), SS = sf_seq_stride(n), q0 = blockIdx.x * cq, w = min(cq, H - q0);
   Cplx<double>* tw = reinterpret_cast<Cplx<double>*>(smem);
-  Cplx<double>* s = tw + half;
-  fill_twiddles<double>(tw, n);
-  for (int idx = threadIdx.x; idx < n * cq; idx += blockDim.x) {
-    const int j = idx >> lcq, c = idx & (cq - 1);
-    const int r = (int)(__brev((unsigned)j) >> (32 - logn));
-    s[c * n + r] = tmp[(int64_t)j * Lx + q0 + c];
-  }
-  __syncthreads();
-  for (int lg = 1; lg <= logn; ++lg) {
-    const int hs = 1 << (lg - 1), stride = n >> lg;
-    for (int idx = threadIdx.x; idx < half * cq; idx += blockDim.x) {
-      const int c = idx / half, jj = idx - c * half;
-      Cplx<double>* sc = s + c * n;
-      const int pos = jj & (hs - 1);
-      const int i0 = ((jj >> (lg - 1)) << lg) + pos, i1 = i0 + hs;
-      const Cplx<double> w = tw[pos * stride], b = sc[i1], a = sc[i0];
-      const double tr = w.re * b.re - w.im * b.im, ti = w.re * b.im + w.im * b.re;
-      sc[i0] = Cplx<double>{a.re + tr, a.im + ti};
-      sc[i1] = Cplx<double>{a.re - tr, a.im - ti};
-    }
-    __syncthreads();
-  }
+  Cplx<double>* s = tw + ((n >> 1) + 1);
+  transform_columns<double>(tmp + q0, H, n, w, tw, s);
+  const int T = blockDim.x, total = w * n;
   const double scale = 1.0 / ((double)Lx * (double)n);
-  for (int idx = threadIdx.x; idx < n * cq; idx += blockDim.x) {
-    const int j = idx >> lcq, c = idx & (cq - 1);
-    const Cplx<double> v = s[c * n + j];
-    out[(int64_t)j * Lx + q0 + c] = (v.re * v.re + v.im * v.im) * scale;
+  StripWalk k(w, T);
+  for (int b = threadIdx.x; b < total; b += T, k.advance()) {
+    const Cplx<double> v = s[k.c * SS + k.j + (k.j >> 4)];
+    const double p = (v.re * v.re + v.im * v.im) * scale;
+    const int q = q0 + k.c;
+    out[(int64_t)k.j * Lx + q] = p;
+    if (q > 0 && 2 * q < Lx) out[(int64_t)((n - k.j) & (n - 1)) * Lx + Lx - q] = p;
   }
 }
 
@@ -794,30 +761,41 @@ cudaError_t launch_init_rest(real* f, const BgParams& bp, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Dynamic shared memory of the one-snapshot passes for transforms of up to 8192 points: the
-// points plus half as many twiddles, 16 bytes each (196,608 bytes, within the 227 KB a block may
-// opt in to).
-constexpr size_t kPsSmemMax = (8192 + 4096) * sizeof(Cplx<double>);
-
-// Columns per block of the one-snapshot column pass: up to 16, as many as fit in kPsSmemMax (one
-// column of 8192 points fills it).
-static int ps_column_strip(int Lx, int Lz) {
-  int cq = 16;
-  while (cq > 1 && ((size_t)Lz * cq + Lz / 2) * sizeof(Cplx<double>) > kPsSmemMax) cq >>= 1;
-  return cq < Lx ? cq : Lx;
+// One pass of the snapshot transforms over `seqs` sequences of n points: threads per block (16 points
+// each, whole sequences), sequences per block and shared memory.  Blocks shrink from 256 threads while
+// the pass has fewer than four blocks per SM of a full chip, to spread the FP64 work; a sequence longer than 4096 points takes a block of its own.
+struct PsPass {
+  int threads, seqs;
+  size_t smem;
+};
+static PsPass ps_pass(int n, int seqs) {
+  int t = sf_threads(n, 1);
+  while (t > 64 && 8 * t >= n && (int64_t)seqs * n < (int64_t)16 * t * 4 * 152) t >>= 1;
+  PsPass p;
+  p.threads = t;
+  p.seqs = std::min(seqs, 16 * t / n);
+  p.smem = ((size_t)(n / 2 + 1) + (size_t)p.seqs * sf_seq_stride(n)) * sizeof(Cplx<double>);
+  return p;
 }
+// The largest of them: one sequence of 8192 points and its twiddles (204,832 bytes of the 227 KB a
+// block may opt in to).
+constexpr size_t kPsSmemMax = (8192 / 2 + 1 + 8192 + 8192 / 16 + 1) * sizeof(Cplx<double>);
 
 cudaError_t prepare_power_spectrum() {
-  cudaError_t e = cudaFuncSetAttribute(ps_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPsSmemMax);
+  fill_tw_tables_kernel<double><<<(TW_TABLE + 255) / 256, 256>>>();
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(ps_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPsSmemMax);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(ps_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPsSmemMax);
 }
 
 cudaError_t launch_power_spectrum(const double* field, int Lx, int Lz, double* out, void* tmp, cudaStream_t s) {
-  const int cq = ps_column_strip(Lx, Lz);
-  ps_rows_kernel<<<Lz, 256, (size_t)(Lx + Lx / 2) * sizeof(Cplx<double>), s>>>(field, Lx, Lz, (Cplx<double>*)tmp);
-  ps_cols_kernel<<<Lx / cq, 256, ((size_t)Lz * cq + Lz / 2) * sizeof(Cplx<double>), s>>>(
-      (const Cplx<double>*)tmp, Lx, Lz, cq, out);
+  const int H = sf_half(Lx);
+  const PsPass r = ps_pass(Lx, Lz / 2), c = ps_pass(Lz, H);
+  // Lz/2 and r.seqs are powers of two: every block of the row pass is full
+  ps_rows_kernel<<<Lz / 2 / r.seqs, r.threads, r.smem, s>>>(field, Lx, 2 * r.seqs, (Cplx<double>*)tmp);
+  ps_cols_kernel<<<(H + c.seqs - 1) / c.seqs, c.threads, c.smem, s>>>((const Cplx<double>*)tmp, Lx, Lz, c.seqs, out);
   return cudaGetLastError();
 }
 
