@@ -666,6 +666,15 @@ cudaError_t enqueue_direct(lb_ctx* c, int cur, int64_t n, const std::vector<int6
   return launch_advance(c->d_t, n, c->stream);
 }
 
+// Whether the persistent launch gives every block an item of its own (PersistArgs::owner): as many
+// blocks as items, and every lattice cut into chunks of the same number of rows.
+int owner_mode(const lb_ctx* c, int grid) {
+  if (grid != (int)c->items.size()) return 0;
+  for (const lb_params& p : c->params)
+    if (std::min(p.Lz, c->rows_per_item) != std::min(c->params[0].Lz, c->rows_per_item)) return 0;
+  return 1;
+}
+
 // Persistent: one cooperative launch per run of plain steps; a sample step that ends a run is an
 // ordinary launch after it (with its sampling kernels), so that the persistent kernel carries the
 // plain variant only.
@@ -691,7 +700,7 @@ cudaError_t enqueue_persistent(lb_ctx* c, int cur, int64_t n, const std::vector<
       if (e == cudaSuccess) e = cudaMemsetAsync(c->d_done, 0, c->items.size() * sizeof(unsigned), c->stream);
       if (e != cudaSuccess) return e;
       const PersistArgs pa{reinterpret_cast<unsigned long long*>(c->d_barrier), c->d_done, c->d_nbr_off, c->d_nbr,
-                           c->d_err, 2000, 0};
+                           c->d_err, 2000, owner_mode(c, grid), 0};
       e = launch_step_persistent<real>(step_args<real>(c, cur, (int)k), c->tile_x, (int)plain, c->noise_mode,
                                        c->bulk_ok, pa, grid, c->stream);
       if (e != cudaSuccess) return e;
@@ -732,7 +741,7 @@ int autotune(lb_ctx* c) {
     if (it != cache.end()) return build_items(c, it->second.first, it->second.second);
   }
   const int txs[] = {32, 64, 128, 256};
-  const int rows[] = {2, 4, 8, 16, 32, 64, 128, 256, 1 << 30};
+  const int rows[] = {1, 2, 3, 4, 6, 8, 16, 32, 64, 128, 256, 1 << 30};
   float best = 1e30f;
   int bx = c->tile_x, br = c->rows_per_item;
   std::vector<std::tuple<float, int, int>> trials;  // (ms, tile_x, rows)
@@ -762,7 +771,7 @@ int autotune(lb_ctx* c) {
         cudaMemsetAsync(c->d_barrier, 0, sizeof(unsigned long long), c->stream);
         cudaMemsetAsync(c->d_done, 0, c->items.size() * sizeof(unsigned), c->stream);
         const PersistArgs pa{reinterpret_cast<unsigned long long*>(c->d_barrier), c->d_done, c->d_nbr_off, c->d_nbr,
-                             c->d_err, 2000, 1};
+                             c->d_err, 2000, owner_mode(c, grid), 1};
         launch_step_persistent<real>(step_args<real>(c, c->cur, 0), tx, steps, c->noise_mode, c->bulk_ok, pa, grid,
                                      c->stream);
       };

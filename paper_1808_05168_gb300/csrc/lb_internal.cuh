@@ -352,6 +352,7 @@ struct PersistArgs {
   const int* nbr;
   int* err;
   int limit_ms;
+  int owner;  // a block per item and items of one length: block b runs item b of every step
   int trial;  // autotuner's trial mode: every step reads src and writes dst (the state is untouched)
 };
 

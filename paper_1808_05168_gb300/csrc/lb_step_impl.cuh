@@ -520,27 +520,37 @@ struct SmemBulk {
                 "shared-memory regions must stay aligned");
 };
 
+static_assert(sizeof(WorkItem) == 16, "a work item loads as one vector");
+__device__ __forceinline__ WorkItem load_item(const WorkItem* p) {
+  const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+  return WorkItem{v.x, v.y, v.z, v.w};
+}
+
 // ======================================================================================
 // Generic path.
 // ======================================================================================
-template <class real, bool SAMPLE, int NOISE>
-__device__ __forceinline__ void process_item(const StepArgs<real>& a, const real* __restrict__ src,
+// ready(): called once the item's constants are in shared memory and before its rows are read; the
+// persistent launch waits for the neighbours there (false: give up).  Returns false if it did.  again:
+// the block has just run the same item (its constants are in place, and ready() has a barrier).
+template <class real, bool SAMPLE, int NOISE, class Ready>
+__device__ __forceinline__ bool process_item(const StepArgs<real>& a, const real* __restrict__ src,
                                              real* __restrict__ dst, int item_index, uint32_t step,
-                                             unsigned char* smem) {
+                                             unsigned char* smem, bool again, Ready ready) {
   double* red = reinterpret_cast<double*>(smem + Smem<real>::red);
   LatticeDev<real>* Ls = reinterpret_cast<LatticeDev<real>*>(smem + Smem<real>::lat);
   const int TX = blockDim.x, W = TX + 2;
   Pr<real>* ring = reinterpret_cast<Pr<real>*>(smem + Smem<real>::ring);
   Pr<real>* stage = reinterpret_cast<Pr<real>*>(smem + Smem<real>::stage(TX));
 
-  const WorkItem it = a.items[item_index];
-  __syncthreads();  // shared memory may still be read for the previous item
-  {
+  const WorkItem it = load_item(a.items + item_index);
+  if (!again) {
+    __syncthreads();  // shared memory may still be read for the previous item
     const uint32_t* s32 = reinterpret_cast<const uint32_t*>(a.lat + it.lattice);
     uint32_t* d32 = reinterpret_cast<uint32_t*>(Ls);
     for (int i = threadIdx.x; i < (int)(sizeof(LatticeDev<real>) / 4); i += TX) d32[i] = s32[i];
+    __syncthreads();
   }
-  __syncthreads();
+  if (!ready()) return false;
   const LatticeDev<real>& L = *Ls;
   const int Lx = L.Lx, Lz = L.Lz, LzLx = Lx * Lz;
   const int tid = threadIdx.x;
@@ -645,6 +655,7 @@ __device__ __forceinline__ void process_item(const StepArgs<real>& a, const real
   }
   cp_wait<0>();  // nothing may land in shared memory after the item
   if (SAMPLE) block_partials(acc_p, acc_a, acc_b, red, a.partials + 3 * item_index);
+  return true;
 }
 
 // ======================================================================================
@@ -676,11 +687,11 @@ __device__ __forceinline__ void bulk_init(unsigned char* smem) {
 }
 
 // ph: expected parity bit per input slot, carried across items by the caller.  Returns false if
-// a wait gave up (the block then stops; a.err is set).
-template <class real, int TX, bool SAMPLE, int NOISE>
+// a wait gave up (the block then stops; a.err is set).  ready(): as process_item.
+template <class real, int TX, bool SAMPLE, int NOISE, class Ready>
 __device__ __forceinline__ bool process_item_bulk(const StepArgs<real>& a, const real* __restrict__ src,
                                                   real* __restrict__ dst, int item_index, uint32_t step,
-                                                  unsigned char* smem, uint32_t& ph, int src_buf) {
+                                                  unsigned char* smem, uint32_t& ph, int src_buf, bool again, Ready ready) {
   using SM = SmemBulk<real, TX>;
   using LAY = typename SM::LAY;
   constexpr int PAD = SM::PAD, SW = SM::SW, W = TX + 2;
@@ -695,20 +706,21 @@ __device__ __forceinline__ bool process_item_bulk(const StepArgs<real>& a, const
   const int4* ptab = reinterpret_cast<const int4*>(smem + SM::ptab);
   const int4* rtab = reinterpret_cast<const int4*>(smem + SM::rtab);
 
-  const WorkItem it = a.items[item_index];
-  __syncthreads();  // shared memory may still be read for the previous item
-  {
+  const WorkItem it = load_item(a.items + item_index);
+  if (!again) {
+    __syncthreads();  // shared memory may still be read for the previous item
     const uint32_t* s32 = reinterpret_cast<const uint32_t*>(a.lat + it.lattice);
     uint32_t* d32 = reinterpret_cast<uint32_t*>(Ls);
     for (int i = threadIdx.x; i < (int)(sizeof(LatticeDev<real>) / 4); i += TX) d32[i] = s32[i];
-    // the tensor maps of this lattice in the source buffer (kept in shared memory, not
-    // registers); null if the input slots were not 128-byte aligned after all
-    if (threadIdx.x == 0)
-      *const_cast<const CUtensorMap**>(tmap_s) = a.tmaps && (smem_u32(instage) & 127u) == 0
-                                                     ? a.tmaps + ((size_t)src_buf * a.n_lat + it.lattice) * 2
-                                                     : nullptr;
   }
-  __syncthreads();
+  // the tensor maps of this lattice in the source buffer (kept in shared memory, not registers); null
+  // if the input slots were not 128-byte aligned after all
+  if (threadIdx.x == 0)
+    *const_cast<const CUtensorMap**>(tmap_s) = a.tmaps && (smem_u32(instage) & 127u) == 0
+                                                   ? a.tmaps + ((size_t)src_buf * a.n_lat + it.lattice) * 2
+                                                   : nullptr;
+  if (!again) __syncthreads();
+  if (!ready()) return false;
   const LatticeDev<real>& L = *Ls;
   const int Lx = L.Lx, Lz = L.Lz, LzLx = Lx * Lz;
   const int tid = threadIdx.x;
@@ -912,7 +924,7 @@ template <class real, bool SAMPLE, int NOISE>
 __global__ void __launch_bounds__(256, MinBlocks<real>::value) step_kernel(StepArgs<real> a) {
   extern __shared__ __align__(128) unsigned char smem[];
   const uint32_t step = (uint32_t)(*a.d_t + a.t_offset);
-  process_item<real, SAMPLE, NOISE>(a, a.src, a.dst, blockIdx.x, step, smem);
+  process_item<real, SAMPLE, NOISE>(a, a.src, a.dst, blockIdx.x, step, smem, false, [] { return true; });
 }
 
 template <class real>
@@ -933,7 +945,8 @@ __global__ void __launch_bounds__(TX, BulkBlocks<real>::value * 128 / TX) step_k
   const uint32_t step = (uint32_t)(*a.d_t + a.t_offset);
   bulk_init<real, TX>(smem);
   uint32_t ph = 0;
-  process_item_bulk<real, TX, SAMPLE, NOISE>(a, a.src, a.dst, blockIdx.x, step, smem, ph, a.src_buf);
+  process_item_bulk<real, TX, SAMPLE, NOISE>(a, a.src, a.dst, blockIdx.x, step, smem, ph, a.src_buf,
+                                             false, [] { return true; });
 }
 
 // ---- the persistent launch: items handed out in order, per-item dependencies -------------
@@ -947,6 +960,10 @@ __global__ void __launch_bounds__(TX, BulkBlocks<real>::value * 128 / TX) step_k
 // it reads is written, and no one still reads the region it overwrites.  The relation is
 // symmetric and the tickets an item waits on were all handed out before its own, so with every
 // block resident (cooperative launch) each wait ends; it is bounded all the same.
+// With a resident block for every item and items of one length (PersistArgs::owner) block b keeps item
+// b for all steps: no ticket to draw, and the item's constants stay in shared memory.  512 x 256 in
+// FP32: 6.75 us per step (128 x 1 items), 9.6 with tickets and the constants reloaded.  Items of different lengths are left to the tickets: the ensemble of 16 seeds, whose 128
+// x 256 items would each have a block of their own, runs 0.56 ms per step with tickets and 0.66 with owners.
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -956,53 +973,59 @@ __device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Thread 0 waits until done[list[q]] >= need for all q (pausing 32 ns .. 1 us between polls);
-// false, for the whole block, if the wait gave up after limit_ms (err is then set) or another
-// block reported an error.  The data behind the flags are then read through bulk copies (the
-// async proxy), hence the proxy fence.
-static __device__ bool wait_items(const unsigned* done, const int* list, int cnt, unsigned need, int* err, int limit_ms) {
+// The first warp waits until done[list[q]] >= need for all q < cnt, a lane per entry, so that the wait
+// costs one round trip to L2 and not one per neighbour (pausing 32 to 256 ns between polls); false, for
+// the whole block, if the wait gave up after limit_ms (err is then set) or another block reported an
+// error.  The data behind the flags are then read through bulk copies (the async proxy), hence the
+// proxy fence.
+static __device__ bool wait_flags(const unsigned* done, const int* list, int cnt, unsigned need, int* err, int limit_ms) {
   __shared__ int ok_s;
-  if (threadIdx.x == 0) {
-    int ok = 1;
+  if (threadIdx.x < 32) {
+    bool ok = true;
     const uint64_t t0 = global_ns(), lim = (uint64_t)limit_ms * 1000000ull;
-    for (int q = 0; q < cnt && ok; ++q) {
+    for (int q = threadIdx.x; q < cnt && ok; q += 32) {
+      const unsigned* flag = done + list[q];
       unsigned pause = 32;
-      while (ld_acquire(done + list[q]) < need) {
+      while (ld_acquire(flag) < need) {
         if (*(volatile int*)err) {
-          ok = 0;
+          ok = false;
           break;
         }
         if (global_ns() - t0 > lim) {
           atomicExch(err, 1);
-          ok = 0;
+          ok = false;
           break;
         }
         __nanosleep(pause);
-        if (pause < 1024) pause <<= 1;
+        if (pause < 256) pause <<= 1;
       }
     }
-    ok_s = ok;
+    ok = __all_sync(0xffffffffu, ok);
+    if (threadIdx.x == 0) ok_s = ok;
   }
   __syncthreads();
   asm volatile("fence.proxy.async.global;" ::: "memory");
   return ok_s != 0;
 }
-
-// Every thread of the block has issued its stores of the item; thread 0 makes them visible and
-// then sets done[i] = value.
-__device__ __forceinline__ void publish_item(unsigned* done, int i, unsigned value) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    st_release(done + i, value);
-  }
+static __device__ bool wait_items(const PersistArgs& p, int i, unsigned need) {
+  const int o = p.nbr_off[i];
+  return wait_flags(p.done, p.nbr + o, p.nbr_off[i + 1] - o, need, p.err, p.limit_ms);
 }
 
-// The next ticket of the block (thread 0 draws it; block-uniform result).  The item's own first
-// barrier orders every read of the shared copy before thread 0 replaces it.
-__device__ __forceinline__ unsigned long long next_ticket(unsigned long long* counter) {
+// Every thread of the block has issued its stores of the item; thread 0 makes them visible and sets
+// done[i] = value (the release orders the whole block's stores, which the barrier put before it).
+__device__ __forceinline__ void publish_item(unsigned* done, int i, unsigned value) {
+  __syncthreads();
+  if (threadIdx.x == 0) st_release(done + i, value);  // cumulative over the barrier
+}
+
+// The block's next ticket (thread 0 draws it; block-uniform result), or with PersistArgs::owner the
+// same item of the next step.  The last ticket is kept in shared memory, not in registers; the item's
+// own first barrier orders every read of it before thread 0 replaces it.
+__device__ __forceinline__ unsigned long long next_ticket(const PersistArgs& p, unsigned n_items, bool first) {
   __shared__ unsigned long long t_s;
-  if (threadIdx.x == 0) t_s = atomicAdd(counter, 1ull);
+  if (threadIdx.x == 0)
+    t_s = !p.owner ? atomicAdd(p.counter, 1ull) : first ? (unsigned long long)blockIdx.x : t_s + n_items;
   __syncthreads();
   return t_s;
 }
@@ -1014,15 +1037,14 @@ __global__ void __launch_bounds__(256, MinBlocks<real>::value)
   extern __shared__ __align__(128) unsigned char smem[];
   const int64_t t0 = *a.d_t + a.t_offset;
   const unsigned long long n = (unsigned)a.n_items, total = (unsigned long long)nsteps * n;
-  for (unsigned long long t; (t = next_ticket(p.counter)) < total;) {
+  bool first = true;
+  for (unsigned long long t; (t = next_ticket(p, (unsigned)n, first)) < total; first = false) {
     const int k = (int)(t / n), i = (int)(t - (unsigned long long)k * n);
-    if (k > 0 && !wait_items(p.done, p.nbr + p.nbr_off[i], p.nbr_off[i + 1] - p.nbr_off[i], (unsigned)k, p.err,
-                             p.limit_ms))
-      return;
+    auto ready = [&] { return k == 0 || wait_items(p, i, (unsigned)k); };
     const bool odd = (k & 1) && !p.trial;
     const real* src = odd ? a.dst : a.src;
     real* dst = odd ? const_cast<real*>(a.src) : a.dst;
-    process_item<real, false, NOISE>(a, src, dst, i, (uint32_t)(t0 + k), smem);
+    if (!process_item<real, false, NOISE>(a, src, dst, i, (uint32_t)(t0 + k), smem, k > 0 && p.owner, ready)) return;
     publish_item(p.done, i, (unsigned)(k + 1));
   }
 }
@@ -1035,16 +1057,15 @@ __global__ void __launch_bounds__(TX, PersistentBlocks<real>::value * 128 / TX)
   bulk_init<real, TX>(smem);
   uint32_t ph = 0;
   const unsigned long long n = (unsigned)a.n_items, total = (unsigned long long)nsteps * n;
-  for (unsigned long long t; (t = next_ticket(p.counter)) < total;) {
+  bool first = true;
+  for (unsigned long long t; (t = next_ticket(p, (unsigned)n, first)) < total; first = false) {
     const int k = (int)(t / n), i = (int)(t - (unsigned long long)k * n);
-    if (k > 0 && !wait_items(p.done, p.nbr + p.nbr_off[i], p.nbr_off[i + 1] - p.nbr_off[i], (unsigned)k, p.err,
-                             p.limit_ms))
-      return;
+    auto ready = [&] { return k == 0 || wait_items(p, i, (unsigned)k); };
     const bool odd = (k & 1) && !p.trial;
     const real* src = odd ? a.dst : a.src;
     real* dst = odd ? const_cast<real*>(a.src) : a.dst;
     if (!process_item_bulk<real, TX, false, NOISE>(a, src, dst, i, (uint32_t)(t0 + k), smem, ph,
-                                                   a.src_buf ^ (odd ? 1 : 0)))
+                                                   a.src_buf ^ (odd ? 1 : 0), k > 0 && p.owner, ready))
       return;  // the blocks that wait on this item give up (bounded)
     publish_item(p.done, i, (unsigned)(k + 1));
   }
@@ -1228,7 +1249,7 @@ __global__ void advance_kernel(int64_t* d_t, int64_t k) { *d_t += k; }
 // Block b marks itself done and waits (bounded) until blocks list[0 .. expected) are.
 __global__ void barrier_probe_kernel(unsigned* done, const int* list, int* err, int expected, int limit_ms) {
   publish_item(done, blockIdx.x, 1u);
-  wait_items(done, list, expected, 1u, err, limit_ms);
+  wait_flags(done, list, expected, 1u, err, limit_ms);
 }
 
 cudaError_t launch_advance(int64_t* d_t, int64_t k, cudaStream_t s) {
