@@ -235,7 +235,7 @@ int lb_import_columns(lb_ctx* ctx, int lattice, int x_first, int n_cols, const v
  * alias field), in memory of the current device (or managed memory); Lx and Lz are powers of two
  * in 2..8192.  Host pointers, another device's memory or other sizes return LB_ERR_BAD_PARAM
  * before anything is launched.  Stream-ordered on `stream` (NULL: legacy default stream), which also
- * orders a device scratch of Lx * Lz * 16 bytes allocated and freed with cudaMallocAsync /
+ * orders a device scratch of (Lx/2 + 1) * Lz * 16 bytes allocated and freed with cudaMallocAsync /
  * cudaFreeAsync; returns before the result is ready. */
 int lb_power_spectrum(const double* field, int Lx, int Lz, double* out, void* stream);
 

@@ -1949,7 +1949,7 @@ int lb_power_spectrum(const double* field, int Lx, int Lz, double* out, void* st
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   void* tmp = nullptr;
-  if (cudaMallocAsync(&tmp, (size_t)Lx * Lz * 2 * sizeof(double), s) != cudaSuccess) {
+  if (cudaMallocAsync(&tmp, (size_t)sf_half(Lx) * Lz * 2 * sizeof(double), s) != cudaSuccess) {
     cudaGetLastError();
     return LB_ERR_OOM;
   }

@@ -83,7 +83,7 @@ __device__ __forceinline__ void neumaier_add(double& sum, double& comp, double v
 // r = 0 .. R-1, turns point r by exp(-2 pi i r k / (Ns R)), forms their R-point DFT in registers
 // and stores output q at (j - k) R + k + q Ns.  After the last pass the sequence holds its DFT
 // X_k = sum_j x_j exp(-2 pi i j k / n) in natural order (the autosort formulation of Stockham's
-// FFT, e.g. Govindaraju et al., SC 2008).  Each thread holds 16 points per pass; a barrier
+// FFT, e.g. Govindaraju et al., SC 2008).  Each thread holds PTS points per pass; a barrier
 // separates its loads from its stores, so one buffer serves every pass.
 
 template <class real>
@@ -145,13 +145,13 @@ __device__ __forceinline__ void dft_regs(Cplx<real>* v) {
 
 // One pass over `seqs` sequences of n points at s + seq * sf_seq_stride(n) (point p at p + p/16);
 // tw: exp(-2 pi i e / n) for e < n/2.
-template <class real, int R>
+template <class real, int R, int PTS>
 __device__ __forceinline__ void stockham_pass(Cplx<real>* s, const Cplx<real>* tw, int n, int Ns, int seqs) {
-  constexpr int BPT = 16 / R;  // butterflies per thread
+  constexpr int BPT = PTS / R;  // butterflies per thread
   const int nb = n / R, lnb = 31 - __clz(nb);
   const int total = seqs * nb, SS = sf_seq_stride(n);
   const int unit = n / (Ns * R), h = n >> 1;
-  Cplx<real> v[16];
+  Cplx<real> v[PTS];
 #pragma unroll
   for (int i = 0; i < BPT; ++i) {
     const int b = threadIdx.x + i * blockDim.x;
@@ -194,15 +194,16 @@ __device__ __forceinline__ void stockham_pass(Cplx<real>* s, const Cplx<real>* t
   __syncthreads();
 }
 
-// DFT of `seqs` sequences of n = 2^m points in place (seqs n <= 16 blockDim.x): radix-16 passes,
-// then one pass of the remaining radix.
-template <class real>
+// DFT of `seqs` sequences of n = 2^m points in place (seqs n <= PTS blockDim.x): passes of radix PTS
+// (4, 8 or 16), then one pass of the remaining radix.
+template <class real, int PTS>
 __device__ void stockham_fft(Cplx<real>* s, const Cplx<real>* tw, int n, int seqs) {
+  constexpr int bits = PTS == 16 ? 4 : PTS == 8 ? 3 : 2;
   int left = 31 - __clz(n), Ns = 1;
-  for (; left >= 4; left -= 4, Ns <<= 4) stockham_pass<real, 16>(s, tw, n, Ns, seqs);
-  if (left == 3) stockham_pass<real, 8>(s, tw, n, Ns, seqs);
-  else if (left == 2) stockham_pass<real, 4>(s, tw, n, Ns, seqs);
-  else if (left == 1) stockham_pass<real, 2>(s, tw, n, Ns, seqs);
+  for (; left >= bits; left -= bits, Ns <<= bits) stockham_pass<real, PTS, PTS>(s, tw, n, Ns, seqs);
+  if (PTS > 8 && left == 3) stockham_pass<real, PTS < 8 ? PTS : 8, PTS>(s, tw, n, Ns, seqs);
+  else if (PTS > 4 && left == 2) stockham_pass<real, 4, PTS>(s, tw, n, Ns, seqs);
+  else if (left == 1) stockham_pass<real, 2, PTS>(s, tw, n, Ns, seqs);
 }
 
 // Global loads per thread that the transforms issue before they wait for the first (row pass,
@@ -216,7 +217,7 @@ struct SfBatch {
 // (n/2 + 1 per row).  Rows 2c and 2c + 1 enter as the real and imaginary parts of sequence c, so one
 // complex transform gives both: with Z = DFT(a + i b), A_q = (Z_q + conj Z_{n-q}) / 2 and
 // B_q = (Z_q - conj Z_{n-q}) / (2 i).  The sequences stay in s.
-template <class real>
+template <class real, int PTS>
 __device__ __forceinline__ void transform_rows(const real* __restrict__ src, int n, int R, Cplx<real>* out,
                                                Cplx<real>* tw, Cplx<real>* s) {
   const int logn = 31 - __clz(n), H = sf_half(n), SS = sf_seq_stride(n), seqs = (R + 1) >> 1;
@@ -244,7 +245,7 @@ __device__ __forceinline__ void transform_rows(const real* __restrict__ src, int
     }
   }
   __syncthreads();
-  stockham_fft<real>(s, tw, n, seqs);
+  stockham_fft<real, PTS>(s, tw, n, seqs);
   const int dc = T / H, dq = T - dc * H;
   int c = threadIdx.x / H, q = threadIdx.x - c * H;
   for (int idx = threadIdx.x; idx < seqs * H; idx += T) {
@@ -274,7 +275,7 @@ __global__ void __launch_bounds__(512) sf_rows_kernel(const DiagLattice* lat, co
   const int n = L.Lx, SS = sf_seq_stride(n), R = sf_row_group(n, L.Lz, cap);
   Cplx<real>* tw = reinterpret_cast<Cplx<real>*>(smem);
   Cplx<real>* s = tw + ((n >> 1) + 1);
-  transform_rows<real>(fields + 4 * L.site_off + (int64_t)task.y * n, n, R,
+  transform_rows<real, 16>(fields + 4 * L.site_off + (int64_t)task.y * n, n, R,
                        tmp + 4 * L.site_off + (int64_t)task.y * sf_half(n), tw, s);
   const int fld = task.y / L.Lz, z0 = task.y - fld * L.Lz;
   for (int r = threadIdx.x; r < R; r += blockDim.x) {
@@ -313,7 +314,7 @@ struct StripWalk {
 
 // The DFTs along z of w adjacent columns (n points, row stride H) of `in`, left in s (sequence c:
 // column c).
-template <class real>
+template <class real, int PTS>
 __device__ __forceinline__ void transform_columns(const Cplx<real>* __restrict__ in, int H, int n, int w,
                                                   Cplx<real>* tw, Cplx<real>* s) {
   load_twiddles<real>(tw, n);
@@ -333,7 +334,7 @@ __device__ __forceinline__ void transform_columns(const Cplx<real>* __restrict__
       if (b0 + i * T < total) s[at[i]] = x[i];
   }
   __syncthreads();
-  stockham_fft<real>(s, tw, n, w);
+  stockham_fft<real, PTS>(s, tw, n, w);
 }
 
 // Column pass: one block per (lattice, field * Lx + q_x0), the strip of cq = sf_col_strip(Lx, Lz,
@@ -352,7 +353,7 @@ __global__ void __launch_bounds__(512) sf_cols_kernel(const DiagLattice* lat, co
   const int cq = sf_col_strip(Lx, n, cap), w = min(cq, H - qx0);
   Cplx<real>* tw = reinterpret_cast<Cplx<real>*>(smem);
   Cplx<real>* s = tw + ((n >> 1) + 1);
-  transform_columns<real>(tmp + 4 * L.site_off + (int64_t)fld * H * n + qx0, H, n, w, tw, s);
+  transform_columns<real, 16>(tmp + 4 * L.site_off + (int64_t)fld * H * n + qx0, H, n, w, tw, s);
   const int64_t base = 4 * L.site_off + (int64_t)fld * Lx * n + qx0;  // accumulators
   const int T = blockDim.x, total = w * n;
   const real scale = real(1) / ((real)Lx * (real)n);
@@ -387,22 +388,24 @@ __global__ void __launch_bounds__(512) sf_cols_kernel(const DiagLattice* lat, co
 // The sample step's transforms on one double-precision field, bound by the FP64 pipe (about 40
 // instructions per point and dimension): two real rows per complex transform, so that only
 // q_x = 0 .. Lx/2 goes through tmp and the column pass, which writes S(-q) = S(q) beside S(q).
-// 2048 x 1024: 158 us (448 us with radix-2 passes over all Lx complex columns).
-__global__ void __launch_bounds__(512) ps_rows_kernel(const double* __restrict__ phi, int Lx, int R,
+// 2048 x 1024: 158 us (448 us with radix-2 passes over all Lx complex columns), 64 x 64: 6.8 us (8.2).
+template <int PTS>
+__global__ void __launch_bounds__(8192 / PTS) ps_rows_kernel(const double* __restrict__ phi, int Lx, int R,
                                                       Cplx<double>* __restrict__ tmp) {
   extern __shared__ __align__(16) unsigned char smem[];
   Cplx<double>* tw = reinterpret_cast<Cplx<double>*>(smem);
   const int64_t z0 = (int64_t)blockIdx.x * R;
-  transform_rows<double>(phi + z0 * Lx, Lx, R, tmp + z0 * sf_half(Lx), tw, tw + ((Lx >> 1) + 1));
+  transform_rows<double, PTS>(phi + z0 * Lx, Lx, R, tmp + z0 * sf_half(Lx), tw, tw + ((Lx >> 1) + 1));
 }
 
-__global__ void __launch_bounds__(512) ps_cols_kernel(const Cplx<double>* __restrict__ tmp, int Lx, int Lz, int cq,
+template <int PTS>
+__global__ void __launch_bounds__(8192 / PTS) ps_cols_kernel(const Cplx<double>* __restrict__ tmp, int Lx, int Lz, int cq,
                                                       double* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int n = Lz, H = sf_half(Lx), SS = sf_seq_stride(n), q0 = blockIdx.x * cq, w = min(cq, H - q0);
   Cplx<double>* tw = reinterpret_cast<Cplx<double>*>(smem);
   Cplx<double>* s = tw + ((n >> 1) + 1);
-  transform_columns<double>(tmp + q0, H, n, w, tw, s);
+  transform_columns<double, PTS>(tmp + q0, H, n, w, tw, s);
   const int T = blockDim.x, total = w * n;
   const double scale = 1.0 / ((double)Lx * (double)n);
   StripWalk k(w, T);
@@ -761,19 +764,23 @@ cudaError_t launch_init_rest(real* f, const BgParams& bp, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// One pass of the snapshot transforms over `seqs` sequences of n points: threads per block (16 points
-// each, whole sequences), sequences per block and shared memory.  Blocks shrink from 256 threads while
-// the pass has fewer than four blocks per SM of a full chip, to spread the FP64 work; a sequence longer than 4096 points takes a block of its own.
+// One pass of the snapshot transforms over `seqs` sequences of n points.  A warp's FP64 instruction
+// holds the SM's pipe for 16 clocks however few of its lanes work, so a small pass wants many threads
+// of few points each (radix 4), a large one few passes through shared memory (radix 16).  Both passes,
+// in us with 4 / 8 / 16 points per thread: 512 x 256 24.6 / 31.9 / 51.3, 1024 x 256 35 / 35 / 53,
+// 1024 x 512 60 / 57 / 62, 2048 x 1024 220 / 211 / 207, 2048 x 4096 876 / 790 / 758; the lines lie at
+// 2^17 and 2^19 complex points of a pass.  Blocks are of 64 or 128 threads (the best at each size), a
+// sequence that needs more takes a block of its own.
 struct PsPass {
-  int threads, seqs;
+  int pts, threads, seqs;
   size_t smem;
 };
 static PsPass ps_pass(int n, int seqs) {
-  int t = sf_threads(n, 1);
-  while (t > 64 && 8 * t >= n && (int64_t)seqs * n < (int64_t)16 * t * 4 * 152) t >>= 1;
   PsPass p;
-  p.threads = t;
-  p.seqs = std::min(seqs, 16 * t / n);
+  const int64_t points = (int64_t)n * seqs;
+  p.pts = points < (1 << 17) && n <= 4096 ? 4 : points < (1 << 19) ? 8 : 16;
+  p.threads = std::max(p.pts == 8 ? 128 : 64, n / p.pts);
+  p.seqs = std::min(seqs, p.pts * p.threads / n);
   p.smem = ((size_t)(n / 2 + 1) + (size_t)p.seqs * sf_seq_stride(n)) * sizeof(Cplx<double>);
   return p;
 }
@@ -781,21 +788,40 @@ static PsPass ps_pass(int n, int seqs) {
 // block may opt in to).
 constexpr size_t kPsSmemMax = (8192 / 2 + 1 + 8192 + 8192 / 16 + 1) * sizeof(Cplx<double>);
 
+template <int PTS>
+static cudaError_t prepare_ps() {
+  cudaError_t e = cudaFuncSetAttribute(ps_rows_kernel<PTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPsSmemMax);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(ps_cols_kernel<PTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPsSmemMax);
+}
+
 cudaError_t prepare_power_spectrum() {
   fill_tw_tables_kernel<double><<<(TW_TABLE + 255) / 256, 256>>>();
   cudaError_t e = cudaDeviceSynchronize();
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(ps_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPsSmemMax);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(ps_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPsSmemMax);
+  if (e == cudaSuccess) e = prepare_ps<4>();
+  if (e == cudaSuccess) e = prepare_ps<8>();
+  if (e == cudaSuccess) e = prepare_ps<16>();
+  return e;
+}
+
+template <int PTS>
+static void launch_ps_rows(const PsPass& r, const double* field, int Lx, int Lz, void* tmp, cudaStream_t s) {
+  // Lz/2 and r.seqs are powers of two: every block is full
+  ps_rows_kernel<PTS><<<Lz / 2 / r.seqs, r.threads, r.smem, s>>>(field, Lx, 2 * r.seqs, (Cplx<double>*)tmp);
+}
+template <int PTS>
+static void launch_ps_cols(const PsPass& c, const void* tmp, int Lx, int Lz, double* out, cudaStream_t s) {
+  ps_cols_kernel<PTS><<<(sf_half(Lx) + c.seqs - 1) / c.seqs, c.threads, c.smem, s>>>((const Cplx<double>*)tmp, Lx, Lz, c.seqs, out);
 }
 
 cudaError_t launch_power_spectrum(const double* field, int Lx, int Lz, double* out, void* tmp, cudaStream_t s) {
-  const int H = sf_half(Lx);
-  const PsPass r = ps_pass(Lx, Lz / 2), c = ps_pass(Lz, H);
-  // Lz/2 and r.seqs are powers of two: every block of the row pass is full
-  ps_rows_kernel<<<Lz / 2 / r.seqs, r.threads, r.smem, s>>>(field, Lx, 2 * r.seqs, (Cplx<double>*)tmp);
-  ps_cols_kernel<<<(H + c.seqs - 1) / c.seqs, c.threads, c.smem, s>>>((const Cplx<double>*)tmp, Lx, Lz, c.seqs, out);
+  const PsPass r = ps_pass(Lx, Lz / 2), c = ps_pass(Lz, sf_half(Lx));
+  if (r.pts == 4) launch_ps_rows<4>(r, field, Lx, Lz, tmp, s);
+  else if (r.pts == 8) launch_ps_rows<8>(r, field, Lx, Lz, tmp, s);
+  else launch_ps_rows<16>(r, field, Lx, Lz, tmp, s);
+  if (c.pts == 4) launch_ps_cols<4>(c, tmp, Lx, Lz, out, s);
+  else if (c.pts == 8) launch_ps_cols<8>(c, tmp, Lx, Lz, out, s);
+  else launch_ps_cols<16>(c, tmp, Lx, Lz, out, s);
   return cudaGetLastError();
 }
 

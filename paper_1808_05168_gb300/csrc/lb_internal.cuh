@@ -485,7 +485,7 @@ template <class real>
 cudaError_t launch_columns(real* f, int Lx, int Lz, int x_first, int n, real* buf, bool to_buf, cudaStream_t s);
 
 // Power spectrum of one real double-precision field (Lx, Lz powers of two, 2..8192), with a
-// caller-provided scratch of Lx * Lz complex doubles; prepare once per device before use.
+// caller-provided scratch of (Lx/2 + 1) * Lz complex doubles; prepare once per device before use.
 cudaError_t prepare_power_spectrum();
 cudaError_t launch_power_spectrum(const double* field, int Lx, int Lz, double* out, void* tmp, cudaStream_t s);
 
