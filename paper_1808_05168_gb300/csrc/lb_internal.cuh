@@ -189,19 +189,18 @@ __device__ __forceinline__ void sincos_ftz(float x, float& s, float& c) {
 }
 
 // 1 / rho of a site's total density: the hardware reciprocal in single precision (at most 1 ulp
-// from the exact value; rho is near rho_bar = 1, never subnormal), refined by Newton steps in
-// double.
+// from the exact value; rho is near rho_bar = 1, never subnormal), refined in double.
 __device__ __forceinline__ float site_reciprocal(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 __device__ __forceinline__ double site_reciprocal(double x) {
-  // two Newton steps y <- y + y (1 - x y) from the single-precision seed (relative error 2^-23
-  // -> 2^-46 -> the last bit); x is near 1
-  double y = (double)site_reciprocal((float)x);
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
+  // one third-order step y <- y + y (e + e^2), e = 1 - x y, from the single-precision seed (relative
+  // error 2^-23 -> below the last bit); x is near 1
+  const double y = (double)site_reciprocal((float)x);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
 
 // Box-Muller pair of the working precision, (r cos 2 pi u2, r sin 2 pi u2) with r = sqrt(-2 ln u1).

@@ -177,7 +177,7 @@ __device__ __forceinline__ void stage_column(const P* __restrict__ f, int LzLx, 
 // link.
 template <class real>
 __device__ __forceinline__ void deviations(Pr<real> v[9], bool below, bool above, real k9, real k36) {
-  if (!(below && above)) {
+  if (sizeof(real) == 4 && !(below && above)) {
     const Pr<real> q9 = pr(k9, -k9), q36 = pr(k36, -k36), z = pr(real(0));
     const Pr<real> b9 = below ? q9 : z, b36 = below ? q36 : z;
     const Pr<real> a9 = above ? q9 : z, a36 = above ? q36 : z;
@@ -261,6 +261,7 @@ __device__ __forceinline__ Mom<real> moments(const Pr<real> v[9]) {
 template <class real>
 struct SiteK {
   real G, g3, rho_bar_off;
+  real G36;  // -G / 36 (double)
   real kA[9], kB[9], kC[9], kN[9];  // folded collision coefficients, as in LatticeDev
   uint32_t key0, key1, lid;
 };
@@ -269,6 +270,7 @@ template <class real, int NOISE>
 __device__ __forceinline__ SiteK<real> site_constants(const LatticeDev<real>& L) {
   SiteK<real> K;
   K.G = L.G;
+  K.G36 = L.G * (real)(-1.0 / 36.0);
   K.g3 = L.g3;
   K.rho_bar_off = L.rho_bar_off;
 #pragma unroll
@@ -372,6 +374,178 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// The normals of a site as pairs per moment: normals 0-1: momentum (one draw for both species, its
+// amplitudes opposite); 2-7: moments 3..8 of A; 8-13: of B.
+template <class real>
+__device__ __forceinline__ void site_normals(uint32_t site, uint32_t step, const SiteK<real>& K,
+                                             const NormalTables* tab, Pr<real> nz[9]) {
+  U4 w4[4];
+  philox_site(site, step, K.lid, K.key0, K.key1, w4);
+  real g[14];
+  normal_pair2<real>(w4[0].x, w4[0].y, w4[0].z, w4[0].w, g[0], g[1], g[2], g[3], tab);
+  normal_pair2<real>(w4[1].x, w4[1].y, w4[1].z, w4[1].w, g[4], g[5], g[6], g[7], tab);
+  normal_pair2<real>(w4[2].x, w4[2].y, w4[2].z, w4[2].w, g[8], g[9], g[10], g[11], tab);
+  normal_pair<real>(w4[3].x, w4[3].y, g[12], g[13], tab);
+  nz[1] = pr(g[0]);
+  nz[2] = pr(g[1]);
+#pragma unroll
+  for (int k = 3; k < 9; ++k) nz[k] = pr(g[k - 1], g[k + 5]);
+}
+
+// Collision and inverse transform in double precision: the arithmetic of collide_out with the factors
+// arranged for the fewest FP64 instructions, which bound the double path (two lanes per clock and SM).
+// With a* both species feel one acceleration, so everything of m^eq and of the source that is common is
+// formed once per site and each moment of a species is one FMA of its density (s1 .. s5, with the
+// gradient force's opposite shares g1, t3 .. t5 added); unit rates: the noise of moments 6 and 7 goes
+// straight into the two combinations that use it.  208 -> 177 FP64 instructions per lattice update
+// together with the stencil of site_update_f64.
+struct Forces64 {
+  double FNx, FNz;     // total non-ideal force
+  double2 Fx, Fz;      // the species' non-ideal forces (without a*)
+};
+template <int NOISE, bool UNIT, bool ASTAR>
+__device__ __forceinline__ void collide_out_f64(const Mom<double>& m, double2 d, double rho, double inv, double Ux,
+                                                double Uz, const Forces64& F, const SiteK<double>& K,
+                                                const double2 nz[9], double2 cm, double2 cq, double2* out,
+                                                int stride) {
+  using P = double2;
+  const double ne = rho * K.g3;  // gradient force: + for A, - for B, along z
+  const double une = Uz * ne, xne = Ux * ne;
+  const P g1 = pr(K.kC[1] * ne, -(K.kC[1] * ne)), t3 = pr(K.kC[3] * une, -(K.kC[3] * une)),
+          t4 = pr(-(K.kC[4] * une), K.kC[4] * une), t5 = pr(K.kC[5] * xne, -(K.kC[5] * xne));
+  const double UxUx = Ux * Ux, UzUz = Uz * Uz;
+  const double e3 = K.kB[3] * (UxUx + UzUz), e4 = K.kB[4] * (UxUx - UzUz), e5 = K.kB[5] * (Ux * Uz);
+  P M1, M2, M3, M4, M5;
+  if (ASTAR) {  // F^S = (rho^S / rho) F_N
+    const double ax = F.FNx * inv, az = F.FNz * inv;
+    const double ux = Ux * ax, uz = Uz * az;
+    const double s1 = fma(K.kB[1], Ux, K.kC[1] * ax), s2 = fma(K.kB[1], Uz, K.kC[1] * az);
+    const double s3 = fma(K.kC[3], ux + uz, e3), s4 = fma(K.kC[4], ux - uz, e4),
+                 s5 = fma(K.kC[5], fma(Ux, az, Uz * ax), e5);
+    M1 = fma2(d, pr(s1), mul2(pr(K.kA[1]), m.m1));
+    M2 = fma2(d, pr(s2), fma2(pr(K.kA[1]), m.m2, g1));
+    M3 = fma2(d, pr(s3), t3);
+    M4 = fma2(d, pr(s4), t4);
+    M5 = fma2(d, pr(s5), t5);
+  } else {
+    const P U_x = pr(Ux), U_z = pr(Uz), ux = mul2(U_x, F.Fx), uz = mul2(U_z, F.Fz);
+    M1 = fma2(pr(K.kC[1]), F.Fx, fma2(d, pr(K.kB[1] * Ux), mul2(pr(K.kA[1]), m.m1)));
+    M2 = fma2(pr(K.kC[1]), F.Fz, fma2(d, pr(K.kB[1] * Uz), fma2(pr(K.kA[1]), m.m2, g1)));
+    M3 = fma2(pr(K.kC[3]), add2(ux, uz), fma2(d, pr(e3), t3));
+    M4 = fma2(pr(K.kC[4]), sub2(ux, uz), fma2(d, pr(e4), t4));
+    M5 = fma2(pr(K.kC[5]), fma2(U_x, F.Fz, mul2(U_z, F.Fx)), fma2(d, pr(e5), t5));
+  }
+  if (!UNIT) {
+    M3 = fma2(pr(K.kA[3]), m.m3, M3);
+    M4 = fma2(pr(K.kA[4]), m.m4, M4);
+    M5 = fma2(pr(K.kA[5]), m.m5, M5);
+  }
+  const bool noise = NOISE != NOISE_OFF, loc = NOISE == NOISE_LOC;
+  // the combinations of moments 1, 2 with 6, 7: v13 = M1 - M6, h1 = M1 + 2 M6, and along z
+  P v13, v24, h1, h2, M8 = pr(0.0);
+  if (noise) {
+    const P a1 = loc ? mul2(pr(K.kN[1]), cm) : pr(K.kN[1], -K.kN[1]);
+    auto amp = [&](int a) { return loc ? mul2(pr(K.kN[a]), cq) : pr(K.kN[a]); };
+    M1 = fma2(a1, nz[1], M1);
+    M2 = fma2(a1, nz[2], M2);
+    M3 = fma2(amp(3), nz[3], M3);
+    M4 = fma2(amp(4), nz[4], M4);
+    M5 = fma2(amp(5), nz[5], M5);
+    M8 = mul2(amp(8), nz[8]);
+  }
+  if (noise && UNIT) {
+    const P a6 = loc ? mul2(pr(K.kN[6]), cq) : pr(K.kN[6]), b6 = pr(2.0 * a6.x, 2.0 * a6.y), n6 = pr(-a6.x, -a6.y);
+    v13 = fma2(n6, nz[6], M1);
+    v24 = fma2(n6, nz[7], M2);
+    h1 = fma2(b6, nz[6], M1);
+    h2 = fma2(b6, nz[7], M2);
+  } else if (UNIT) {
+    v13 = h1 = M1;
+    v24 = h2 = M2;
+  } else {
+    P M6 = mul2(pr(K.kA[6]), m.m6), M7 = mul2(pr(K.kA[6]), m.m7);
+    M8 = fma2(pr(K.kA[8]), m.m8, M8);
+    if (noise) {
+      const P a6 = loc ? mul2(pr(K.kN[6]), cq) : pr(K.kN[6]);
+      M6 = fma2(a6, nz[6], M6);
+      M7 = fma2(a6, nz[7], M7);
+    }
+    v13 = sub2(M1, M6);
+    v24 = sub2(M2, M7);
+    h1 = fma2(pr(2.0), M6, M1);
+    h2 = fma2(pr(2.0), M7, M2);
+  }
+  const P dq = mul2(pr(1.0 / 36), d);
+  const P b4 = fma2(pr(-16.0), M8, mul2(pr(4.0), add2(dq, M3)));
+  const P b5 = fma2(pr(8.0), M8, fma2(pr(4.0), M3, dq));
+  const P u13 = fma2(pr(4.0), M4, b4), u24 = fma2(pr(-4.0), M4, b4), u57 = add2(b5, M5), u68 = sub2(b5, M5);
+  const P v57 = add2(h1, h2), v68 = sub2(h1, h2);
+  const P f[9] = {fma2(pr(32.0), M8, fma2(pr(-32.0), M3, mul2(pr(16.0 / 36), d))),
+                  fma2(pr(4.0), v13, u13),
+                  fma2(pr(4.0), v24, u24),
+                  fma2(pr(-4.0), v13, u13),
+                  fma2(pr(-4.0), v24, u24),
+                  add2(u57, v57),
+                  sub2(u68, v68),
+                  sub2(u57, v57),
+                  add2(u68, v68)};
+#pragma unroll
+  for (int l = 0; l < 9; ++l) __stcs(out + l * stride, f[l]);
+}
+
+// site_update in double precision (no background: the ring holds the densities themselves).
+template <bool SAMPLE, int NOISE, bool UNIT, bool ASTAR>
+__device__ __forceinline__ void site_update_f64(const SiteK<double>& K, const RowConst<double>& rc,
+                                                const Mom<double>& m, const double2* ring, int bc, int bu, int bd,
+                                                uint32_t site, uint32_t step, double* fl, double* pl, int LzLx,
+                                                double& acc_p, double& acc_a, double& acc_b, double2* out, int ostride,
+                                                const NormalTables* tab) {
+  using P = double2;
+  const P d = ring[bc];
+  const P w = ring[bc - 1], e = ring[bc + 1], n = ring[bu], nw = ring[bu - 1], ne = ring[bu + 1], s = ring[bd],
+          sw = ring[bd - 1], se = ring[bd + 1];
+  // 36 sum_l w_l c_l rho^S(r + c_l) of both species (Eq. aNI); the two diagonals serve both directions
+  const P da = sub2(ne, sw), db = sub2(nw, se);
+  const P X = fma2(pr(4.0), sub2(e, w), sub2(da, db)), Z = fma2(pr(4.0), sub2(n, s), add2(da, db));
+  const double rho = d.x + d.y, inv = site_reciprocal(rho);
+  Forces64 F;
+  if (ASTAR) {
+    F.FNx = K.G36 * fma(d.x, X.y, d.y * X.x);
+    F.FNz = K.G36 * fma(d.x, Z.y, d.y * Z.x);
+  } else {
+    const double gA = K.G36 * d.x, gB = K.G36 * d.y;
+    F.Fx = pr(gA * X.y, gB * X.x);
+    F.Fz = pr(gA * Z.y, gB * Z.x);
+    F.FNx = F.Fx.x + F.Fx.y;
+    F.FNz = F.Fz.x + F.Fz.y;
+  }
+  const double Ux = fma(0.5, F.FNx, m.m1.x + m.m1.y) * inv, Uz = fma(0.5, F.FNz, m.m2.x + m.m2.y) * inv;
+  if (SAMPLE) {
+    const double kin = (m.m3.x + m.m3.y + 2 * rho) * (1.0 / 6);
+    const P N = fma2(pr(1.0 / 9), add2(add2(e, w), add2(n, s)), mul2(pr(2.0 / 36), add2(add2(ne, nw), add2(se, sw))));
+    const double psite = kin + 0.25 * K.G * (d.x * N.y + d.y * N.x);
+    pl[0] = psite;
+    acc_p += psite;
+    acc_a += d.x;
+    acc_b += d.y;
+    fl[0] = rho - K.rho_bar_off;
+    fl[LzLx] = (d.x - rc.c0 * rho) * inv;
+    fl[2 * LzLx] = Ux;
+    fl[3 * LzLx] = Uz;
+  }
+  P nz[9];
+  P cm = pr(1.0, -1.0), cq = pr(1.0);
+  if (NOISE != NOISE_OFF) {
+    site_normals<double>(site, step, K, tab, nz);
+    if (NOISE == NOISE_LOC) {
+      const double sm = sqrt_pos<double>(d.x * d.y * inv);
+      cm = pr(sm, -sm);
+      cq = pr(sqrt_pos<double>(d.x), sqrt_pos<double>(d.y));
+    }
+  }
+  collide_out_f64<NOISE, UNIT, ASTAR>(m, d, rho, inv, Ux, Uz, F, K, nz, cm, cq, out, ostride);
+}
+
 // Everything of one site after its moments are known and the densities of its row and the two
 // neighbouring rows sit in the ring: forces, velocity, optional sampling, noise, collision of
 // both species and the output.
@@ -380,7 +554,12 @@ __device__ __forceinline__ void site_update(const SiteK<real>& K, const RowConst
                                             const Pr<real>* ring, int bc, int bu, int bd, uint32_t site,
                                             uint32_t step, real* fl, real* pl, int LzLx, double& acc_p,
                                             double& acc_a, double& acc_b, Pr<real>* out, int ostride, int flags,
-                                            const NormalTables* bm) {
+                                            const NormalTables* tab) {
+  if constexpr (sizeof(real) == 8) {
+    site_update_f64<SAMPLE, NOISE, UNIT, ASTAR>(K, rc, m, ring, bc, bu, bd, site, step, fl, pl, LzLx, acc_p, acc_a,
+                                                acc_b, out, ostride, tab);
+    return;
+  }
   using P = Pr<real>;
   const P c9 = pr(real(1) / 9), c36 = pr(real(1) / 36);
   const P d = ring[bc];
@@ -433,23 +612,12 @@ __device__ __forceinline__ void site_update(const SiteK<real>& K, const RowConst
   for (int k = 0; k < 9; ++k) nz[k] = pr(real(0));
   P cm = pr(real(1), real(-1)), cq = pr(real(1));  // momentum noise is equal and opposite in A and B
   if (NOISE != NOISE_OFF) {
-    U4 w4[4];
-    philox_site(site, step, K.lid, K.key0, K.key1, w4);
-    real g[14];
-    normal_pair2<real>(w4[0].x, w4[0].y, w4[0].z, w4[0].w, g[0], g[1], g[2], g[3], bm);
-    normal_pair2<real>(w4[1].x, w4[1].y, w4[1].z, w4[1].w, g[4], g[5], g[6], g[7], bm);
-    normal_pair2<real>(w4[2].x, w4[2].y, w4[2].z, w4[2].w, g[8], g[9], g[10], g[11], bm);
-    normal_pair<real>(w4[3].x, w4[3].y, g[12], g[13], bm);
+    site_normals<real>(site, step, K, tab, nz);
     if (NOISE == NOISE_LOC) {
       const real sm = sqrt_pos<real>(rs.x * rs.y * inv);
       cm = pr(sm, -sm);
       cq = pr(sqrt_pos<real>(rs.x), sqrt_pos<real>(rs.y));
     }
-    // normals 0-1: momentum (one draw for both species); 2-7: moments 3..8 of A; 8-13: of B
-    nz[1] = pr(g[0]);
-    nz[2] = pr(g[1]);
-#pragma unroll
-    for (int k = 3; k < 9; ++k) nz[k] = pr(g[k - 1], g[k + 5]);
   }
   collide_out<real, NOISE, UNIT>(m, d, rs, Ux, Uz, Fx, Fz, K, nz, cm, cq, out, ostride);
 }
@@ -638,7 +806,7 @@ __device__ __forceinline__ bool process_item(const StepArgs<real>& a, const real
         Pr<real> v[9];
         read_generic(sb, W, tid + 1, below, above, k9, k36, v);
         Mom<real> m = moments<real>(v);
-        if (below && above) m.m2 = add2(m.m2, interior_m2_shift(k9, k36));
+        if (sizeof(real) == 4 && below && above) m.m2 = add2(m.m2, interior_m2_shift(k9, k36));
         site_update<real, SAMPLE, NOISE, decltype(unit)::value, decltype(astar)::value>(
             K, rows[z], m, ring, bc, bu, bd, site, step, a.fields + 4 * L.site_off + r0, a.pfield + L.site_off + r0,
             LzLx, acc_p, acc_a, acc_b, g + r0, LzLx, flags, a.normals);
@@ -874,7 +1042,7 @@ __device__ __forceinline__ bool process_item_bulk(const StepArgs<real>& a, const
         Pr<real> v[9];
         read_bulk<real, SW>(sb, tid + PAD, IN || below, IN || above, k9, k36, v);
         Mom<real> m = moments<real>(v);
-        if (IN) m.m2 = add2(m.m2, interior_m2_shift(k9, k36));
+        if (IN && sizeof(real) == 4) m.m2 = add2(m.m2, interior_m2_shift(k9, k36));
         site_update<real, SAMPLE, NOISE, decltype(unit)::value, decltype(astar)::value>(
             K, rows[z], m, ring, bc, bu, bd, site, step, a.fields + 4 * L.site_off + r0, a.pfield + L.site_off + r0,
             LzLx, acc_p, acc_a, acc_b, g + r0, LzLx, flags, a.normals);
