@@ -21,7 +21,8 @@
 //      population of the species, and pushes the result back along the streaming map (the
 //      transpose of the pull with mid-way bounce-back is a one-to-one scatter).
 // The forward states are recomputed segment by segment from checkpoints (every C steps) into a
-// ring of C states, so memory is O(T/C + C) states.
+// ring of C states, so memory is O(T/C + C) states.  Passes 2 and 3 come twice: arranged for the
+// default options, and with every option.
 //
 // Supported: every lattice of a batch at once, each with its own loss and gradient; the a*
 // correction on or off, wall ghosts copying the adjacent row or taking the fixed wall
@@ -181,7 +182,7 @@ __device__ __forceinline__ void normals14(uint32_t site, uint32_t step, const La
 // slot of `partials` (zeroed before the sweep; one fixed summation order, step after step).
 // The state may be single precision (FP32 deviations); the transposed step is evaluated in double
 // precision throughout, since the loss is a small difference of two runs' pressures.
-template <class real, bool NOISE, bool OPTS>
+template <class real, bool NOISE>
 __global__ void adj_local_kernel(const real* __restrict__ f, const double* __restrict__ fbar,
                                  const LatticeDev<real>* lat, const RowConst<real>* rows,
                                  const AdjConst* __restrict__ kcs, const AdjMap map, const double* __restrict__ rho,
@@ -202,9 +203,7 @@ __global__ void adj_local_kernel(const real* __restrict__ f, const double* __res
   fl += 18 * L.site_off;
   sb += 4 * L.site_off;
   double gG = 0, gS = 0, gD = 0;
-  // the default options (a* on, copy-rule ghosts, hom noise) are compiled without the branches
-  const bool astar = !OPTS || (L.flags & DF_ASTAR), fixed = OPTS && (L.flags & DF_WALL_FIXED),
-             loc = OPTS && NOISE && (L.flags & DF_NOISE_LOC);
+  const bool astar = L.flags & DF_ASTAR, fixed = L.flags & DF_WALL_FIXED, loc = NOISE && (L.flags & DF_NOISE_LOC);
   if (i < N) {
     const int x = i % Lx, z = i / Lx;
     double v[18];
@@ -495,6 +494,357 @@ __global__ void adj_gather_push_kernel(const LatticeDev<real>* lat, const RowCon
   }
 }
 
+// ---- the default options (a*, copy-rule ghosts, hom noise) ----------------------------------------
+// The transposed step is bound by the FP64 pipe (two lanes per clock and SM), so these kernels are
+// arranged for the fewest FP64 instructions: about 355 per site and step against about 1000 of the
+// kernels above, which remain for the other options.
+//  - what both species share is formed once from their density-weighted sums T_a = sum_s rho^S t^S_a;
+//  - with a* the sensitivities of m^eq and of the source act on the same combinations of the moments,
+//    so one dot product per species (K_1 .. K_5) gives both shares of rho^S;
+//  - the link weights, 1/N_a and the rates are folded into AdjConst;
+//  - the moments' sensitivities are handed over (3 per species with unit rates, else 9) and turned
+//    into populations by the gather, not written as 18 populations and read again;
+//  - what a site's pressure owes its neighbours' densities is, under the copy rule, what they owe it:
+//    the local pass adds it twice and the gather has only the forces' share to collect;
+//  - the parameters' shares stay per site (one addition each) instead of a warp reduction per step;
+//  - FP32 populations are widened by their bits (the conversion instruction runs at the FP64 rate).
+// 256 x 128, 500 steps, FP64: 62 -> 52 ms for the whole gradient; eight lattices from FP32 state, 300
+// steps: 133 -> 83 ms (the local pass 290 -> 171 us a step, the gather 92 -> 28).
+
+// A stored population as a double; exactly the conversion, in integer instructions where the value is
+// normal.
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = b & 0x7F800000u;
+  if (e == 0u || e == 0x7F800000u) return (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+template <class real>
+struct PairOfState;
+template <>
+struct PairOfState<float> {
+  using type = float2;
+};
+template <>
+struct PairOfState<double> {
+  using type = double2;
+};
+
+// Links 1..8 of both species pulled at (x, z): v[s][l], the wall rows' background shifts applied per
+// link (in interior rows they leave every moment but m_2 alone and the caller adds them there; none in
+// FP64).
+template <class real>
+__device__ __forceinline__ void pull_pairs(const real* __restrict__ f, const LatticeDev<real>& L, int x, int z,
+                                           double v[2][9]) {
+  using P = typename PairOfState<real>::type;
+  const P* g = reinterpret_cast<const P*>(f);
+  const int Lx = L.Lx, Lz = L.Lz, N = Lx * Lz;
+  const int xm = x == 0 ? Lx - 1 : x - 1, xp = x + 1 == Lx ? 0 : x + 1;
+  const bool wall = z == 0 || z == Lz - 1;
+  P w[9];
+#pragma unroll
+  for (int l = 1; l < 9; ++l) {
+    const int zs = z - LB_CZ(l), xs = LB_CX(l) == 0 ? x : (LB_CX(l) > 0 ? xm : xp);
+    const bool in = LB_CZ(l) == 0 || (zs >= 0 && zs < Lz);
+    w[l] = g[in ? l * N + zs * Lx + xs : LB_OPP(l) * N + z * Lx + x];
+  }
+#pragma unroll
+  for (int l = 1; l < 9; ++l) {
+    v[0][l] = widen(w[l].x);
+    v[1][l] = widen(w[l].y);
+    if (sizeof(real) == 4 && LB_CZ(l) != 0 && wall) {
+      const int zs = z - LB_CZ(l);
+      if (zs >= 0 && zs < Lz) {
+        const double q = l <= 4 ? (double)L.k9 : (double)L.k36, sh = LB_CZ(l) > 0 ? -q : q;
+        v[0][l] += sh;
+        v[1][l] -= sh;
+      }
+    }
+  }
+}
+
+template <class real, bool NOISE, bool UNIT>
+__global__ void __launch_bounds__(kAdjBlock)
+    adj_local_default(const real* __restrict__ f, const double* __restrict__ fbar, const LatticeDev<real>* lat,
+                      const AdjConst* __restrict__ kcs, const AdjMap map, const double* __restrict__ rho, uint32_t step,
+                      double sign, double* __restrict__ mom, double* __restrict__ sb, double* __restrict__ shares,
+                      const NormalTables* tab) {
+  constexpr int NM = UNIT ? 3 : 9;
+  const int li = adj_lattice(map);
+  const LatticeDev<real>& L = lat[li];
+  const AdjConst& k = kcs[li];
+  const int Lx = L.Lx, Lz = L.Lz, N = Lx * Lz, i = adj_site(map, li);
+  if (i >= N) return;
+  const int64_t so = L.site_off;
+  f += L.f_off;
+  fbar += 18 * so;
+  rho += 2 * so;
+  mom += 18 * so;
+  sb += 8 * so;
+  shares += 3 * so;
+  const int z = i / Lx, x = i - z * Lx;
+  const double alpha = sign * k.w_loss;  // weight of this site's pressure in the loss
+  const bool wall = z == 0 || z == Lz - 1;
+
+  // moments 1, 2, 4, 5 of both species
+  double m1[2], m2[2], m4[2], m5[2];
+  {
+    double v[2][9];
+    pull_pairs<real>(f, L, x, z, v);
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const double a57 = v[s][5] - v[s][7], a68 = v[s][6] - v[s][8];
+      m1[s] = (v[s][1] - v[s][3]) + (a57 - a68);
+      m2[s] = (v[s][2] - v[s][4]) + (a57 + a68);
+      m4[s] = (v[s][1] + v[s][3]) - (v[s][2] + v[s][4]);
+      m5[s] = (v[s][5] + v[s][7]) - (v[s][6] + v[s][8]);
+    }
+    if (sizeof(real) == 4 && !wall) {
+      const double q = 2 * (double)L.k9 + 4 * (double)L.k36;
+      m2[0] -= q;
+      m2[1] += q;
+    }
+  }
+  // neighbour sums: X, Z = 36 sum_l w_l c_l rho (Eq. aNI), n18 = 18 sum_l w_l |c_l|^2 rho; copy-rule ghosts
+  double r[2], X[2], Z[2], n18[2];
+  {
+    const int xm = x == 0 ? Lx - 1 : x - 1, xp = x + 1 == Lx ? 0 : x + 1;
+    const int zu = min(z + 1, Lz - 1) * Lx, zd = max(z - 1, 0) * Lx, zc = z * Lx;
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const double* p = rho + s * N;
+      const double e = p[zc + xp], w = p[zc + xm], n = p[zu + x], d = p[zd + x];
+      const double ne = p[zu + xp], nw = p[zu + xm], se = p[zd + xp], sw = p[zd + xm];
+      const double da = ne - sw, db = nw - se;
+      r[s] = p[i];
+      X[s] = fma(4.0, e - w, da - db);
+      Z[s] = fma(4.0, n - d, da + db);
+      n18[s] = fma(2.0, (e + w) + (n + d), (ne + sw) + (nw + se));
+    }
+  }
+  const double G = L.G, Gm = G * (-1.0 / 36.0);
+  const double inv = site_reciprocal(r[0] + r[1]);
+  const double Tx = fma(r[0], X[1], r[1] * X[0]), Tz = fma(r[0], Z[1], r[1] * Z[0]);
+  const double Fx = Gm * Tx, Fz = Gm * Tz;          // F_N
+  const double ax = Fx * inv, az = Fz * inv;        // F_N / rho
+  const double ne = (r[0] + r[1]) * (double)L.g3;   // gradient forcing, + for A, - for B
+  const double Px = fma(0.5, Fx, m1[0] + m1[1]), Pz = fma(0.5, Fz, m2[0] + m2[1]);
+  const double Ux = Px * inv, Uz = Pz * inv;
+  const double UxUx = Ux * Ux, UzUz = Uz * Uz, UxUz = Ux * Uz, Ud = UxUx - UzUz;
+  const double ux = Ux * ax, uz = Uz * az, ap = ux + uz, am = ux - uz, cr = fma(Uz, ax, Ux * az);
+
+  // t_a: the moments of w_l fbar_l up to a factor each (sbar_a = t_0/36, t_1/12, t_2/12, t_3/36, t_4/4,
+  // t_5/4, t_6/12, t_7/12, t_8/72 with the 1/N_a of the transposed inverse transform)
+  double t[2][9];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    double g[9];
+#pragma unroll
+    for (int l = 0; l < 9; ++l) g[l] = fbar[(s * 9 + l) * N + i];
+    const double s57 = g[5] + g[7], s68 = g[6] + g[8], a57 = g[5] - g[7], a68 = g[6] - g[8];
+    const double s13 = g[1] + g[3], s24 = g[2] + g[4], d13 = g[1] - g[3], d24 = g[2] - g[4];
+    const double dg = s57 + s68, e = s13 + s24, amm = a57 - a68, app = a57 + a68;
+    t[s][0] = fma(16.0, g[0], fma(4.0, e, dg));
+    t[s][1] = fma(4.0, d13, amm);
+    t[s][2] = fma(4.0, d24, app);
+    t[s][3] = fma(-8.0, g[0], e + dg);
+    t[s][4] = s13 - s24;
+    t[s][5] = s57 - s68;
+    if (!UNIT) {
+      t[s][6] = fma(-2.0, d13, amm);
+      t[s][7] = fma(-2.0, d24, app);
+      t[s][8] = fma(4.0, g[0], fma(-2.0, e, dg));
+    }
+  }
+  // shares of rho^S through m^eq and through the source
+  const double K1 = fma(k.l1, Ux, k.o1 * ax), K2 = fma(k.l1, Uz, k.o1 * az);
+  const double K3 = fma(k.l3, UxUx + UzUz, k.o3 * ap), K4 = fma(k.l4, Ud, k.o4 * am), K5 = fma(k.l4, UxUz, k.o5 * cr);
+  double rb[2];
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+    rb[s] = fma(t[s][5], K5, fma(t[s][4], K4, fma(t[s][3], K3, fma(t[s][2], K2, fma(t[s][1], K1, t[s][0] * (1.0 / 36))))));
+  double T[6], d[6];
+#pragma unroll
+  for (int a = 1; a < 6; ++a) {
+    T[a] = fma(r[0], t[0][a], r[1] * t[1][a]);
+    d[a] = t[0][a] - t[1][a];
+  }
+  const double p = (2 * k.l3) * T[3], q = (2 * k.l4) * T[4], rr = k.l4 * T[5];
+  const double po = k.o3 * T[3], qo = k.o4 * T[4], ro = k.o5 * T[5];
+  const double sp = po + qo, sm = po - qo, k34 = fma(k.o3, d[3], -(k.o4 * d[4])), o5d = k.o5 * d[5];
+  const double Ubx = fma(o5d, ne, fma(ro, az, fma(sp, ax, fma(rr, Uz, fma(p + q, Ux, k.l1 * T[1])))));
+  const double Ubz = fma(k34, ne, fma(ro, ax, fma(sm, az, fma(rr, Ux, fma(p - q, Uz, k.l1 * T[2])))));
+  const double Wx = fma(ro, Uz, fma(sp, Ux, k.o1 * T[1])), Wz = fma(ro, Ux, fma(sm, Uz, k.o1 * T[2]));
+  const double Pbx = Ubx * inv, Pbz = Ubz * inv;
+  const double FNbx = fma(0.5, Pbx, Wx * inv), FNbz = fma(0.5, Pbz, Wz * inv);
+  const double invb = fma(Wx, Fx, fma(Wz, Fz, fma(Ubx, Px, Ubz * Pz)));
+  const double rt = fma((double)L.g3, fma(o5d, Ux, fma(k34, Uz, k.o1 * d[2])), -(invb * (inv * inv)));
+  const double yx = Gm * FNbx, yz = Gm * FNbz, pg = (alpha * (1.0 / 36)) * G;
+  rb[0] += fma(pg, n18[1], fma(yx, X[1], fma(yz, Z[1], rt)));
+  rb[1] += fma(pg, n18[0], fma(yx, X[0], fma(yz, Z[0], rt)));
+  // sensitivities of the neighbour sums (by 36): (x, z, x + z, z - x) of A, then of B
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const double sx = yx * r[1 - s], sz = yz * r[1 - s];
+    double* o = sb + (int64_t)(4 * s) * N + i;
+    o[0] = sx;
+    o[N] = sz;
+    o[2 * (int64_t)N] = sx + sz;
+    o[3 * (int64_t)N] = sz - sx;
+  }
+  // the parameters' shares
+  const double gG = fma(alpha * (1.0 / 72), fma(r[0], n18[1], r[1] * n18[0]), fma(FNbx, Tx, FNbz * Tz) * (-1.0 / 36));
+  double ld = fma(T[1], fma(-0.5, ax, Ux), T[2] * fma(-0.5, az, Uz));
+  ld = fma(-0.5 * ne, d[2], ld);
+  double ls = fma(T[4], Ud - am, T[5] * fma(-0.5, cr, UxUz));
+  ls = fma(ne, fma(Uz, d[4], -0.5 * (Ux * d[5])), ls);
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    ld = fma(-t[s][1], m1[s], fma(-t[s][2], m2[s], ld));
+    ls = fma(-t[s][4], m4[s], fma(-t[s][5], m5[s], ls));
+  }
+  if (NOISE) {
+    real nn[14];
+    normals14<real>((uint32_t)i, step, L, tab, nn);
+    ld = fma(k.dsm, fma(widen(nn[0]), d[1], widen(nn[1]) * d[2]), ld);
+    ls = fma(k.d4, fma(t[0][4], widen(nn[3]), t[1][4] * widen(nn[9])), ls);
+    ls = fma(k.d5, fma(t[0][5], widen(nn[4]), t[1][5] * widen(nn[10])), ls);
+  }
+  shares[i] += gG;
+  shares[N + i] = fma(0.25, ls, shares[N + i]);
+  shares[2 * (int64_t)N + i] = fma(1.0 / 12, ld, shares[2 * (int64_t)N + i]);
+  // the moments' sensitivities
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    double* o = mom + (int64_t)(NM * s) * N + i;
+    o[0] = rb[s];
+    o[N] = fma(k.b1, t[s][1], Pbx);
+    o[2 * (int64_t)N] = fma(k.b1, t[s][2], Pbz);
+    if (!UNIT) {
+      o[3 * (int64_t)N] = k.b3 * t[s][3];
+      o[4 * (int64_t)N] = k.b4 * t[s][4];
+      o[5 * (int64_t)N] = k.b4 * t[s][5];
+      o[6 * (int64_t)N] = k.b6 * t[s][6];
+      o[7 * (int64_t)N] = k.b6 * t[s][7];
+      o[8 * (int64_t)N] = k.b8 * t[s][8];
+    }
+  }
+}
+
+// Gather the forces' share of the neighbours, turn the moments' sensitivities into populations and push
+// them along the transposed streaming map; with f_next also the densities of the state before.  Two
+// threads per site, one per species, as adj_gather_push_kernel.
+template <class real, bool UNIT>
+__global__ void __launch_bounds__(2 * kAdjBlock)
+    adj_push_default(const LatticeDev<real>* lat, const RowConst<real>* rows, const AdjConst* __restrict__ kcs,
+                     const AdjMap map, const double* __restrict__ mom, const double* __restrict__ sb, double sign,
+                     double* __restrict__ fbar_prev, const real* __restrict__ f_next, double* __restrict__ rho_next) {
+  constexpr int NM = UNIT ? 3 : 9;
+  const int li = adj_lattice(map);
+  const LatticeDev<real>& L = lat[li];
+  const int Lx = L.Lx, Lz = L.Lz, N = Lx * Lz;
+  const int t = adj_site(map, li), i = t >> 1, sp = t & 1;  // site, species
+  if (i >= N) return;
+  const int64_t so = L.site_off;
+  const int z = i / Lx, x = i - z * Lx;
+  const int xm = x == 0 ? Lx - 1 : x - 1, xp = x + 1 == Lx ? 0 : x + 1;
+  const bool wall = z == 0 || z == Lz - 1;
+  if (f_next) {  // this species' density of f_next at the site (interior rows: the shifts sum to zero)
+    const real* g = f_next + L.f_off;
+    double a = 0;
+#pragma unroll
+    for (int l = 0; l < 9; ++l) {
+      const int zs = z - LB_CZ(l), xs = LB_CX(l) == 0 ? x : (LB_CX(l) > 0 ? xm : xp);
+      const bool in = LB_CZ(l) == 0 || (zs >= 0 && zs < Lz);
+      a += widen(g[2 * (in ? l * N + zs * Lx + xs : LB_OPP(l) * N + z * Lx + x) + sp]);
+    }
+    if (sizeof(real) == 4) {
+      const RowConst<real>& rc = rows[L.row_off + z];
+      a += (double)(sp == 0 ? rc.bgA : rc.bgB);
+      if (wall) {  // link 2 (or 4), and 5, 6 (or 7, 8), carry their shift
+        const double q = (double)L.k9 + 2 * (double)L.k36;
+        if (z > 0) a += sp == 0 ? -q : q;
+        if (z < Lz - 1) a += sp == 0 ? q : -q;
+      }
+    }
+    rho_next[2 * so + (int64_t)sp * N + i] = a;
+  }
+  const double* sx = sb + 8 * so + (int64_t)(4 * sp) * N;
+  const double *sz = sx + N, *s5 = sz + N, *s6 = s5 + N;  // x + z, z - x
+  double rb;
+  if (!wall) {
+    const int zc = z * Lx, zu = zc + Lx, zd = zc - Lx;
+    rb = fma(4.0, (sx[zc + xm] - sx[zc + xp]) + (sz[zd + x] - sz[zu + x]),
+             (s5[zd + xm] - s5[zu + xp]) + (s6[zd + xp] - s6[zu + xm]));
+  } else {
+    // link by link: the neighbours inside the walls, and through the ghost next to this row (a copy of
+    // it) the sites of this row
+    rb = 0.0;
+#pragma unroll
+    for (int l = 1; l < 9; ++l) {
+      const int xs = LB_CX(l) == 0 ? x : (LB_CX(l) > 0 ? xm : xp), zs = z - LB_CZ(l);
+      auto owed = [&](int zz) {
+        const int j = zz * Lx + xs;
+        return (l <= 4 ? 4.0 : 1.0) * ((double)LB_CX(l) * sx[j] + (double)LB_CZ(l) * sz[j]);
+      };
+      if (zs >= 0 && zs < Lz) rb += owed(zs);
+      if ((z == 0 && LB_CZ(l) == -1) || (z == Lz - 1 && LB_CZ(l) == 1)) rb += owed(z);
+    }
+  }
+  const double* mo = mom + 18 * so + (int64_t)(NM * sp) * N + i;
+  const double alpha = sign * kcs[li].w_loss;
+  double o[9];
+  if (UNIT) {
+    const double m0 = mo[0] + rb, m1 = mo[N], m2 = mo[2 * (int64_t)N];
+    const double ma = fma(0.5, alpha, m0), md = m0 + alpha;  // kinetic pressure: alpha |c_l|^2 / 2
+    const double hp = m1 + m2, hm = m1 - m2;
+    o[0] = m0;
+    o[1] = ma + m1;
+    o[2] = ma + m2;
+    o[3] = ma - m1;
+    o[4] = ma - m2;
+    o[5] = md + hp;
+    o[6] = md - hm;
+    o[7] = md - hp;
+    o[8] = md + hm;
+  } else {
+    double m[9];
+#pragma unroll
+    for (int a = 0; a < 9; ++a) m[a] = mo[(int64_t)a * N];
+    m[0] += rb;
+    transpose_moments(m, o);
+#pragma unroll
+    for (int l = 1; l < 9; ++l) o[l] += l <= 4 ? 0.5 * alpha : alpha;
+  }
+  double* out = fbar_prev + 18 * so;
+#pragma unroll
+  for (int l = 0; l < 9; ++l) {
+    const int zs = z - LB_CZ(l), xs = LB_CX(l) == 0 ? x : (LB_CX(l) > 0 ? xm : xp);
+    const bool in = LB_CZ(l) == 0 || (zs >= 0 && zs < Lz);
+    out[in ? (sp * 9 + l) * (int64_t)N + zs * Lx + xs : (sp * 9 + LB_OPP(l)) * (int64_t)N + z * Lx + x] = o[l];
+  }
+}
+
+// grads[3 i + p] = sum over the sites of lattice i of its parameter shares [3][N]: block (i, p), threads
+// strided over the sites, then a fixed tree (deterministic).
+template <class real>
+__global__ void __launch_bounds__(1024) adj_sum_shares(const double* shares, const LatticeDev<real>* lat, double* grads) {
+  const LatticeDev<real>& L = lat[blockIdx.x];
+  const int N = L.Lx * L.Lz;
+  const double* p = shares + 3 * L.site_off + (int64_t)blockIdx.y * N;
+  double a = 0;
+  for (int i = threadIdx.x; i < N; i += 1024) a += p[i];
+  __shared__ double red[32];
+  a = warp_sum(a);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    a = warp_sum(red[threadIdx.x]);
+    if (threadIdx.x == 0) grads[3 * blockIdx.x + blockIdx.y] = a;
+  }
+}
+
 // grads[3 i + k] = sum over the blocks b of lattice i of partials[3 b + k]: one warp per lattice
 // (block i), lanes strided over the blocks, then a fixed butterfly (deterministic).
 __global__ void adj_sum_partials(const double* partials, const AdjMap map, double* grads) {
@@ -523,36 +873,52 @@ __global__ void adj_sum_partials(const double* partials, const AdjMap map, doubl
 template <class real>
 cudaError_t launch_adjoint_step(const real* f_prev, const real* f_next, const double* fbar, double* fbar_prev,
                                 const LatticeDev<real>* lat, const RowConst<real>* rows, const AdjConst* kcs,
-                                bool options, const AdjMap& map, uint32_t step, bool noise, double sign,
+                                bool options, bool unit, const AdjMap& map, uint32_t step, bool noise, double sign,
                                 bool rho_ready, double* rho, double* rho_next, double* fl, double* sb,
                                 double* partials, const NormalTables* tab, cudaStream_t s) {
   const int nb = map.n_blocks;
   if (!rho_ready) adj_rho_kernel<real><<<nb, kAdjBlock, 0, s>>>(f_prev, lat, rows, map, rho);
-  auto local = [&](auto noise_c, auto opts_c) {
-    adj_local_kernel<real, decltype(noise_c)::value, decltype(opts_c)::value>
-        <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, rows, kcs, map, rho, step, sign, fl, sb, partials, tab);
-  };
   using T = std::true_type;
   using F = std::false_type;
-  if (noise) options ? local(T(), T()) : local(T(), F());
-  else options ? local(F(), T()) : local(F(), F());
-  adj_gather_push_kernel<real>
-      <<<nb, 2 * kAdjBlock, 0, s>>>(lat, rows, kcs, map, rho, fl, sb, sign, fbar_prev, f_next, rho_next);
+  if (options) {
+    auto local = [&](auto noise_c) {
+      adj_local_kernel<real, decltype(noise_c)::value>
+          <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, rows, kcs, map, rho, step, sign, fl, sb, partials, tab);
+    };
+    noise ? local(T()) : local(F());
+    adj_gather_push_kernel<real>
+        <<<nb, 2 * kAdjBlock, 0, s>>>(lat, rows, kcs, map, rho, fl, sb, sign, fbar_prev, f_next, rho_next);
+    return cudaGetLastError();
+  }
+  auto pair = [&](auto noise_c, auto unit_c) {
+    constexpr bool U = decltype(unit_c)::value;
+    adj_local_default<real, decltype(noise_c)::value, U>
+        <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, kcs, map, rho, step, sign, fl, sb, partials, tab);
+    adj_push_default<real, U>
+        <<<nb, 2 * kAdjBlock, 0, s>>>(lat, rows, kcs, map, fl, sb, sign, fbar_prev, f_next, rho_next);
+  };
+  if (noise) unit ? pair(T(), T()) : pair(T(), F());
+  else unit ? pair(F(), T()) : pair(F(), F());
   return cudaGetLastError();
 }
 
-cudaError_t launch_adjoint_gradient(const double* partials, const AdjMap& map, double* grads, cudaStream_t s) {
-  adj_sum_partials<<<map.n_lat, 32, 0, s>>>(partials, map, grads);
+template <class real>
+cudaError_t launch_adjoint_gradient(const double* partials, const LatticeDev<real>* lat, bool options,
+                                    const AdjMap& map, double* grads, cudaStream_t s) {
+  if (options) adj_sum_partials<<<map.n_lat, 32, 0, s>>>(partials, map, grads);
+  else adj_sum_shares<real><<<dim3(map.n_lat, 3), 1024, 0, s>>>(partials, lat, grads);
   return cudaGetLastError();
 }
 
-template cudaError_t launch_adjoint_step<float>(const float*, const float*, const double*, double*,
-                                                const LatticeDev<float>*, const RowConst<float>*, const AdjConst*,
-                                                bool, const AdjMap&, uint32_t, bool, double, bool, double*, double*,
-                                                double*, double*, double*, const NormalTables*, cudaStream_t);
-template cudaError_t launch_adjoint_step<double>(const double*, const double*, const double*, double*,
-                                                 const LatticeDev<double>*, const RowConst<double>*, const AdjConst*,
-                                                 bool, const AdjMap&, uint32_t, bool, double, bool, double*, double*,
-                                                 double*, double*, double*, const NormalTables*, cudaStream_t);
+#define LB_ADJ_INST(real)                                                                                             \
+  template cudaError_t launch_adjoint_step<real>(const real*, const real*, const double*, double*,                    \
+                                                 const LatticeDev<real>*, const RowConst<real>*, const AdjConst*,     \
+                                                 bool, bool, const AdjMap&, uint32_t, bool, double, bool, double*,    \
+                                                 double*, double*, double*, double*, const NormalTables*,             \
+                                                 cudaStream_t);                                                       \
+  template cudaError_t launch_adjoint_gradient<real>(const double*, const LatticeDev<real>*, bool, const AdjMap&,     \
+                                                     double*, cudaStream_t);
+LB_ADJ_INST(float)
+LB_ADJ_INST(double)
 
 }  // namespace lbk

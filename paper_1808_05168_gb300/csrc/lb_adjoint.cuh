@@ -26,6 +26,10 @@ struct AdjConst {
   double pm, dpm, pa[9], dp4, dp5;
   bool options;   // any of no a*, fixed wall composition, loc noise (the kernels that handle them)
   double w_loss;  // 1 / (T N): the loss's weight of one site's pressure at one step (set per call)
+  // The default options' kernels: the factors of m^eq (l*), of the source (o*) and of the moments
+  // themselves (b*) with 1/N_a and the weights of the links folded in (adj_local_default).
+  double l1, l3, l4, o1, o3, o4, o5, b1, b3, b4, b6, b8;
+  bool unit;      // the rates of moments 3..8 are 1: their b* vanish
 };
 
 template <class real>
@@ -43,6 +47,11 @@ inline AdjConst adjoint_constants(const LatticeDev<real>& L) {
   for (int a = 0; a < 9; ++a) k.pa[a] = a >= 3 ? (double)L.pref[a] : 0.0;
   k.dp4 = dsigma(k.pa[4], ls);
   k.dp5 = dsigma(k.pa[5], ls);
+  const double le = (double)L.lam[3], lq = (double)L.lam[6], leps = (double)L.lam[8];
+  k.l1 = ld / 12, k.l3 = le / 12, k.l4 = ls / 4;
+  k.o1 = (1 - 0.5 * ld) / 12, k.o3 = (1 - 0.5 * le) / 6, k.o4 = (1 - 0.5 * ls) / 2, k.o5 = (1 - 0.5 * ls) / 4;
+  k.b1 = (1 - ld) / 12, k.b3 = (1 - le) / 36, k.b4 = (1 - ls) / 4, k.b6 = (1 - lq) / 12, k.b8 = (1 - leps) / 72;
+  k.unit = L.flags & DF_UNIT;
   k.options = !(L.flags & DF_ASTAR) || (L.flags & (DF_WALL_FIXED | DF_NOISE_LOC));
   return k;
 }
@@ -66,13 +75,17 @@ struct AdjMap {
 // go to rho_next for the next step.  kcs: the lattices' AdjConst (device); options: any lattice
 // uses a non-default option of the step; sign: +1 for the noisy run, -1 for the noiseless one
 // (the loss weight of a site is sign w_loss).  The sensitivities are double precision for either
-// state precision.
+// state precision.  Without options the parameter shares are kept per site instead, 3 doubles at
+// 3 site_off ([3][N] per lattice), and sb takes 8 doubles per site; unit: every lattice's rates of
+// moments 3..8 are 1.
 template <class real>
 cudaError_t launch_adjoint_step(const real* f_prev, const real* f_next, const double* fbar, double* fbar_prev,
                                 const LatticeDev<real>* lat, const RowConst<real>* rows, const AdjConst* kcs,
-                                bool options, const AdjMap& map, uint32_t step, bool noise, double sign,
+                                bool options, bool unit, const AdjMap& map, uint32_t step, bool noise, double sign,
                                 bool rho_ready, double* rho, double* rho_next, double* fl, double* sb,
                                 double* partials, const NormalTables* tab, cudaStream_t s);
-cudaError_t launch_adjoint_gradient(const double* partials, const AdjMap& map, double* grads, cudaStream_t s);
+template <class real>
+cudaError_t launch_adjoint_gradient(const double* partials, const LatticeDev<real>* lat, bool options,
+                                    const AdjMap& map, double* grads, cudaStream_t s);
 
 }  // namespace lbk

@@ -1089,7 +1089,7 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
     AdjMap map{nullptr, nullptr, 0, 0};
     std::vector<int> first, lat_of;  // the adjoint's blocks, lattice by lattice
     std::vector<AdjConst> hkcs;      // the lattices' constants of the transposed step
-    bool options = false;
+    bool options = false, unit = true;
     int noise = NOISE_OFF;
     double sign = 1.0;
     int fcur = 0;
@@ -1145,6 +1145,7 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
           make_lattice<real>(p, c->flags, c->dev32, R.x->f_off[i], R.x->site_off[i], R.x->row_off[i]));
       R.hkcs[i].w_loss = 1.0 / ((double)T * (double)(p.Lx * p.Lz));
       R.options = R.options || R.hkcs[i].options;
+      R.unit = R.unit && R.hkcs[i].unit;
     }
   }
   for (int pass = 0; pass < 2; ++pass) {
@@ -1169,8 +1170,8 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
         R.fb = (double*)piece(2 * R.S, sizeof(double));
         R.rho = (double*)piece(4 * R.NS, sizeof(double));  // two density sets
         R.fl = (double*)piece(R.S, sizeof(double));
-        R.sb = (double*)piece(4 * R.NS, sizeof(double));
-        R.gpart = (double*)piece((size_t)3 * nblk, sizeof(double));
+        R.sb = (double*)piece(8 * R.NS, sizeof(double));
+        R.gpart = (double*)piece(3 * (R.options ? (size_t)nblk : R.NS), sizeof(double));
         R.map_buf = (int*)piece((size_t)nblk + n + 1, sizeof(int));
         R.kcs = (AdjConst*)piece(n, sizeof(AdjConst));
       }
@@ -1212,7 +1213,7 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
   {
     NvtxRange rr("lb adjoint: forward runs");
     for (Run& R : runs) {
-      if (want_grad) ok(cudaMemsetAsync(R.gpart, 0, (size_t)3 * R.map.n_blocks * sizeof(double), R.s));
+      if (want_grad) ok(cudaMemsetAsync(R.gpart, 0, 3 * (R.options ? (size_t)R.map.n_blocks : R.NS) * sizeof(double), R.s));
       for (int i = 0; i < n; ++i) {
         const lb_params& p = R.x->params[i];
         const BgParams bp{p.Lx, p.Lz, c->dev32 ? 1 : 0, kRhoBar, p.grad_c0};
@@ -1254,7 +1255,7 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
           ok(launch_adjoint_step<real>(R.ring + (k - c0) * R.S, k > c0 ? R.ring + (k - 1 - c0) * R.S : nullptr,
                                        R.fb + R.fcur * R.S, R.fb + (1 - R.fcur) * R.S,
                                        (const LatticeDev<real>*)R.x->d_lat, (const RowConst<real>*)R.x->d_rows, R.kcs,
-                                       R.options, R.map, (uint32_t)k, R.noise != NOISE_OFF, R.sign, k < c0 + len - 1,
+                                       R.options, R.unit, R.map, (uint32_t)k, R.noise != NOISE_OFF, R.sign, k < c0 + len - 1,
                                        rho_k, rho_n, R.fl, R.sb, R.gpart, c->normals, R.s));
           R.fcur = 1 - R.fcur;
         }
@@ -1262,7 +1263,8 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
       }
     }
     for (int q = 0; q < 2 && e == cudaSuccess; ++q)
-      ok(launch_adjoint_gradient(runs[q].gpart, runs[q].map, d_grad + (size_t)3 * n * q, runs[q].s));
+      ok(launch_adjoint_gradient<real>(runs[q].gpart, (const LatticeDev<real>*)runs[q].x->d_lat, runs[q].options,
+                                       runs[q].map, d_grad + (size_t)3 * n * q, runs[q].s));
   }
   // join the second stream, then read the results
   ok(cudaEventRecord(ev[1], s1));
