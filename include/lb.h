@@ -270,8 +270,9 @@ int lb_power_spectrum_noalloc(const double* field, int Lx, int Lz, double* out, 
  * (LB_WALL_FIXED), hom or loc noise (LB_NOISE_LOC, whose amplitudes follow the local densities).
  * The runs with and without noise are independent until they are combined and run on two
  * streams (the context's and one of the call's own), each with its own buffers; the noiseless one,
- * uniform in x, on two columns.  Device memory: about steps/ckpt_every + ckpt_every + 8 states,
- * allocated for the call and freed before it returns.  Synchronous. */
+ * uniform in x, on two columns.  Device memory: about steps/ckpt_every + 1.4 ckpt_every + 8 states
+ * (default options without the gradient: 33 states, 1 GB at most where two are less), allocated for
+ * the call and freed before it returns.  Synchronous. */
 int lb_pressure_shift_gradient(lb_ctx* ctx, int64_t steps, int64_t ckpt_every, double grad[3], double* loss);
 
 /* lb_pressure_shift_gradient for every lattice of a batch in one sweep: each lattice's own loss

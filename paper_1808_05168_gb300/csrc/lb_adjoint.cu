@@ -531,24 +531,30 @@ struct PairOfState<double> {
   using type = double2;
 };
 
-// Links 1..8 of both species pulled at (x, z): v[s][l], the wall rows' background shifts applied per
-// link (in interior rows they leave every moment but m_2 alone and the caller adds them there; none in
-// FP64).
+// The nine pairs pulled at (x, z), as stored (Eq. LB, reflected at the walls).
 template <class real>
-__device__ __forceinline__ void pull_pairs(const real* __restrict__ f, const LatticeDev<real>& L, int x, int z,
-                                           double v[2][9]) {
+__device__ __forceinline__ void load_pairs(const real* __restrict__ f, int Lx, int Lz, int x, int z,
+                                           typename PairOfState<real>::type w[9]) {
   using P = typename PairOfState<real>::type;
   const P* g = reinterpret_cast<const P*>(f);
-  const int Lx = L.Lx, Lz = L.Lz, N = Lx * Lz;
-  const int xm = x == 0 ? Lx - 1 : x - 1, xp = x + 1 == Lx ? 0 : x + 1;
-  const bool wall = z == 0 || z == Lz - 1;
-  P w[9];
+  const int N = Lx * Lz, xm = x == 0 ? Lx - 1 : x - 1, xp = x + 1 == Lx ? 0 : x + 1;
 #pragma unroll
-  for (int l = 1; l < 9; ++l) {
+  for (int l = 0; l < 9; ++l) {
     const int zs = z - LB_CZ(l), xs = LB_CX(l) == 0 ? x : (LB_CX(l) > 0 ? xm : xp);
     const bool in = LB_CZ(l) == 0 || (zs >= 0 && zs < Lz);
     w[l] = g[in ? l * N + zs * Lx + xs : LB_OPP(l) * N + z * Lx + x];
   }
+}
+
+// Links 1..8 of both species widened, v[s][l], the wall rows' background shifts applied per link (in
+// interior rows they leave every moment but m_2 alone and the caller adds them there; none in FP64).
+template <class real>
+__device__ __forceinline__ void pull_pairs(const real* __restrict__ f, const LatticeDev<real>& L, int x, int z,
+                                           double v[2][9]) {
+  typename PairOfState<real>::type w[9];
+  const int Lz = L.Lz;
+  const bool wall = z == 0 || z == Lz - 1;
+  load_pairs<real>(f, L.Lx, Lz, x, z, w);
 #pragma unroll
   for (int l = 1; l < 9; ++l) {
     v[0][l] = widen(w[l].x);
@@ -562,6 +568,133 @@ __device__ __forceinline__ void pull_pairs(const real* __restrict__ f, const Lat
       }
     }
   }
+}
+
+// ---- densities and pressures of a segment's states -------------------------------------------------
+// The wall rows' shifts on the stored FP32 pairs, as `deviations` of the step kernels.
+__device__ __forceinline__ void shift_wall32(float2 w[9], bool below, bool above, float k9, float k36) {
+  const float b9 = below ? k9 : 0.f, b36 = below ? k36 : 0.f, a9 = above ? k9 : 0.f, a36 = above ? k36 : 0.f;
+  w[2] = make_float2(w[2].x - b9, w[2].y + b9);
+  w[4] = make_float2(w[4].x + a9, w[4].y - a9);
+  w[5] = make_float2(w[5].x - b36, w[5].y + b36);
+  w[6] = make_float2(w[6].x - b36, w[6].y + b36);
+  w[7] = make_float2(w[7].x + a36, w[7].y - a36);
+  w[8] = make_float2(w[8].x + a36, w[8].y - a36);
+}
+
+// Pre-collision densities of every site of the `gridDim.y` states at f, f + S, ..: absolute densities in
+// double (rho: [2][N] per lattice at 2 site_off, states 2 NS apart; null: not wanted) and, for FP32, the
+// deviations in single precision, summed as the step kernels do (dev: pairs at site_off, NS apart).
+template <class real>
+__global__ void __launch_bounds__(kAdjBlock)
+    adj_density_default(const real* __restrict__ f, int64_t S, const LatticeDev<real>* lat, const RowConst<real>* rows,
+                        const AdjMap map, double* __restrict__ rho, float2* __restrict__ dev, int64_t NS) {
+  const int li = adj_lattice(map);
+  const LatticeDev<real>& L = lat[li];
+  const int Lx = L.Lx, Lz = L.Lz, N = Lx * Lz, i = adj_site(map, li);
+  if (i >= N) return;
+  const int z = i / Lx, x = i - z * Lx, k = blockIdx.y;
+  typename PairOfState<real>::type w[9];
+  load_pairs<real>(f + k * S + L.f_off, Lx, Lz, x, z, w);
+  if constexpr (sizeof(real) == 4) {
+    if (z == 0 || z == Lz - 1) {
+      // absolute: the shifts of the non-reflected links in double (in interior rows they sum to zero)
+      if (rho) {
+        const double q = (double)L.k9 + 2 * (double)L.k36, sh = (z > 0 ? -q : 0.0) + (z < Lz - 1 ? q : 0.0);
+        double a = sh, b = -sh;
+#pragma unroll
+        for (int l = 0; l < 9; ++l) {
+          a += widen(w[l].x);
+          b += widen(w[l].y);
+        }
+        double* r = rho + 2 * (k * NS + L.site_off) + i;
+        r[0] = (double)rows[L.row_off + z].bgA + a;
+        r[N] = (double)rows[L.row_off + z].bgB + b;
+      }
+      shift_wall32(w, z > 0, z < Lz - 1, L.k9, L.k36);
+    } else if (rho) {
+      double a = 0, b = 0;
+#pragma unroll
+      for (int l = 0; l < 9; ++l) {
+        a += widen(w[l].x);
+        b += widen(w[l].y);
+      }
+      double* r = rho + 2 * (k * NS + L.site_off) + i;
+      r[0] = (double)rows[L.row_off + z].bgA + a;
+      r[N] = (double)rows[L.row_off + z].bgB + b;
+    }
+    dev[k * NS + L.site_off + i] =
+        make_float2((((w[0].x + w[1].x) + (w[2].x + w[3].x)) + ((w[4].x + w[5].x) + (w[6].x + w[7].x))) + w[8].x,
+                    (((w[0].y + w[1].y) + (w[2].y + w[3].y)) + ((w[4].y + w[5].y) + (w[6].y + w[7].y))) + w[8].y);
+  } else {
+    double* r = rho + 2 * (k * NS + L.site_off) + i;
+    r[0] = (((w[0].x + w[1].x) + (w[2].x + w[3].x)) + ((w[4].x + w[5].x) + (w[6].x + w[7].x))) + w[8].x;
+    r[N] = (((w[0].y + w[1].y) + (w[2].y + w[3].y)) + ((w[4].y + w[5].y) + (w[6].y + w[7].y))) + w[8].y;
+  }
+}
+
+// The mechanical pressure of one site (Sec. III.C), minus its row's background in FP32: the arithmetic
+// of site_update of the step kernels, in the state's precision.  d: the densities (FP32: deviations) as
+// pairs through at(row offset, column).
+template <class real, class P, class At>
+__device__ __forceinline__ real site_pressure(const P w[9], real G, const RowConst<real>& rc, At at, int Lx, int Lz,
+                                              int x, int z) {
+  real m3[2];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    auto v = [&](int l) { return s == 0 ? w[l].x : w[l].y; };
+    const real e = (v(1) + v(3)) + (v(2) + v(4)), dg = (v(5) + v(7)) + (v(6) + v(8));
+    m3[s] = fma(real(-2), v(0), fma(real(4), dg, e));
+  }
+  const int xm = x == 0 ? Lx - 1 : x - 1, xp = x + 1 == Lx ? 0 : x + 1;
+  const int r0 = z * Lx, ru = min(z + 1, Lz - 1) * Lx, rd = max(z - 1, 0) * Lx;
+  const P d = at(r0 + x), wv = at(r0 + xm), e = at(r0 + xp), n = at(ru + x), nw = at(ru + xm), ne = at(ru + xp),
+          s = at(rd + x), sw = at(rd + xm), se = at(rd + xp);
+  const real kin = (m3[0] + m3[1] + 2 * (d.x + d.y)) * (real(1) / 6);
+  const real c9 = real(1) / 9, c18 = real(2) / 36;
+  const real NA = fma(c9, (e.x + wv.x) + (n.x + s.x), c18 * ((ne.x + nw.x) + (se.x + sw.x)));
+  const real NB = fma(c9, (e.y + wv.y) + (n.y + s.y), c18 * ((ne.y + nw.y) + (se.y + sw.y)));
+  const real inter = d.x * (rc.nbB + NB) + rc.bgA * NB + d.y * (rc.nbA + NA) + rc.bgB * NA;
+  return kin + real(0.25) * G * inter;
+}
+
+// The pressure of the `gridDim.y` states at f, f + S, .. summed over each block's sites:
+// part[state][block].
+template <class real>
+__global__ void __launch_bounds__(kAdjBlock)
+    adj_pressure(const real* __restrict__ f, int64_t S, const LatticeDev<real>* lat, const RowConst<real>* rows,
+                 const AdjMap map, const double* __restrict__ rho, const float2* __restrict__ dev, int64_t NS,
+                 double* __restrict__ part) {
+  using P = typename PairOfState<real>::type;
+  const int li = adj_lattice(map);
+  const LatticeDev<real>& L = lat[li];
+  const int Lx = L.Lx, Lz = L.Lz, N = Lx * Lz, i = adj_site(map, li), k = blockIdx.y;
+  double p = 0;
+  if (i < N) {
+    const int z = i / Lx, x = i - z * Lx;
+    P w[9];
+    load_pairs<real>(f + k * S + L.f_off, Lx, Lz, x, z, w);
+    const RowConst<real>& rc = rows[L.row_off + z];
+    if constexpr (sizeof(real) == 4) {
+      if (z == 0 || z == Lz - 1) shift_wall32(w, z > 0, z < Lz - 1, L.k9, L.k36);
+      const float2* d = dev + k * NS + L.site_off;
+      p = (double)site_pressure<float>(w, L.G, rc, [&](int j) { return d[j]; }, Lx, Lz, x, z);
+    } else {
+      const double* d = rho + 2 * (k * NS + L.site_off);
+      p = site_pressure<double>(w, L.G, rc, [&](int j) { return make_double2(d[j], d[N + j]); }, Lx, Lz, x, z);
+    }
+  }
+  p = warp_sum(p);
+  if (threadIdx.x == 0) part[(int64_t)k * map.n_blocks + blockIdx.x] = p;
+}
+
+// out[state * n_lat + lattice]: the sums over the lattices' blocks, in a fixed order (one warp each).
+__global__ void adj_sum_pressure(const double* __restrict__ part, const AdjMap map, double* __restrict__ out) {
+  const int li = blockIdx.x, k = blockIdx.y, b1 = map.first[li + 1];
+  double a = 0;
+  for (int b = map.first[li] + threadIdx.x; b < b1; b += 32) a += part[(int64_t)k * map.n_blocks + b];
+  a = warp_sum(a);
+  if (threadIdx.x == 0) out[(int64_t)k * map.n_lat + li] = a;
 }
 
 template <class real, bool NOISE, bool UNIT>
@@ -733,13 +866,13 @@ __global__ void __launch_bounds__(kAdjBlock)
 }
 
 // Gather the forces' share of the neighbours, turn the moments' sensitivities into populations and push
-// them along the transposed streaming map; with f_next also the densities of the state before.  Two
-// threads per site, one per species, as adj_gather_push_kernel.
+// them along the transposed streaming map.  Two threads per site, one per species, as
+// adj_gather_push_kernel.
 template <class real, bool UNIT>
 __global__ void __launch_bounds__(2 * kAdjBlock)
-    adj_push_default(const LatticeDev<real>* lat, const RowConst<real>* rows, const AdjConst* __restrict__ kcs,
-                     const AdjMap map, const double* __restrict__ mom, const double* __restrict__ sb, double sign,
-                     double* __restrict__ fbar_prev, const real* __restrict__ f_next, double* __restrict__ rho_next) {
+    adj_push_default(const LatticeDev<real>* lat, const AdjConst* __restrict__ kcs, const AdjMap map,
+                     const double* __restrict__ mom, const double* __restrict__ sb, double sign,
+                     double* __restrict__ fbar_prev) {
   constexpr int NM = UNIT ? 3 : 9;
   const int li = adj_lattice(map);
   const LatticeDev<real>& L = lat[li];
@@ -750,26 +883,6 @@ __global__ void __launch_bounds__(2 * kAdjBlock)
   const int z = i / Lx, x = i - z * Lx;
   const int xm = x == 0 ? Lx - 1 : x - 1, xp = x + 1 == Lx ? 0 : x + 1;
   const bool wall = z == 0 || z == Lz - 1;
-  if (f_next) {  // this species' density of f_next at the site (interior rows: the shifts sum to zero)
-    const real* g = f_next + L.f_off;
-    double a = 0;
-#pragma unroll
-    for (int l = 0; l < 9; ++l) {
-      const int zs = z - LB_CZ(l), xs = LB_CX(l) == 0 ? x : (LB_CX(l) > 0 ? xm : xp);
-      const bool in = LB_CZ(l) == 0 || (zs >= 0 && zs < Lz);
-      a += widen(g[2 * (in ? l * N + zs * Lx + xs : LB_OPP(l) * N + z * Lx + x) + sp]);
-    }
-    if (sizeof(real) == 4) {
-      const RowConst<real>& rc = rows[L.row_off + z];
-      a += (double)(sp == 0 ? rc.bgA : rc.bgB);
-      if (wall) {  // link 2 (or 4), and 5, 6 (or 7, 8), carry their shift
-        const double q = (double)L.k9 + 2 * (double)L.k36;
-        if (z > 0) a += sp == 0 ? -q : q;
-        if (z < Lz - 1) a += sp == 0 ? q : -q;
-      }
-    }
-    rho_next[2 * so + (int64_t)sp * N + i] = a;
-  }
   const double* sx = sb + 8 * so + (int64_t)(4 * sp) * N;
   const double *sz = sx + N, *s5 = sz + N, *s6 = s5 + N;  // x + z, z - x
   double rb;
@@ -826,8 +939,7 @@ __global__ void __launch_bounds__(2 * kAdjBlock)
   }
 }
 
-// grads[3 i + p] = sum over the sites of lattice i of its parameter shares [3][N]: block (i, p), threads
-// strided over the sites, then a fixed tree (deterministic).
+// grads[3 i + p] = sum over the sites of lattice i of its shares [3][N]: block (i, p), threads strided over the sites, then a fixed tree (deterministic).
 template <class real>
 __global__ void __launch_bounds__(1024) adj_sum_shares(const double* shares, const LatticeDev<real>* lat, double* grads) {
   const LatticeDev<real>& L = lat[blockIdx.x];
@@ -873,51 +985,89 @@ __global__ void adj_sum_partials(const double* partials, const AdjMap map, doubl
 template <class real>
 cudaError_t launch_adjoint_step(const real* f_prev, const real* f_next, const double* fbar, double* fbar_prev,
                                 const LatticeDev<real>* lat, const RowConst<real>* rows, const AdjConst* kcs,
-                                bool options, bool unit, const AdjMap& map, uint32_t step, bool noise, double sign,
-                                bool rho_ready, double* rho, double* rho_next, double* fl, double* sb,
-                                double* partials, const NormalTables* tab, cudaStream_t s) {
+                                const AdjMap& map, uint32_t step, bool noise, double sign, bool rho_ready, double* rho,
+                                double* rho_next, double* fl, double* sb, double* partials, const NormalTables* tab,
+                                cudaStream_t s) {
   const int nb = map.n_blocks;
   if (!rho_ready) adj_rho_kernel<real><<<nb, kAdjBlock, 0, s>>>(f_prev, lat, rows, map, rho);
-  using T = std::true_type;
-  using F = std::false_type;
-  if (options) {
-    auto local = [&](auto noise_c) {
-      adj_local_kernel<real, decltype(noise_c)::value>
-          <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, rows, kcs, map, rho, step, sign, fl, sb, partials, tab);
-    };
-    noise ? local(T()) : local(F());
-    adj_gather_push_kernel<real>
-        <<<nb, 2 * kAdjBlock, 0, s>>>(lat, rows, kcs, map, rho, fl, sb, sign, fbar_prev, f_next, rho_next);
-    return cudaGetLastError();
-  }
+  if (noise)
+    adj_local_kernel<real, true>
+        <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, rows, kcs, map, rho, step, sign, fl, sb, partials, tab);
+  else
+    adj_local_kernel<real, false>
+        <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, rows, kcs, map, rho, step, sign, fl, sb, partials, tab);
+  adj_gather_push_kernel<real>
+      <<<nb, 2 * kAdjBlock, 0, s>>>(lat, rows, kcs, map, rho, fl, sb, sign, fbar_prev, f_next, rho_next);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_adjoint_gradient(const double* partials, const AdjMap& map, double* grads, cudaStream_t s) {
+  adj_sum_partials<<<map.n_lat, 32, 0, s>>>(partials, map, grads);
+  return cudaGetLastError();
+}
+
+template <class real>
+cudaError_t launch_adjoint_densities(const real* f, int64_t S, int n_states, const LatticeDev<real>* lat,
+                                     const RowConst<real>* rows, const AdjMap& map, double* rho, float* dev, int64_t NS,
+                                     cudaStream_t s) {
+  adj_density_default<real><<<dim3(map.n_blocks, n_states), kAdjBlock, 0, s>>>(f, S, lat, rows, map, rho,
+                                                                               reinterpret_cast<float2*>(dev), NS);
+  return cudaGetLastError();
+}
+
+template <class real>
+cudaError_t launch_adjoint_pressures(const real* f, int64_t S, int n_states, const LatticeDev<real>* lat,
+                                     const RowConst<real>* rows, const AdjMap& map, const double* rho, const float* dev,
+                                     int64_t NS, double* part, double* out, cudaStream_t s) {
+  adj_pressure<real><<<dim3(map.n_blocks, n_states), kAdjBlock, 0, s>>>(
+      f, S, lat, rows, map, rho, reinterpret_cast<const float2*>(dev), NS, part);
+  adj_sum_pressure<<<dim3(map.n_lat, n_states), 32, 0, s>>>(part, map, out);
+  return cudaGetLastError();
+}
+
+template <class real>
+cudaError_t launch_adjoint_step_default(const real* f_prev, const double* fbar, double* fbar_prev,
+                                        const LatticeDev<real>* lat, const AdjConst* kcs, bool unit, const AdjMap& map,
+                                        uint32_t step, bool noise, double sign, const double* rho, double* mom, double* sb,
+                                        double* shares, const NormalTables* tab, cudaStream_t s) {
+  const int nb = map.n_blocks;
   auto pair = [&](auto noise_c, auto unit_c) {
     constexpr bool U = decltype(unit_c)::value;
     adj_local_default<real, decltype(noise_c)::value, U>
-        <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, kcs, map, rho, step, sign, fl, sb, partials, tab);
-    adj_push_default<real, U>
-        <<<nb, 2 * kAdjBlock, 0, s>>>(lat, rows, kcs, map, fl, sb, sign, fbar_prev, f_next, rho_next);
+        <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, kcs, map, rho, step, sign, mom, sb, shares, tab);
+    adj_push_default<real, U><<<nb, 2 * kAdjBlock, 0, s>>>(lat, kcs, map, mom, sb, sign, fbar_prev);
   };
+  using T = std::true_type;
+  using F = std::false_type;
   if (noise) unit ? pair(T(), T()) : pair(T(), F());
   else unit ? pair(F(), T()) : pair(F(), F());
   return cudaGetLastError();
 }
 
 template <class real>
-cudaError_t launch_adjoint_gradient(const double* partials, const LatticeDev<real>* lat, bool options,
-                                    const AdjMap& map, double* grads, cudaStream_t s) {
-  if (options) adj_sum_partials<<<map.n_lat, 32, 0, s>>>(partials, map, grads);
-  else adj_sum_shares<real><<<dim3(map.n_lat, 3), 1024, 0, s>>>(partials, lat, grads);
+cudaError_t launch_adjoint_gradient_default(const double* shares, const LatticeDev<real>* lat, int n_lat, double* grads,
+                                            cudaStream_t s) {
+  adj_sum_shares<real><<<dim3(n_lat, 3), 1024, 0, s>>>(shares, lat, grads);
   return cudaGetLastError();
 }
 
 #define LB_ADJ_INST(real)                                                                                             \
   template cudaError_t launch_adjoint_step<real>(const real*, const real*, const double*, double*,                    \
                                                  const LatticeDev<real>*, const RowConst<real>*, const AdjConst*,     \
-                                                 bool, bool, const AdjMap&, uint32_t, bool, double, bool, double*,    \
-                                                 double*, double*, double*, double*, const NormalTables*,             \
-                                                 cudaStream_t);                                                       \
-  template cudaError_t launch_adjoint_gradient<real>(const double*, const LatticeDev<real>*, bool, const AdjMap&,     \
-                                                     double*, cudaStream_t);
+                                                 const AdjMap&, uint32_t, bool, double, bool, double*, double*,       \
+                                                 double*, double*, double*, const NormalTables*, cudaStream_t);       \
+  template cudaError_t launch_adjoint_densities<real>(const real*, int64_t, int, const LatticeDev<real>*,             \
+                                                      const RowConst<real>*, const AdjMap&, double*, float*, int64_t, \
+                                                      cudaStream_t);                                                  \
+  template cudaError_t launch_adjoint_pressures<real>(const real*, int64_t, int, const LatticeDev<real>*,             \
+                                                      const RowConst<real>*, const AdjMap&, const double*,            \
+                                                      const float*, int64_t, double*, double*, cudaStream_t);         \
+  template cudaError_t launch_adjoint_step_default<real>(const real*, const double*, double*, const LatticeDev<real>*, \
+                                                         const AdjConst*, bool, const AdjMap&, uint32_t, bool, double, \
+                                                         const double*, double*, double*, double*,                    \
+                                                         const NormalTables*, cudaStream_t);                          \
+  template cudaError_t launch_adjoint_gradient_default<real>(const double*, const LatticeDev<real>*, int, double*,    \
+                                                             cudaStream_t);
 LB_ADJ_INST(float)
 LB_ADJ_INST(double)
 

@@ -75,17 +75,38 @@ struct AdjMap {
 // go to rho_next for the next step.  kcs: the lattices' AdjConst (device); options: any lattice
 // uses a non-default option of the step; sign: +1 for the noisy run, -1 for the noiseless one
 // (the loss weight of a site is sign w_loss).  The sensitivities are double precision for either
-// state precision.  Without options the parameter shares are kept per site instead, 3 doubles at
-// 3 site_off ([3][N] per lattice), and sb takes 8 doubles per site; unit: every lattice's rates of
-// moments 3..8 are 1.
+// state precision.
 template <class real>
 cudaError_t launch_adjoint_step(const real* f_prev, const real* f_next, const double* fbar, double* fbar_prev,
                                 const LatticeDev<real>* lat, const RowConst<real>* rows, const AdjConst* kcs,
-                                bool options, bool unit, const AdjMap& map, uint32_t step, bool noise, double sign,
-                                bool rho_ready, double* rho, double* rho_next, double* fl, double* sb,
-                                double* partials, const NormalTables* tab, cudaStream_t s);
+                                const AdjMap& map, uint32_t step, bool noise, double sign, bool rho_ready, double* rho,
+                                double* rho_next, double* fl, double* sb, double* partials, const NormalTables* tab,
+                                cudaStream_t s);
+cudaError_t launch_adjoint_gradient(const double* partials, const AdjMap& map, double* grads, cudaStream_t s);
+
+// The same for lattices of the default options (AdjConst::options false for all), whose densities and
+// pressures come for all states of a segment at once.  n_states states at f, f + S, ..; NS: sites of the
+// batch.  rho: [2][N] per lattice at 2 site_off, 2 NS doubles per state (FP32 states may pass null); dev:
+// FP32 states only, the density deviations as the step kernels sum them, 2 NS floats per state.
 template <class real>
-cudaError_t launch_adjoint_gradient(const double* partials, const LatticeDev<real>* lat, bool options,
-                                    const AdjMap& map, double* grads, cudaStream_t s);
+cudaError_t launch_adjoint_densities(const real* f, int64_t S, int n_states, const LatticeDev<real>* lat,
+                                     const RowConst<real>* rows, const AdjMap& map, double* rho, float* dev, int64_t NS,
+                                     cudaStream_t s);
+// out[state * n_lat + lattice]: the pressure summed over the lattice's sites (minus the background in
+// FP32); part: n_blocks doubles per state.
+template <class real>
+cudaError_t launch_adjoint_pressures(const real* f, int64_t S, int n_states, const LatticeDev<real>* lat,
+                                     const RowConst<real>* rows, const AdjMap& map, const double* rho, const float* dev,
+                                     int64_t NS, double* part, double* out, cudaStream_t s);
+// Buffers per site: mom up to 18 doubles, sb 8, shares 3 ([3][N] per lattice at 3 site_off, zeroed before
+// the sweep).  rho: the densities of f_prev.  unit: every lattice's rates of moments 3..8 are 1.
+template <class real>
+cudaError_t launch_adjoint_step_default(const real* f_prev, const double* fbar, double* fbar_prev,
+                                        const LatticeDev<real>* lat, const AdjConst* kcs, bool unit, const AdjMap& map,
+                                        uint32_t step, bool noise, double sign, const double* rho, double* mom, double* sb,
+                                        double* shares, const NormalTables* tab, cudaStream_t s);
+template <class real>
+cudaError_t launch_adjoint_gradient_default(const double* shares, const LatticeDev<real>* lat, int n_lat, double* grads,
+                                            cudaStream_t s);
 
 }  // namespace lbk

@@ -1083,6 +1083,8 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
     size_t S = 0, NS = 0;  // reals per state; sites of the batch
     real *ck = nullptr, *ring = nullptr, *cur = nullptr, *fields = nullptr, *pfield = nullptr;
     double *fb = nullptr, *rho = nullptr, *fl = nullptr, *sb = nullptr, *partials = nullptr, *gpart = nullptr;
+    double* psum = nullptr;  // pressure sums of every step and lattice
+    float* dev = nullptr;
     DiagStats* stats = nullptr;
     AdjConst* kcs = nullptr;
     int* map_buf = nullptr;
@@ -1148,6 +1150,17 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
       R.unit = R.unit && R.hkcs[i].unit;
     }
   }
+  // Default options: no step is sampled.  The forward run makes the checkpoints by persistent launches
+  // of C plain steps and stops at the last of them; a segment's states come from another such launch,
+  // and their densities and pressures from one launch each for all of them.  The loss alone takes
+  // segments of up to 32 states (1 GB of them at most) and no checkpoints.  The pressures are summed per
+  // step, in one order, so the loss does not depend on the segments.  Other options, and runs whose
+  // pressures per step would take over 512 MB, go step by step with the pressure of every step sampled.
+  // 256 x 128, 500 steps, FP64:
+  // the gradient 52 -> 42 ms, the loss alone 22 -> 16 ms; eight lattices from FP32 state, 300 steps: 83 -> 76 ms.
+  const bool fused = !runs[0].options && T * n <= ((int64_t)1 << 26);
+  const int64_t loss_len = std::max<int64_t>(1, std::min<int64_t>(32, ((int64_t)1 << 30) / (int64_t)(c->n_f * sizeof(real))));
+  const int64_t seg_len = want_grad ? C : std::min(T, loss_len), nseg = (T + seg_len - 1) / seg_len;
   for (int pass = 0; pass < 2; ++pass) {
     if (pass == 1) {
       arena = (char*)ctx_malloc(c, bytes);
@@ -1159,20 +1172,28 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
     }
     for (Run& R : runs) {
       const int nblk = R.first[n];
-      R.ck = (real*)piece(nck * R.S, sizeof(real));
-      R.cur = (real*)piece(2 * R.S, sizeof(real));
-      R.fields = (real*)piece(4 * R.NS, sizeof(real));
-      R.pfield = (real*)piece(R.NS, sizeof(real));
-      R.partials = (double*)piece(3 * R.x->items.size(), sizeof(double));
-      R.stats = (DiagStats*)piece(n, sizeof(DiagStats));
+      if (want_grad || !fused) R.ck = (real*)piece(nck * R.S, sizeof(real));
+      if (want_grad || !fused) R.cur = (real*)piece(2 * R.S, sizeof(real));
+      if (!fused) {
+        R.fields = (real*)piece(4 * R.NS, sizeof(real));
+        R.pfield = (real*)piece(R.NS, sizeof(real));
+        R.partials = (double*)piece(3 * R.x->items.size(), sizeof(double));
+        R.stats = (DiagStats*)piece(n, sizeof(DiagStats));
+      } else {
+        R.partials = (double*)piece((size_t)std::min<int64_t>(seg_len, 16384) * nblk, sizeof(double));
+        R.psum = (double*)piece((size_t)T * n, sizeof(double));
+        if (c->dev32) R.dev = (float*)piece((size_t)seg_len * 2 * R.NS, sizeof(float));
+      }
+      // the states of a segment; the loss alone also makes the next one's first there
+      if (want_grad || fused) R.ring = (real*)piece((size_t)(seg_len + (want_grad ? 0 : 1)) * R.S, sizeof(real));
+      // densities: of every state of the segment, or two sets
+      if (want_grad || (fused && !c->dev32)) R.rho = (double*)piece((fused ? 2 * seg_len : 4) * R.NS, sizeof(double));
+      if (want_grad || fused) R.map_buf = (int*)piece((size_t)nblk + n + 1, sizeof(int));
       if (want_grad) {
-        R.ring = (real*)piece(C * R.S, sizeof(real));
         R.fb = (double*)piece(2 * R.S, sizeof(double));
-        R.rho = (double*)piece(4 * R.NS, sizeof(double));  // two density sets
         R.fl = (double*)piece(R.S, sizeof(double));
-        R.sb = (double*)piece(8 * R.NS, sizeof(double));
-        R.gpart = (double*)piece(3 * (R.options ? (size_t)nblk : R.NS), sizeof(double));
-        R.map_buf = (int*)piece((size_t)nblk + n + 1, sizeof(int));
+        R.sb = (double*)piece((fused ? 8 : 4) * R.NS, sizeof(double));
+        R.gpart = (double*)piece(fused ? 3 * R.NS : 3 * (size_t)nblk, sizeof(double));
         R.kcs = (AdjConst*)piece(n, sizeof(AdjConst));
       }
     }
@@ -1183,14 +1204,15 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
   auto ok = [&](cudaError_t r) {
     if (e == cudaSuccess && r != cudaSuccess) e = r;
   };
-  if (want_grad)
-    for (Run& R : runs) {
-      const int nblk = R.first[n];
+  for (Run& R : runs) {
+    const int nblk = R.first[n];
+    if (want_grad || fused) {
       ok(cudaMemcpy(R.map_buf, R.lat_of.data(), (size_t)nblk * sizeof(int), cudaMemcpyHostToDevice));
       ok(cudaMemcpy(R.map_buf + nblk, R.first.data(), (size_t)(n + 1) * sizeof(int), cudaMemcpyHostToDevice));
-      ok(cudaMemcpy(R.kcs, R.hkcs.data(), (size_t)n * sizeof(AdjConst), cudaMemcpyHostToDevice));
       R.map = AdjMap{R.map_buf, R.map_buf + nblk, nblk, n};
     }
+    if (want_grad) ok(cudaMemcpy(R.kcs, R.hkcs.data(), (size_t)n * sizeof(AdjConst), cudaMemcpyHostToDevice));
+  }
   ok(cudaMemsetAsync(zero_t, 0, sizeof(int64_t), st));
   ok(cudaMemsetAsync(d_grad, 0, (size_t)6 * n * sizeof(double), st));
   ok(cudaEventRecord(ev[0], st));  // the second run's stream starts after the set-up
@@ -1208,28 +1230,85 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
     a.err = c->d_err;
     return a;
   };
-  // forward runs from rest, step by step in both streams: checkpoints f*_{c-1} before every C-th
-  // step, pressure of every step
+  // nsteps plain steps of a run from step k on: between two buffers in turn, or (ring) each into the
+  // next state of the ring
+  auto plain_steps = [&](Run& R, real* src, real* dst, int64_t k, int64_t nsteps, bool ring) {
+    if (nsteps <= 0) return;
+    lb_ctx* x = R.x;
+    if (x->coop_grid < 0) x->coop_grid = persistent_grid<real>(x->tile_x, R.noise, x->bulk_ok);
+    const int grid = std::min<int>(x->coop_grid, (int)x->items.size());
+    if (grid > 0) {
+      ok(cudaMemsetAsync(x->d_barrier, 0, sizeof(unsigned long long), R.s));
+      ok(cudaMemsetAsync(x->d_done, 0, x->items.size() * sizeof(unsigned), R.s));
+      const PersistArgs pa{reinterpret_cast<unsigned long long*>(x->d_barrier), x->d_done, x->d_nbr_off, x->d_nbr,
+                           c->d_err, 2000, owner_mode(x, grid), 0, ring ? (int64_t)R.S : 0};
+      ok(launch_step_persistent<real>(args(R, src, dst, k), x->tile_x, (int)nsteps, R.noise, x->bulk_ok, pa, grid, R.s));
+      return;
+    }
+    for (int64_t i = 0; i < nsteps; ++i) {
+      real* from = ring ? src + i * R.S : ((i & 1) ? dst : src);
+      real* to = ring ? dst + i * R.S : ((i & 1) ? src : dst);
+      ok(launch_step<real>(args(R, from, to, k + i), x->tile_x, false, R.noise, x->bulk_ok, R.s));
+    }
+  };
+  auto copy_state = [&](Run& R, real* to, const real* from) {
+    ok(cudaMemcpyAsync(to, from, R.S * sizeof(real), cudaMemcpyDeviceToDevice, R.s));
+  };
+  // the densities and pressures of the len states in the ring, steps t0 ..
+  auto segment_fields = [&](Run& R, int64_t t0, int64_t len) {
+    const auto* lat = (const LatticeDev<real>*)R.x->d_lat;
+    const auto* rows = (const RowConst<real>*)R.x->d_rows;
+    constexpr int64_t kMost = 16384;  // states per launch (a grid's second dimension ends at 65535)
+    for (int64_t i = 0; i < len; i += kMost) {
+      const int m = (int)std::min(kMost, len - i);
+      const real* f = R.ring + i * R.S;
+      double* rho = R.rho ? R.rho + i * 2 * R.NS : nullptr;
+      float* dev = R.dev ? R.dev + i * 2 * R.NS : nullptr;
+      ok(launch_adjoint_densities<real>(f, R.S, m, lat, rows, R.map, rho, dev, R.NS, R.s));
+      ok(launch_adjoint_pressures<real>(f, R.S, m, lat, rows, R.map, rho, dev, R.NS, R.partials, R.psum + (t0 + i) * n,
+                                        R.s));
+    }
+  };
+  // forward runs from rest in both streams: checkpoints f*_{c-1} before every C-th step, the pressure of
+  // every step
   {
     NvtxRange rr("lb adjoint: forward runs");
     for (Run& R : runs) {
-      if (want_grad) ok(cudaMemsetAsync(R.gpart, 0, 3 * (R.options ? (size_t)R.map.n_blocks : R.NS) * sizeof(double), R.s));
+      if (want_grad) ok(cudaMemsetAsync(R.gpart, 0, 3 * (fused ? R.NS : (size_t)R.map.n_blocks) * sizeof(double), R.s));
       for (int i = 0; i < n; ++i) {
         const lb_params& p = R.x->params[i];
         const BgParams bp{p.Lx, p.Lz, c->dev32 ? 1 : 0, kRhoBar, p.grad_c0};
-        ok(launch_init_rest<real>(R.cur + R.x->f_off[i], bp, R.s));
+        ok(launch_init_rest<real>((fused && !want_grad ? R.ring : R.cur) + R.x->f_off[i], bp, R.s));
       }
-      ok(cudaMemsetAsync(R.stats, 0, (size_t)n * sizeof(DiagStats), R.s));
+      if (!fused) ok(cudaMemsetAsync(R.stats, 0, (size_t)n * sizeof(DiagStats), R.s));
     }
-    for (int64_t k = 0; k < T && e == cudaSuccess; ++k)
-      for (Run& R : runs) {
-        real* src = R.cur + (k & 1) * R.S;
-        real* dst = R.cur + ((k + 1) & 1) * R.S;
-        if (k % C == 0)
-          ok(cudaMemcpyAsync(R.ck + (k / C) * R.S, src, R.S * sizeof(real), cudaMemcpyDeviceToDevice, R.s));
-        ok(launch_step<real>(args(R, src, dst, k), R.x->tile_x, true, R.noise, R.x->bulk_ok, R.s));
-        ok(launch_finalize(R.x->d_diag, n, R.partials, R.stats, R.s));
-      }
+    if (fused && want_grad) {
+      for (Run& R : runs) copy_state(R, R.ck, R.cur);
+      for (int64_t seg = 0; seg + 1 < nck && e == cudaSuccess; ++seg)
+        for (Run& R : runs) {
+          // the segment's first state lies in buffer (seg C) mod 2
+          real* b[2] = {R.cur + ((seg * C) & 1) * R.S, R.cur + ((seg * C + 1) & 1) * R.S};
+          plain_steps(R, b[0], b[1], seg * C, C, false);
+          copy_state(R, R.ck + (seg + 1) * R.S, b[C & 1]);
+        }
+    } else if (fused) {
+      for (int64_t seg = 0; seg < nseg && e == cudaSuccess; ++seg)
+        for (Run& R : runs) {
+          const int64_t t0 = seg * seg_len, len = std::min(seg_len, T - t0);
+          if (seg > 0) copy_state(R, R.ring, R.ring + seg_len * R.S);
+          plain_steps(R, R.ring, R.ring + R.S, t0, seg + 1 < nseg ? len : len - 1, true);
+          segment_fields(R, t0, len);
+        }
+    } else {
+      for (int64_t k = 0; k < T && e == cudaSuccess; ++k)
+        for (Run& R : runs) {
+          real* src = R.cur + (k & 1) * R.S;
+          real* dst = R.cur + ((k + 1) & 1) * R.S;
+          if (k % C == 0) copy_state(R, R.ck + (k / C) * R.S, src);
+          ok(launch_step<real>(args(R, src, dst, k), R.x->tile_x, true, R.noise, R.x->bulk_ok, R.s));
+          ok(launch_finalize(R.x->d_diag, n, R.partials, R.stats, R.s));
+        }
+    }
   }
   // reverse sweeps, one checkpoint segment at a time in both streams; a run's sign (+ noisy,
   // - noiseless) enters through the loss weight alpha = sign / (T N) of each lattice, to which the
@@ -1239,51 +1318,86 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
     for (Run& R : runs) ok(cudaMemsetAsync(R.fb, 0, R.S * sizeof(double), R.s));
     for (int64_t seg = nck - 1; seg >= 0 && e == cudaSuccess; --seg) {
       const int64_t c0 = seg * C, len = std::min<int64_t>(C, T - c0);
-      for (Run& R : runs)
-        ok(cudaMemcpyAsync(R.ring, R.ck + seg * R.S, R.S * sizeof(real), cudaMemcpyDeviceToDevice, R.s));
-      for (int64_t i = 1; i < len; ++i)
-        for (Run& R : runs)
-          ok(launch_step<real>(args(R, R.ring + (i - 1) * R.S, R.ring + i * R.S, c0 + i - 1), R.x->tile_x, false,
-                               R.noise, R.x->bulk_ok, R.s));
-      // the densities of each step's state come with the previous step's gather (within a
-      // segment; at its top they are computed on their own)
+      for (Run& R : runs) {
+        copy_state(R, R.ring, R.ck + seg * R.S);
+        plain_steps(R, R.ring, R.ring + R.S, c0, len - 1, true);
+        if (fused) segment_fields(R, c0, len);
+      }
+      // without `fused` the densities of each step's state come with the previous step's gather (within
+      // a segment; at its top they are computed on their own)
       int rcur = 0;
       for (int64_t k = c0 + len - 1; k >= c0 && e == cudaSuccess; --k) {
         for (Run& R : runs) {
-          double* rho_k = R.rho + (size_t)rcur * 2 * R.NS;
-          double* rho_n = R.rho + (size_t)(1 - rcur) * 2 * R.NS;
-          ok(launch_adjoint_step<real>(R.ring + (k - c0) * R.S, k > c0 ? R.ring + (k - 1 - c0) * R.S : nullptr,
-                                       R.fb + R.fcur * R.S, R.fb + (1 - R.fcur) * R.S,
-                                       (const LatticeDev<real>*)R.x->d_lat, (const RowConst<real>*)R.x->d_rows, R.kcs,
-                                       R.options, R.unit, R.map, (uint32_t)k, R.noise != NOISE_OFF, R.sign, k < c0 + len - 1,
-                                       rho_k, rho_n, R.fl, R.sb, R.gpart, c->normals, R.s));
+          const real *f_prev = R.ring + (k - c0) * R.S, *f_next = k > c0 ? R.ring + (k - 1 - c0) * R.S : nullptr;
+          double *fb = R.fb + R.fcur * R.S, *fb_prev = R.fb + (1 - R.fcur) * R.S;
+          const auto* lat = (const LatticeDev<real>*)R.x->d_lat;
+          const auto* rows = (const RowConst<real>*)R.x->d_rows;
+          const bool noise = R.noise != NOISE_OFF;
+          if (fused) {
+            ok(launch_adjoint_step_default<real>(f_prev, fb, fb_prev, lat, R.kcs, R.unit, R.map, (uint32_t)k, noise,
+                                                 R.sign, R.rho + (k - c0) * 2 * R.NS, R.fl, R.sb, R.gpart, c->normals,
+                                                 R.s));
+          } else {
+            double* rho_k = R.rho + (size_t)rcur * 2 * R.NS;
+            double* rho_n = R.rho + (size_t)(1 - rcur) * 2 * R.NS;
+            ok(launch_adjoint_step<real>(f_prev, f_next, fb, fb_prev, lat, rows, R.kcs, R.map, (uint32_t)k, noise,
+                                         R.sign, k < c0 + len - 1, rho_k, rho_n, R.fl, R.sb, R.gpart, c->normals, R.s));
+          }
           R.fcur = 1 - R.fcur;
         }
         rcur = 1 - rcur;
       }
     }
-    for (int q = 0; q < 2 && e == cudaSuccess; ++q)
-      ok(launch_adjoint_gradient<real>(runs[q].gpart, (const LatticeDev<real>*)runs[q].x->d_lat, runs[q].options,
-                                       runs[q].map, d_grad + (size_t)3 * n * q, runs[q].s));
+    for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+      double* out = d_grad + (size_t)3 * n * q;
+      if (fused)
+        ok(launch_adjoint_gradient_default<real>(runs[q].gpart, (const LatticeDev<real>*)runs[q].x->d_lat, n, out,
+                                                 runs[q].s));
+      else ok(launch_adjoint_gradient(runs[q].gpart, runs[q].map, out, runs[q].s));
+    }
   }
   // join the second stream, then read the results
   ok(cudaEventRecord(ev[1], s1));
   ok(cudaStreamWaitEvent(st, ev[1], 0));
   std::vector<DiagStats> hs(2 * (size_t)n);
-  std::vector<double> hg(6 * (size_t)n, 0.0);
-  ok(cudaMemcpyAsync(hs.data(), runs[0].stats, (size_t)n * sizeof(DiagStats), cudaMemcpyDeviceToHost, st));
-  ok(cudaMemcpyAsync(hs.data() + n, runs[1].stats, (size_t)n * sizeof(DiagStats), cudaMemcpyDeviceToHost, st));
+  std::vector<double> hg(6 * (size_t)n, 0.0), hp[2];
+  for (int q = 0; q < 2; ++q) {
+    if (fused) {
+      hp[q].resize((size_t)T * n);
+      ok(cudaMemcpyAsync(hp[q].data(), runs[q].psum, hp[q].size() * sizeof(double), cudaMemcpyDeviceToHost, st));
+    } else {
+      ok(cudaMemcpyAsync(hs.data() + (size_t)q * n, runs[q].stats, (size_t)n * sizeof(DiagStats), cudaMemcpyDeviceToHost,
+                         st));
+    }
+  }
   if (want_grad) ok(cudaMemcpyAsync(hg.data(), d_grad, hg.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   ok(cudaStreamSynchronize(st));
+  // time averages of the mean pressure, per run and lattice (compensated sums over the steps)
+  std::vector<double> mean(2 * (size_t)n);
+  bool nonfinite = false;
+  for (int q = 0; q < 2; ++q)
+    for (int i = 0; i < n; ++i) {
+      double sum = hs[(size_t)q * n + i].P_sum, comp = hs[(size_t)q * n + i].P_comp;
+      if (fused) {
+        const DiagLattice& d = runs[q].x->diag[i];
+        sum = comp = 0.0;
+        for (int64_t t = 0; t < T; ++t) {
+          const double v = d.P_bg_mean + hp[q][(size_t)t * n + i] / d.n_sites, r = sum + v;
+          comp += std::fabs(sum) >= std::fabs(v) ? (sum - r) + v : (v - r) + sum;
+          sum = r;
+        }
+        nonfinite = nonfinite || !std::isfinite(sum);
+      } else {
+        nonfinite = nonfinite || hs[(size_t)q * n + i].nonfinite != 0;
+      }
+      mean[(size_t)q * n + i] = (sum + comp) / (double)T;
+    }
   release();
   if (e != cudaSuccess) return cuda_err(e);
-  for (const DiagStats& x : hs)
-    if (x.nonfinite) return LB_ERR_NONFINITE;
+  if (nonfinite) return LB_ERR_NONFINITE;
   for (int i = 0; i < n; ++i) {
     const bool same = c->params[i].kT == 0.0;  // both runs are the same run: the shift is exactly zero
-    if (losses)
-      losses[i] = same ? 0.0
-                       : (hs[i].P_sum + hs[i].P_comp) / (double)T - (hs[n + i].P_sum + hs[n + i].P_comp) / (double)T;
+    if (losses) losses[i] = same ? 0.0 : mean[i] - mean[(size_t)n + i];
     if (want_grad)
       for (int k = 0; k < 3; ++k)
         grads[3 * i + k] = same ? 0.0 : hg[3 * i + k] + hg[(size_t)3 * n + 3 * i + k];

@@ -1209,9 +1209,9 @@ __global__ void __launch_bounds__(256, MinBlocks<real>::value)
   for (unsigned long long t; (t = next_ticket(p, (unsigned)n, first)) < total; first = false) {
     const int k = (int)(t / n), i = (int)(t - (unsigned long long)k * n);
     auto ready = [&] { return k == 0 || wait_items(p, i, (unsigned)k); };
-    const bool odd = (k & 1) && !p.trial;
-    const real* src = odd ? a.dst : a.src;
-    real* dst = odd ? const_cast<real*>(a.src) : a.dst;
+    const bool odd = (k & 1) && !p.trial && !p.ring;
+    const real* src = odd ? a.dst : a.src + k * p.ring;
+    real* dst = odd ? const_cast<real*>(a.src) : a.dst + k * p.ring;
     if (!process_item<real, false, NOISE>(a, src, dst, i, (uint32_t)(t0 + k), smem, k > 0 && p.owner, ready)) return;
     publish_item(p.done, i, (unsigned)(k + 1));
   }
@@ -1229,9 +1229,9 @@ __global__ void __launch_bounds__(TX, PersistentBlocks<real>::value * 128 / TX)
   for (unsigned long long t; (t = next_ticket(p, (unsigned)n, first)) < total; first = false) {
     const int k = (int)(t / n), i = (int)(t - (unsigned long long)k * n);
     auto ready = [&] { return k == 0 || wait_items(p, i, (unsigned)k); };
-    const bool odd = (k & 1) && !p.trial;
-    const real* src = odd ? a.dst : a.src;
-    real* dst = odd ? const_cast<real*>(a.src) : a.dst;
+    const bool odd = (k & 1) && !p.trial && !p.ring;
+    const real* src = odd ? a.dst : a.src + k * p.ring;
+    real* dst = odd ? const_cast<real*>(a.src) : a.dst + k * p.ring;
     if (!process_item_bulk<real, TX, false, NOISE>(a, src, dst, i, (uint32_t)(t0 + k), smem, ph,
                                                    a.src_buf ^ (odd ? 1 : 0), k > 0 && p.owner, ready))
       return;  // the blocks that wait on this item give up (bounded)

@@ -28,3 +28,15 @@ def test_rates_and_short_lattices(rates, prec, gtol):
                                                G=p.G, grad_c0=p.grad_c0, seed=p.seed, lattice_id=p.lattice_id)
         np.testing.assert_allclose(g, o_g, rtol=0, atol=gtol * np.max(np.abs(o_g)))
         assert abs(loss - want) <= (1e-10 if prec == "fp64" else 1e-4) * abs(want)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "dev32"])
+def test_loss_does_not_depend_on_segments_or_mode(prec):
+    """The pressures are summed step by step in one order: the loss alone (segments of 32 states), and with
+    the gradient in segments of 1, 7 and 40 states, is the same number."""
+    ps = [LatticeParams(34, 10, kT=1e-3, G=0.5, grad_c0=0.02, seed=2), LatticeParams(16, 6, kT=1e-4, G=0.3, seed=4, lattice_id=1)]
+    with Simulation(ps, precision=prec) as sim:
+        want, _ = sim.pressure_shift_gradients(40, 40, want_grad=False)
+        for ckpt in (1, 7, 40):
+            losses, _ = sim.pressure_shift_gradients(40, ckpt)
+            assert np.array_equal(losses, want)
