@@ -105,6 +105,7 @@ struct lb_ctx {
   int sf_threads = 256, sf_cap = 4096;  // sample-step transforms (sf_threads, SfPlan)
   size_t sf_smem_rows = 0, sf_smem_cols = 0;
   int64_t* d_t = nullptr;
+  bool device_t = false;  // the launches being enqueued go into a graph: they count steps on the device
   unsigned* d_barrier = nullptr;  // the persistent launch's ticket counter (64-bit)
   unsigned* d_done = nullptr;     // persistent launch: steps completed per item
   int* d_nbr_off = nullptr;       // persistent launch: dependency lists of the items (CSR)
@@ -591,8 +592,9 @@ bool is_sample(const lb_ctx* c, int64_t t) {
   return c->every > 0 && t >= c->discard && (t - c->discard) % c->every == 0;
 }
 
+// k: the step counted from c->t (device_t: from the device's counter); t_store: StepArgs.
 template <class real>
-StepArgs<real> step_args(lb_ctx* c, int cur, int t_offset) {
+StepArgs<real> step_args(lb_ctx* c, int cur, int64_t k, int64_t t_store = -1) {
   StepArgs<real> a;
   a.lat = (const LatticeDev<real>*)c->d_lat;
   a.rows = (const RowConst<real>*)c->d_rows;
@@ -601,7 +603,9 @@ StepArgs<real> step_args(lb_ctx* c, int cur, int t_offset) {
   a.src = (const real*)c->f[cur];
   a.dst = (real*)c->f[cur ^ 1];
   a.d_t = c->d_t;
-  a.t_offset = t_offset;
+  a.device_t = c->device_t;
+  a.t_offset = (int)(uint32_t)(k + (c->device_t ? 0 : c->t));
+  a.t_store = t_store;
   a.fields = (real*)c->fields;
   a.pfield = (real*)c->pfield;
   a.partials = c->partials;
@@ -610,6 +614,7 @@ StepArgs<real> step_args(lb_ctx* c, int cur, int t_offset) {
   a.tmaps = c->tma ? c->d_tmaps : nullptr;
   a.n_lat = c->n_lat;
   a.src_buf = cur;
+  a.overlap = !c->device_t;
   return a;
 }
 
@@ -645,6 +650,16 @@ cudaError_t enqueue_sample(lb_ctx* c) {
   return launch_finalize(c->d_diag, c->n_lat, c->partials, c->stats, c->stream);
 }
 
+// Launches that a graph replays leave the device's step counter to a kernel of its own; others have it
+// stored by the call's last launch (t_after).
+cudaError_t advance(lb_ctx* c, int64_t n) {
+  if (!c->device_t) return cudaSuccess;
+  c->launches += 1;
+  return launch_advance(c->d_t, n, c->stream);
+}
+
+int64_t t_after(const lb_ctx* c, int64_t k, int64_t n) { return k == n ? c->t + n : -1; }
+
 // Enqueue `n` steps starting from buffer `cur`, with sampling by the bit mask.  Direct
 // launches: one step kernel per step.
 template <class real>
@@ -653,7 +668,7 @@ cudaError_t enqueue_direct(lb_ctx* c, int cur, int64_t n, const std::vector<int6
   for (int64_t k = 0; k < n; ++k) {
     const bool sample = si < sample_offsets.size() && sample_offsets[si] == k;
     if (sample) ++si;
-    cudaError_t e = launch_step<real>(step_args<real>(c, cur, (int)k), c->tile_x, sample, c->noise_mode, c->bulk_ok, c->stream);
+    cudaError_t e = launch_step<real>(step_args<real>(c, cur, k, t_after(c, k + 1, n)), c->tile_x, sample, c->noise_mode, c->bulk_ok, c->stream);
     if (e != cudaSuccess) return e;
     c->launches += 1;
     if (sample) {
@@ -662,8 +677,7 @@ cudaError_t enqueue_direct(lb_ctx* c, int cur, int64_t n, const std::vector<int6
     }
     cur ^= 1;
   }
-  c->launches += 1;
-  return launch_advance(c->d_t, n, c->stream);
+  return advance(c, n);
 }
 
 // Whether the persistent launch gives every block an item of its own (PersistArgs::owner): as many
@@ -701,14 +715,14 @@ cudaError_t enqueue_persistent(lb_ctx* c, int cur, int64_t n, const std::vector<
       if (e != cudaSuccess) return e;
       const PersistArgs pa{reinterpret_cast<unsigned long long*>(c->d_barrier), c->d_done, c->d_nbr_off, c->d_nbr,
                            c->d_err, 2000, owner_mode(c, grid), 0};
-      e = launch_step_persistent<real>(step_args<real>(c, cur, (int)k), c->tile_x, (int)plain, c->noise_mode,
+      e = launch_step_persistent<real>(step_args<real>(c, cur, k, t_after(c, k + plain, n)), c->tile_x, (int)plain, c->noise_mode,
                                        c->bulk_ok, pa, grid, c->stream);
       if (e != cudaSuccess) return e;
       c->launches += 1;
       if (plain & 1) cur ^= 1;
     }
     if (sample) {
-      e = launch_step<real>(step_args<real>(c, cur, (int)(end - 1)), c->tile_x, true, c->noise_mode, c->bulk_ok,
+      e = launch_step<real>(step_args<real>(c, cur, end - 1, t_after(c, end, n)), c->tile_x, true, c->noise_mode, c->bulk_ok,
                             c->stream);
       if (e != cudaSuccess) return e;
       c->launches += 1;
@@ -718,8 +732,7 @@ cudaError_t enqueue_persistent(lb_ctx* c, int cur, int64_t n, const std::vector<
     }
     k = end;
   }
-  c->launches += 1;
-  return launch_advance(c->d_t, n, c->stream);
+  return advance(c, n);
 }
 
 template <class real>
@@ -826,6 +839,10 @@ int step_impl(lb_ctx* c, int64_t n) {
   }
   const bool persistent = c->flags & LB_PERSISTENT;
   const bool graph = c->flags & LB_GRAPH;
+  // captured by the library's own graphs, or by a caller's capture of the stream
+  cudaStreamCaptureStatus cap_status = cudaStreamCaptureStatusNone;
+  if (!graph && cudaStreamIsCapturing(c->stream, &cap_status) != cudaSuccess) cudaGetLastError();
+  c->device_t = graph || cap_status != cudaStreamCaptureStatusNone;
   int64_t done = 0;
   while (done < n) {
     // segment: everything left (direct launches), or what one graph holds: up to 64 per-step
@@ -1098,7 +1115,6 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
   } runs[2];
   char* arena = nullptr;
   double* d_grad = nullptr;  // 3 n per run
-  int64_t* zero_t = nullptr;
   cudaStream_t st = c->stream, s1 = nullptr;
   cudaEvent_t ev[2] = {nullptr, nullptr};
   auto release = [&]() {
@@ -1198,7 +1214,6 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
       }
     }
     d_grad = (double*)piece((size_t)6 * n, sizeof(double));
-    zero_t = (int64_t*)piece(1, sizeof(int64_t));
   }
   cudaError_t e = cudaSuccess;
   auto ok = [&](cudaError_t r) {
@@ -1213,7 +1228,6 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
     }
     if (want_grad) ok(cudaMemcpy(R.kcs, R.hkcs.data(), (size_t)n * sizeof(AdjConst), cudaMemcpyHostToDevice));
   }
-  ok(cudaMemsetAsync(zero_t, 0, sizeof(int64_t), st));
   ok(cudaMemsetAsync(d_grad, 0, (size_t)6 * n * sizeof(double), st));
   ok(cudaEventRecord(ev[0], st));  // the second run's stream starts after the set-up
   ok(cudaStreamWaitEvent(s1, ev[0], 0));
@@ -1222,8 +1236,10 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
     a.src = src;
     a.dst = dst;
     a.tmaps = nullptr;  // the context's tensor maps describe its own state buffers, not these
-    a.d_t = zero_t;
+    a.device_t = 0;
     a.t_offset = (int)k;
+    a.t_store = -1;
+    a.overlap = 1;
     a.fields = R.fields;
     a.pfield = R.pfield;
     a.partials = R.partials;
@@ -1987,7 +2003,7 @@ int lb_load_checkpoint(lb_ctx* c, const void* host_buf, size_t bytes) {
   }
   if (ok && h.corr_mask) ok = to_device(c->corr_R, c->corr_R_n * sizeof(double)) &&
                               (c->corr_C_n == 0 || to_device(c->corr_C, c->corr_C_n * sizeof(double)));
-  // the step count, on the host and in the device counter that keys the noise
+  // the step count, on the host and in the device counter
   if (ok) ok = cudaMemcpy(c->d_t, &h.t, sizeof(int64_t), cudaMemcpyHostToDevice) == cudaSuccess;
   if (!ok) return LB_ERR_CUDA;
   c->t = h.t;

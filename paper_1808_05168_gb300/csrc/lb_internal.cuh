@@ -285,7 +285,12 @@ struct StepArgs {
   int n_items;
   const real* src;
   real* dst;
-  const int64_t* d_t;  // device step counter; the step index is *d_t + t_offset
+  // The step index is t_offset (mod 2^32), or with device_t (launches that a graph replays) *d_t +
+  // t_offset.  d_t: the device's step counter; without device_t the last launch of a call stores t_store
+  // there (negative: no store), so that it always holds the steps taken.
+  int64_t* d_t;
+  int device_t;
+  int64_t t_store;
   int t_offset;
   real* fields;        // sampled fields [4][Lz][Lx] per lattice (sample steps only)
   real* pfield;        // sampled pressure [Lz][Lx] per lattice, minus the row background in
@@ -299,7 +304,17 @@ struct StepArgs {
   const CUtensorMap* tmaps;
   int n_lat;
   int src_buf;
+  int overlap;  // launch_step: may start before the launch before it on the stream has ended (not while
+                // capturing)
 };
+
+// The step index of a launch's first step; one thread of the grid keeps the device's counter.
+template <class real>
+__device__ __forceinline__ int64_t launch_step_index(const StepArgs<real>& a) {
+  if (a.device_t) return *a.d_t + a.t_offset;
+  if (a.t_store >= 0 && blockIdx.x == 0 && threadIdx.x == 0) *a.d_t = a.t_store;
+  return a.t_offset;
+}
 
 // The stored state of a lattice: [link l][row z][column x][species s], so the populations of both
 // species of one (link, site) are adjacent and one 8-byte (FP32) or 16-byte (FP64) access moves
