@@ -75,6 +75,7 @@ class Simulation:
         flags |= 0 if tensor_maps else capi.LB_NO_TENSOR_MAPS
         self.flags = flags
         self.precision = precision
+        self._shapes = {}
         if allocator is None:
             self.h = capi.lb_create_batch([p.to_c() for p in self.lattices], flags)
         else:
@@ -135,7 +136,12 @@ class Simulation:
 
     # ---- results
     def shape(self, lattice: int = 0):
-        return capi.lb_lattice_shape(self.h, lattice)
+        # a context's shapes never change: asked for once (an index out of range always asks)
+        s = self._shapes.get(lattice)
+        if s is None:
+            s = capi.lb_lattice_shape(self.h, lattice)
+            self._shapes[lattice] = s
+        return s
 
     def structure_factor(self, field: str = "c", lattice: int = 0, qz0_only: bool = False):
         Lx, Lz = self.shape(lattice)

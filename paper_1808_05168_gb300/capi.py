@@ -73,6 +73,8 @@ _lock = threading.Lock()
 def load():
     """Load the compiled library; raises if it has not been built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -358,13 +360,11 @@ def lb_set_site_map(h, lattice, x0, Lx_global):
 
 def lb_export_columns(h, lattice, x_first, n_cols, device_ptr):
     """device_ptr: device address of 18 * Lz * n_cols values of the storage type."""
-    _check(load().lb_export_columns(h, int(lattice), int(x_first), int(n_cols), ctypes.c_void_p(int(device_ptr))),
-           "lb_export_columns")
+    _check(load().lb_export_columns(h, int(lattice), int(x_first), int(n_cols), int(device_ptr)), "lb_export_columns")
 
 
 def lb_import_columns(h, lattice, x_first, n_cols, device_ptr):
-    _check(load().lb_import_columns(h, int(lattice), int(x_first), int(n_cols), ctypes.c_void_p(int(device_ptr))),
-           "lb_import_columns")
+    _check(load().lb_import_columns(h, int(lattice), int(x_first), int(n_cols), int(device_ptr)), "lb_import_columns")
 
 
 def lb_power_spectrum(field_ptr, Lx, Lz, out_ptr, stream_handle=0):

@@ -1001,6 +1001,40 @@ int sync_and_check(lb_ctx* c) {
   return LB_OK;
 }
 
+// A result of n doubles that `launch(out)` puts on the device, the error flag behind it: one copy, after
+// the context's pending work.  The transforms' buffer holds it meanwhile (free between samples; the
+// stream orders it), if it is large enough.
+bool read_fits(const lb_ctx* c, size_t n) {
+  return c->diag_ready && (n + 1) * sizeof(double) <= 4 * (size_t)c->n_sites * 2 * (c->dev32 ? sizeof(float) : sizeof(double));
+}
+template <class Launch>
+int read_result(lb_ctx* c, double* host, size_t n, Launch launch) {
+  double* out = static_cast<double*>(c->tmp);
+  if (launch(out) != cudaSuccess) return LB_ERR_CUDA;
+  constexpr size_t kOneCopy = 32768;  // longer results go straight to the caller, the flag after them
+  double small[64], flag = 0.0;
+  std::vector<double> buf;
+  double* h = small;
+  cudaError_t e;
+  if (n <= kOneCopy) {
+    if (n + 1 > 64) {
+      buf.resize(n + 1);
+      h = buf.data();
+    }
+    e = cudaMemcpyAsync(h, out, (n + 1) * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+  } else {
+    e = cudaMemcpyAsync(host, out, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, out + n, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+  }
+  if (e != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) return LB_ERR_CUDA;
+  if ((n <= kOneCopy ? h[n] : flag) != 0.0) {
+    cudaMemset(c->d_err, 0, sizeof(int));
+    return LB_ERR_TIMEOUT;
+  }
+  if (n <= kOneCopy) std::copy(h, h + n, host);
+  return LB_OK;
+}
+
 int lattice_ok(lb_ctx* c, int lattice) { return c && lattice >= 0 && lattice < c->n_lat; }
 
 int ensure_scratch(lb_ctx* c) {
@@ -1564,31 +1598,19 @@ int lb_structure_factor(lb_ctx* c, int lattice, int field, int mode, double* out
   const int Lx = c->params[lattice].Lx, Lz = c->params[lattice].Lz;
   const size_t need = mode == LB_SF_QXQZ ? (size_t)Lx * Lz : (size_t)Lx;
   if (n_out != need) return LB_ERR_SIZE;
-  int rc = sync_and_check(c);
-  if (rc) return rc;
-  if (n_samples) *n_samples = c->nsamples;
   if (!c->diag_ready || c->nsamples == 0) {
+    int rc = sync_and_check(c);
+    if (rc) return rc;
     std::fill(out, out + need, 0.0);
-    return LB_OK;
+  } else {
+    const size_t off = 4 * (size_t)c->site_off[lattice] + (size_t)field * Lx * Lz;
+    int rc = read_result(c, out, need, [&](double* d) {
+      return launch_read_spectrum(c->acc_sum + off, c->acc_comp + off, Lx, Lz, (int)need, 1.0 / (double)c->nsamples,
+                                  c->d_err, d, c->stream);
+    });
+    if (rc) return rc;
   }
-  const size_t full = (size_t)Lx * Lz;
-  const size_t off = 4 * (size_t)c->site_off[lattice] + (size_t)field * full;
-  // LB_SF_QX needs the q_z = 0 row only (q_x > Lx/2 comes from row 0 as well)
-  const size_t ncopy = mode == LB_SF_QXQZ ? full : (size_t)Lx;
-  std::vector<double> s(ncopy), k(ncopy);
-  if (cudaMemcpy(s.data(), c->acc_sum + off, ncopy * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
-      cudaMemcpy(k.data(), c->acc_comp + off, ncopy * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return LB_ERR_CUDA;
-  // accumulated: q_x = 0 .. Lx/2 (Kahan sums: total = sum - comp); the rest by S(q) = S(-q)
-  const double inv = 1.0 / (double)c->nsamples;
-  const int rows_out = mode == LB_SF_QXQZ ? Lz : 1;
-  for (int n = 0; n < rows_out; ++n)
-    for (int q = 0; q < Lx; ++q) {
-      const int nn = q <= Lx / 2 ? n : (Lz - n) % Lz;
-      const int qq = q <= Lx / 2 ? q : Lx - q;
-      const size_t src = (size_t)nn * Lx + qq;
-      out[(size_t)n * Lx + q] = (s[src] - k[src]) * inv;
-    }
+  if (n_samples) *n_samples = c->nsamples;
   return LB_OK;
 }
 
@@ -1674,25 +1696,36 @@ int lb_set_correlations(lb_ctx* c, int field_mask, int n_modes, const int* modes
   return LB_OK;
 }
 
+namespace {
+// n accumulated values of a correlation, divided by the number of samples.
+int read_correlation(lb_ctx* c, const double* sums, size_t n, double* out, int64_t* n_samples) {
+  const double inv = c->corr_samples ? 1.0 / (double)c->corr_samples : 0.0;
+  int rc = LB_OK;
+  if (c->corr_samples > 0 && read_fits(c, n)) {
+    rc = read_result(c, out, n, [&](double* d) { return launch_read_scaled(sums, nullptr, (int)n, inv, c->d_err, d, c->stream); });
+    if (rc) return rc;
+  } else {
+    rc = sync_and_check(c);
+    if (rc) return rc;
+    if (c->corr_samples == 0) {
+      std::fill(out, out + n, 0.0);
+    } else {
+      if (cudaMemcpy(out, sums, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess) return LB_ERR_CUDA;
+      for (size_t i = 0; i < n; ++i) out[i] *= inv;
+    }
+  }
+  if (n_samples) *n_samples = c->corr_samples;
+  return LB_OK;
+}
+}  // namespace
+
 int lb_correlation(lb_ctx* c, int lattice, int field, double* out, size_t n_out, int64_t* n_samples) {
   if (!lattice_ok(c, lattice) || field < 0 || field > 3 || !out) return LB_ERR_BAD_PARAM;
   const int Lz = c->params[lattice].Lz;
   const size_t LL = (size_t)Lz * Lz;
   if (n_out != LL) return LB_ERR_SIZE;
   if (!(c->corr_mask & (1 << field))) return LB_ERR_STATE;
-  int rc = sync_and_check(c);
-  if (rc) return rc;
-  if (n_samples) *n_samples = c->corr_samples;
-  if (c->corr_samples == 0) {
-    std::fill(out, out + LL, 0.0);
-    return LB_OK;
-  }
-  if (cudaMemcpy(out, c->corr_R + c->diag[lattice].r_off + (size_t)field * LL, LL * sizeof(double),
-                 cudaMemcpyDeviceToHost) != cudaSuccess)
-    return LB_ERR_CUDA;
-  const double inv = 1.0 / (double)c->corr_samples;
-  for (size_t i = 0; i < LL; ++i) out[i] *= inv;
-  return LB_OK;
+  return read_correlation(c, c->corr_R + c->diag[lattice].r_off + (size_t)field * LL, LL, out, n_samples);
 }
 
 int lb_mode_correlation(lb_ctx* c, int lattice, int field, int mode_index, double* out, size_t n_out,
@@ -1704,57 +1737,57 @@ int lb_mode_correlation(lb_ctx* c, int lattice, int field, int mode_index, doubl
   const size_t LL = (size_t)Lz * Lz, nm = c->corr_modes.size();
   if (n_out != 2 * LL) return LB_ERR_SIZE;
   if (!(c->corr_mask & (1 << field))) return LB_ERR_STATE;
-  int rc = sync_and_check(c);
-  if (rc) return rc;
-  if (n_samples) *n_samples = c->corr_samples;
-  if (c->corr_samples == 0) {
-    std::fill(out, out + 2 * LL, 0.0);
-    return LB_OK;
-  }
   const size_t off = c->diag[lattice].c_off + (((size_t)field * nm + mode_index) * LL) * 2;
-  if (cudaMemcpy(out, c->corr_C + off, 2 * LL * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return LB_ERR_CUDA;
-  const double inv = 1.0 / (double)c->corr_samples;
-  for (size_t i = 0; i < 2 * LL; ++i) out[i] *= inv;
-  return LB_OK;
+  return read_correlation(c, c->corr_C + off, 2 * LL, out, n_samples);
 }
 
 int lb_profile(lb_ctx* c, int lattice, int field, double* out, size_t n_out, int64_t* n_samples) {
   if (!lattice_ok(c, lattice) || field < 0 || field > LB_FIELD_P || !out) return LB_ERR_BAD_PARAM;
   const lb_params& p = c->params[lattice];
   if (n_out != (size_t)p.Lz) return LB_ERR_SIZE;
-  int rc = sync_and_check(c);
-  if (rc) return rc;
-  if (n_samples) *n_samples = c->nsamples;
   if (!c->diag_ready || c->nsamples == 0) {
+    int rc = sync_and_check(c);
+    if (rc) return rc;
     std::fill(out, out + p.Lz, 0.0);
-    return LB_OK;
+  } else {
+    const size_t off = (size_t)field * c->n_rows + c->row_off[lattice];
+    int rc = read_result(c, out, p.Lz, [&](double* d) {
+      return launch_read_scaled(c->prof_sum + off, c->prof_comp + off, p.Lz, 1.0 / (double)c->nsamples, c->d_err, d,
+                                c->stream);
+    });
+    if (rc) return rc;
+    // the accumulated row means are of deviations: add rho_bar, c_0(z) or the row's background
+    // pressure (zero in FP64 mode) back
+    if (field == LB_FIELD_RHO) {
+      for (int z = 0; z < p.Lz; ++z) out[z] += kRhoBar;
+    } else if (field == LB_FIELD_C || field == LB_FIELD_P) {
+      const std::vector<RowD> rd = make_rows(p, c->flags, c->dev32);
+      for (int z = 0; z < p.Lz; ++z) out[z] += field == LB_FIELD_C ? rd[z].c0 : rd[z].Pbg;
+    }
   }
-  const size_t off = (size_t)field * c->n_rows + c->row_off[lattice];
-  std::vector<double> s(p.Lz), k(p.Lz);
-  if (cudaMemcpy(s.data(), c->prof_sum + off, p.Lz * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
-      cudaMemcpy(k.data(), c->prof_comp + off, p.Lz * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return LB_ERR_CUDA;
-  // the accumulated row means are of deviations: add rho_bar, c_0(z) or the row's background
-  // pressure (zero in FP64 mode) back
-  const std::vector<RowD> rd = make_rows(p, c->flags, c->dev32);
-  const double inv = 1.0 / (double)c->nsamples;
-  for (int z = 0; z < p.Lz; ++z) {
-    double v = (s[z] + k[z]) * inv;
-    if (field == LB_FIELD_RHO) v += kRhoBar;
-    else if (field == LB_FIELD_C) v += rd[z].c0;
-    else if (field == LB_FIELD_P) v += rd[z].Pbg;
-    out[z] = v;
-  }
+  if (n_samples) *n_samples = c->nsamples;
   return LB_OK;
 }
 
 int lb_mean_pressure(lb_ctx* c, int lattice, double* last, double* time_avg) {
   if (!lattice_ok(c, lattice)) return LB_ERR_BAD_PARAM;
-  int rc = sync_and_check(c);
-  if (rc) return rc;
   DiagStats st;
-  if (cudaMemcpy(&st, c->stats + lattice, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return LB_ERR_CUDA;
+  if (c->diag_ready) {
+    // the statistics as doubles (a multiple of one, and byte for byte what the copy returns)
+    static_assert(sizeof(DiagStats) % sizeof(double) == 0, "the statistics are copied as doubles");
+    constexpr size_t n = sizeof(DiagStats) / sizeof(double);
+    double h[n];
+    int rc = read_result(c, h, n, [&](double* d) {
+      cudaError_t e = cudaMemcpyAsync(d, c->stats + lattice, sizeof(st), cudaMemcpyDeviceToDevice, c->stream);
+      return e != cudaSuccess ? e : launch_read_scaled(nullptr, nullptr, 0, 0.0, c->d_err, d + n, c->stream);
+    });
+    if (rc) return rc;
+    std::memcpy(&st, h, sizeof(st));
+  } else {
+    int rc = sync_and_check(c);
+    if (rc) return rc;
+    if (cudaMemcpy(&st, c->stats + lattice, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return LB_ERR_CUDA;
+  }
   if (st.nonfinite) return LB_ERR_NONFINITE;
   if (last) *last = st.P_last;
   if (time_avg) *time_avg = c->nsamples ? (st.P_sum + st.P_comp) / (double)c->nsamples : 0.0;

@@ -495,6 +495,13 @@ template <class real>
 cudaError_t launch_from_absolute(const double* in, const BgParams& bp, real* f, cudaStream_t s);
 template <class real>
 cudaError_t launch_init_rest(real* f, const BgParams& bp, cudaStream_t s);
+// Results for the host in out[0 .. n), the error flag as a double in out[n]: the first n bins of a
+// spectrum from its Kahan sums, mirrored and scaled; and (a + b) inv, or a inv with b null.
+cudaError_t launch_read_spectrum(const double* sum, const double* comp, int Lx, int Lz, int n, double inv, const int* err,
+                                 double* out, cudaStream_t s);
+cudaError_t launch_read_scaled(const double* a, const double* b, int n, double inv, const int* err, double* out,
+                               cudaStream_t s);
+
 // Columns x_first .. x_first + n - 1 of all 18 planes of a stored state f (Lx x Lz) to or from a
 // packed buffer [18][Lz][n] (x-slab halo exchange).
 template <class real>
