@@ -511,15 +511,6 @@ __global__ void adj_gather_push_kernel(const LatticeDev<real>* lat, const RowCon
 // 256 x 128, 500 steps, FP64: 62 -> 52 ms for the whole gradient; eight lattices from FP32 state, 300
 // steps: 133 -> 83 ms (the local pass 290 -> 171 us a step, the gather 92 -> 28).
 
-// A stored population as a double; exactly the conversion, in integer instructions where the value is
-// normal.
-__device__ __forceinline__ double widen(double x) { return x; }
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t b = __float_as_uint(x), e = b & 0x7F800000u;
-  if (e == 0u || e == 0x7F800000u) return (double)x;
-  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
-}
-
 template <class real>
 struct PairOfState;
 template <>

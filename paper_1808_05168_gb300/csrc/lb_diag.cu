@@ -481,8 +481,8 @@ __device__ __forceinline__ double2 block_total(double a, double b) {
 
 // The sums over species A and B of a 16-byte group of stored pairs.
 __device__ __forceinline__ void add_group(const float4 v, double& a, double& b) {
-  a += (double)v.x + (double)v.z;
-  b += (double)v.y + (double)v.w;
+  a += widen(v.x) + widen(v.z);
+  b += widen(v.y) + widen(v.w);
 }
 __device__ __forceinline__ void add_group(const double2 v, double& a, double& b) {
   a += v.x;

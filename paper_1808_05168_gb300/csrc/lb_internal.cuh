@@ -276,6 +276,15 @@ __device__ __forceinline__ float sqrt_pos<float>(float v) { return sqrtf(v); }
 template <>
 __device__ __forceinline__ double sqrt_pos<double>(double v) { return sqrt(v); }
 
+// A stored population as a double; exactly the conversion, in integer instructions where the value is
+// normal.
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = b & 0x7F800000u;
+  if (e == 0u || e == 0x7F800000u) return (double)x;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
 // Host-side launch helpers implemented in lb_step.cu / lb_diag.cu.
 template <class real>
 struct StepArgs {

@@ -33,6 +33,7 @@
 
 #include <cstdio>
 
+#include "lb_fixed64.cuh"
 #include "lb_internal.cuh"
 
 namespace lbk {
@@ -392,6 +393,46 @@ __device__ __forceinline__ void site_normals(uint32_t site, uint32_t step, const
   for (int k = 3; k < 9; ++k) nz[k] = pr(g[k - 1], g[k + 5]);
 }
 
+// The inverse transform of one species from dq = rho / 36, the moments 3, 4, 5, 8 and the combinations
+// v13 = M1 - M6, h1 = M1 + 2 M6 (along z: v24, h2), all times 1/36: sums with powers of two, formed in
+// integers of one scale (lb_fixed64.cuh); in double where that does not apply.
+__device__ __forceinline__ void inverse64(double dq, double M3, double M4, double M5, double M8, double v13, double v24,
+                                          double h1, double h2, double f[9]) {
+  const uint32_t e = max(max(max(fixed_field(dq), fixed_field(M3)), max(fixed_field(M4), fixed_field(M5))),
+                         max(max(fixed_field(M8), fixed_field(v13)),
+                             max(max(fixed_field(v24), fixed_field(h1)), fixed_field(h2))));
+  if (fixed_ok(e)) {
+    const long long q = to_fixed(dq, e), q3 = to_fixed(M3, e), q4 = to_fixed(M4, e), q5 = to_fixed(M5, e),
+                    q8 = to_fixed(M8, e), p13 = to_fixed(v13, e), p24 = to_fixed(v24, e), g1 = to_fixed(h1, e),
+                    g2 = to_fixed(h2, e);
+    // the weights 16, 4 and 1 of the links go into the exponents
+    const long long b4 = q + q3 - 4 * q8, b5 = q + 4 * (q3 + 2 * q8);
+    const long long u13 = b4 + q4, u24 = b4 - q4, u57 = b5 + q5, u68 = b5 - q5, w57 = g1 + g2, w68 = g1 - g2;
+    f[0] = from_fixed<4>(q + 2 * (q8 - q3), e);
+    f[1] = from_fixed<2>(u13 + p13, e);
+    f[2] = from_fixed<2>(u24 + p24, e);
+    f[3] = from_fixed<2>(u13 - p13, e);
+    f[4] = from_fixed<2>(u24 - p24, e);
+    f[5] = from_fixed<0>(u57 + w57, e);
+    f[6] = from_fixed<0>(u68 - w68, e);
+    f[7] = from_fixed<0>(u57 - w57, e);
+    f[8] = from_fixed<0>(u68 + w68, e);
+  } else {
+    const double b4 = fma(-16.0, M8, 4.0 * (dq + M3)), b5 = fma(8.0, M8, fma(4.0, M3, dq));
+    const double u13 = fma(4.0, M4, b4), u24 = fma(-4.0, M4, b4), u57 = b5 + M5, u68 = b5 - M5;
+    const double w57 = h1 + h2, w68 = h1 - h2;
+    f[0] = fma(32.0, M8, fma(-32.0, M3, 16.0 * dq));
+    f[1] = fma(4.0, v13, u13);
+    f[2] = fma(4.0, v24, u24);
+    f[3] = fma(-4.0, v13, u13);
+    f[4] = fma(-4.0, v24, u24);
+    f[5] = u57 + w57;
+    f[6] = u68 - w68;
+    f[7] = u57 - w57;
+    f[8] = u68 + w68;
+  }
+}
+
 // Collision and inverse transform in double precision: the arithmetic of collide_out with the factors
 // arranged for the fewest FP64 instructions, which bound the double path (two lanes per clock and SM).
 // With a* both species feel one acceleration, so everything of m^eq and of the source that is common is
@@ -476,19 +517,11 @@ __device__ __forceinline__ void collide_out_f64(const Mom<double>& m, double2 d,
     h2 = fma2(pr(2.0), M7, M2);
   }
   const P dq = mul2(pr(1.0 / 36), d);
-  const P b4 = fma2(pr(-16.0), M8, mul2(pr(4.0), add2(dq, M3)));
-  const P b5 = fma2(pr(8.0), M8, fma2(pr(4.0), M3, dq));
-  const P u13 = fma2(pr(4.0), M4, b4), u24 = fma2(pr(-4.0), M4, b4), u57 = add2(b5, M5), u68 = sub2(b5, M5);
-  const P v57 = add2(h1, h2), v68 = sub2(h1, h2);
-  const P f[9] = {fma2(pr(32.0), M8, fma2(pr(-32.0), M3, mul2(pr(16.0 / 36), d))),
-                  fma2(pr(4.0), v13, u13),
-                  fma2(pr(4.0), v24, u24),
-                  fma2(pr(-4.0), v13, u13),
-                  fma2(pr(-4.0), v24, u24),
-                  add2(u57, v57),
-                  sub2(u68, v68),
-                  sub2(u57, v57),
-                  add2(u68, v68)};
+  double fA[9], fB[9];
+  inverse64(dq.x, M3.x, M4.x, M5.x, M8.x, v13.x, v24.x, h1.x, h2.x, fA);
+  inverse64(dq.y, M3.y, M4.y, M5.y, M8.y, v13.y, v24.y, h1.y, h2.y, fB);
+  const P f[9] = {pr(fA[0], fB[0]), pr(fA[1], fB[1]), pr(fA[2], fB[2]), pr(fA[3], fB[3]), pr(fA[4], fB[4]),
+                  pr(fA[5], fB[5]), pr(fA[6], fB[6]), pr(fA[7], fB[7]), pr(fA[8], fB[8])};
 #pragma unroll
   for (int l = 0; l < 9; ++l) __stcs(out + l * stride, f[l]);
 }
