@@ -891,6 +891,33 @@ int step_impl(lb_ctx* c, int64_t n) {
   return LB_OK;
 }
 
+// Rows per item of the default tile (128 columns): the shortest items that the resident blocks (slots)
+// take in one wave, so that every SM gets the same share and no wave is nearly empty; where that makes
+// items of more than 32 rows, the shortest that they take in three (a last wave then costs little, and
+// blocks that run ahead even out the rest).  One launch per step, us, items of one wave / of three waves /
+// of the former rule (halved from Lz to 4 x 152 items, at least 16 rows, or 2 below 32 MB): 1024 x 512 in
+// FP32 20.2 / 22.4 / 28.4, 1024 x 1024 35.6 / 40.5 / 41.5 and in FP64 367 / 378 / 394, 2048 x 1024 63 / 66 /
+// 73, 4096 x 1024 122 / 120 / 136 and in FP64 1522 / 1309 / 1436, 8192 x 2048 460 / 434 / 510; 256 x 128 in
+// FP64 19.7 (items of one row) against 22.3.
+int default_rows(const lb_ctx* c, int slots) {
+  auto fits = [&](int rows, int64_t most) {
+    int64_t items = 0;
+    for (const lb_params& p : c->params) items += (int64_t)((p.Lx + 127) / 128) * ((p.Lz + rows - 1) / rows);
+    return items <= most;
+  };
+  auto shortest = [&](int64_t most) {
+    int lo = 1, hi = c->max_Lz;  // the shortest that fits, or whole lattices
+    while (lo < hi) {
+      const int mid = lo + (hi - lo) / 2;
+      if (fits(mid, most)) hi = mid;
+      else lo = mid + 1;
+    }
+    return lo;
+  };
+  const int one = shortest(slots);
+  return one <= 32 ? one : shortest(3 * (int64_t)slots);
+}
+
 int create_impl(lb_ctx** out, int n, const lb_params* ps, int flags, lb_alloc_fn alloc_fn = nullptr,
                 lb_free_fn free_fn = nullptr, void* alloc_user = nullptr) {
   NvtxRange r("lb_create");
@@ -962,14 +989,9 @@ int create_impl(lb_ctx** out, int n, const lb_params* ps, int flags, lb_alloc_fn
               cudaMemset(c->d_mass, 0, MASS_BUF * sizeof(double)) != cudaSuccess))
     rc = LB_ERR_CUDA;
   if (!rc) {
-    // default tile: 128 columns; rows per item chosen so that the grid has a few waves, down to
-    // 16 rows, or to 2 when a state buffer fits well inside L2 (32 MB): short items re-read two
-    // halo rows each, which then come from L2 (on 256 x 128: 16 items of 16 rows 0.149 s per
-    // 2 x 2000 steps, 128 items of 2 rows 0.132 s)
-    int rows = c->max_Lz;
-    const int64_t cols = [&] { int64_t s = 0; for (auto& p : c->params) s += (p.Lx + 127) / 128; return s; }();
-    const int min_rows = c->n_f * rs <= ((size_t)32 << 20) ? 2 : 16;
-    while (rows > min_rows && cols * ((c->max_Lz + rows - 1) / rows) < 4 * 152) rows /= 2;
+    const int slots = c->dev32 ? persistent_grid<float>(128, c->noise_mode, c->bulk_ok)
+                               : persistent_grid<double>(128, c->noise_mode, c->bulk_ok);
+    const int rows = default_rows(c, slots > 0 ? slots : 4 * 152);
     rc = build_items(c, 128, rows);
   }
   if (!rc) {
@@ -1109,8 +1131,9 @@ int create_noiseless(lb_ctx** out, const lb_ctx* c) {
   }
   int rc = create_impl(out, c->n_lat, ps.data(), c->flags & ~(LB_GRAPH | LB_PERSISTENT | LB_AUTOTUNE), c->alloc_fn,
                        c->free_fn, c->alloc_user);
-  // one shape of items whatever the batch, so that a lattice's sums are those of the lattice alone
-  if (!rc && (rc = lb_set_tile(*out, 32, 2)) != LB_OK) {
+  // one shape of items whatever the batch, so that a lattice's sums are those of the lattice alone; rows of
+  // their own, since its steps are the latency of an item
+  if (!rc && (rc = lb_set_tile(*out, 32, 1)) != LB_OK) {
     lb_destroy(*out);
     *out = nullptr;
   }
