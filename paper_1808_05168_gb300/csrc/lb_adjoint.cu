@@ -688,8 +688,10 @@ __global__ void adj_sum_pressure(const double* __restrict__ part, const AdjMap m
   if (threadIdx.x == 0) out[(int64_t)k * map.n_lat + li] = a;
 }
 
+// 16 warps per SM (128 registers): eight lattices of 256 x 128 246 us per step, 255 with the 12 that the
+// compiler's own 168 registers leave.
 template <class real, bool NOISE, bool UNIT>
-__global__ void __launch_bounds__(kAdjBlock)
+__global__ void __launch_bounds__(kAdjBlock, 16)
     adj_local_default(const real* __restrict__ f, const double* __restrict__ fbar, const LatticeDev<real>* lat,
                       const AdjConst* __restrict__ kcs, const AdjMap map, const double* __restrict__ rho, uint32_t step,
                       double sign, double* __restrict__ mom, double* __restrict__ sb, double* __restrict__ shares,
@@ -757,6 +759,18 @@ __global__ void __launch_bounds__(kAdjBlock)
   const double Ux = Px * inv, Uz = Pz * inv;
   const double UxUx = Ux * Ux, UzUz = Uz * Uz, UxUz = Ux * Uz, Ud = UxUx - UzUz;
   const double ux = Ux * ax, uz = Uz * az, ap = ux + uz, am = ux - uz, cr = fma(Uz, ax, Ux * az);
+
+  double nz[6];  // the normals of moments 1, 2 and of A's and B's 4, 5
+  if (NOISE) {
+    real nn[14];
+    normals14<real>((uint32_t)i, step, L, tab, nn);
+    nz[0] = widen(nn[0]), nz[1] = widen(nn[1]), nz[2] = widen(nn[3]), nz[3] = widen(nn[4]), nz[4] = widen(nn[9]),
+    nz[5] = widen(nn[10]);
+  }
+  // so far only what older launches left: the sensitivities come from the grid before this one, and the
+  // next one (launched to overlap as well) may start, all before that grid having ended
+  wait_for_previous_grid();
+  let_next_grid_start();
 
   // t_a: the moments of w_l fbar_l up to a factor each (sbar_a = t_0/36, t_1/12, t_2/12, t_3/36, t_4/4,
   // t_5/4, t_6/12, t_7/12, t_8/72 with the 1/N_a of the transposed inverse transform)
@@ -829,11 +843,9 @@ __global__ void __launch_bounds__(kAdjBlock)
     ls = fma(-t[s][4], m4[s], fma(-t[s][5], m5[s], ls));
   }
   if (NOISE) {
-    real nn[14];
-    normals14<real>((uint32_t)i, step, L, tab, nn);
-    ld = fma(k.dsm, fma(widen(nn[0]), d[1], widen(nn[1]) * d[2]), ld);
-    ls = fma(k.d4, fma(t[0][4], widen(nn[3]), t[1][4] * widen(nn[9])), ls);
-    ls = fma(k.d5, fma(t[0][5], widen(nn[4]), t[1][5] * widen(nn[10])), ls);
+    ld = fma(k.dsm, fma(nz[0], d[1], nz[1] * d[2]), ld);
+    ls = fma(k.d4, fma(t[0][4], nz[2], t[1][4] * nz[4]), ls);
+    ls = fma(k.d5, fma(t[0][5], nz[3], t[1][5] * nz[5]), ls);
   }
   shares[i] += gG;
   shares[N + i] = fma(0.25, ls, shares[N + i]);
@@ -874,6 +886,8 @@ __global__ void __launch_bounds__(2 * kAdjBlock)
   const int z = i / Lx, x = i - z * Lx;
   const int xm = x == 0 ? Lx - 1 : x - 1, xp = x + 1 == Lx ? 0 : x + 1;
   const bool wall = z == 0 || z == Lz - 1;
+  wait_for_previous_grid();
+  let_next_grid_start();
   const double* sx = sb + 8 * so + (int64_t)(4 * sp) * N;
   const double *sz = sx + N, *s5 = sz + N, *s6 = s5 + N;  // x + z, z - x
   double rb;
@@ -1024,9 +1038,9 @@ cudaError_t launch_adjoint_step_default(const real* f_prev, const double* fbar, 
   const int nb = map.n_blocks;
   auto pair = [&](auto noise_c, auto unit_c) {
     constexpr bool U = decltype(unit_c)::value;
-    adj_local_default<real, decltype(noise_c)::value, U>
-        <<<nb, kAdjBlock, 0, s>>>(f_prev, fbar, lat, kcs, map, rho, step, sign, mom, sb, shares, tab);
-    adj_push_default<real, U><<<nb, 2 * kAdjBlock, 0, s>>>(lat, kcs, map, mom, sb, sign, fbar_prev);
+    launch_overlapped(true, adj_local_default<real, decltype(noise_c)::value, U>, dim3(nb), kAdjBlock, 0, s, f_prev, fbar, lat,
+                      kcs, map, rho, step, sign, mom, sb, shares, tab);
+    launch_overlapped(true, adj_push_default<real, U>, dim3(nb), 2 * kAdjBlock, 0, s, lat, kcs, map, mom, sb, sign, fbar_prev);
   };
   using T = std::true_type;
   using F = std::false_type;

@@ -285,6 +285,30 @@ __device__ __forceinline__ double widen(float x) {
   return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(b << 29));
 }
 
+// ---- programmatic dependent launches ----------------------------------------------------------------
+// A grid launched with overlap may start once every block of the grid before it on the stream has called
+// let_next_grid_start (or ended); it calls wait_for_previous_grid, which returns when that grid has ended
+// and its writes are visible, before it touches what that grid reads or writes.  Without the launch
+// attribute both calls are no-ops.
+__device__ __forceinline__ void let_next_grid_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... Params, class... Args>
+inline void launch_overlapped(bool overlap, void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                              Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // Host-side launch helpers implemented in lb_step.cu / lb_diag.cu.
 template <class real>
 struct StepArgs {

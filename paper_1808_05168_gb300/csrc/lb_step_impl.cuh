@@ -1130,9 +1130,6 @@ struct MinBlocks {
 // grid to end.  512 x 256 in FP32, one launch per step: 11.3 -> 8.4 us.  (Let go at the start of the blocks, the
 // next grid's blocks fill whatever slots are free and stay unevenly spread over the SMs: 1024 x 1024 in
 // FP32 45 -> 54 us.)  Without the launch attribute both are no-ops.
-__device__ __forceinline__ void let_next_grid_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 template <class real, bool SAMPLE, int NOISE>
 __global__ void __launch_bounds__(256, MinBlocks<real>::value) step_kernel(StepArgs<real> a) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -1330,18 +1327,8 @@ struct Family {
   }
   template <bool SAMPLE, int NOISE>
   static void launch(const StepArgs<real>& a, int tile_x, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.n_items);
-    cfg.blockDim = dim3(TX == 0 ? tile_x : TX);
-    cfg.dynamicSmemBytes = smem(tile_x);
-    cfg.stream = s;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = a.overlap ? 1 : 0;
-    if constexpr (TX == 0) cudaLaunchKernelEx(&cfg, step_kernel<real, SAMPLE, NOISE>, a);
-    else cudaLaunchKernelEx(&cfg, step_kernel_bulk<real, TX, SAMPLE, NOISE>, a);
+    if constexpr (TX == 0) launch_overlapped(a.overlap, step_kernel<real, SAMPLE, NOISE>, dim3(a.n_items), tile_x, smem(tile_x), s, a);
+    else launch_overlapped(a.overlap, step_kernel_bulk<real, TX, SAMPLE, NOISE>, dim3(a.n_items), TX, smem(TX), s, a);
   }
 };
 
