@@ -931,7 +931,9 @@ __device__ __forceinline__ bool process_item_bulk(const StepArgs<real>& a, const
   const int nact = min(TX, Lx - x0);
   const bool active = tid < nact;
   const int x = x0 + (active ? tid : 0);
-  const bool do_left = tid == 0, do_right = tid == nact - 1;
+  // the halo columns of a row's densities: left by thread TX-2, right by TX-1, in one pass of the last warp
+  const bool edge = tid >= TX - 2;
+  const int ej = tid == TX - 2 ? 0 : nact + 1;  // its place in the ring row; its input column is one less
   const Pr<real>* f = reinterpret_cast<const Pr<real>*>(src + L.f_off);  // [link][z][x] pairs
   Pr<real>* g = reinterpret_cast<Pr<real>*>(dst + L.f_off);
   const real k9 = L.k9, k36 = L.k36;
@@ -1023,8 +1025,7 @@ __device__ __forceinline__ bool process_item_bulk(const StepArgs<real>& a, const
     wait_row(slot);
     const int b = ring_slot(r) * W;
     if (active) ring[b + tid + 1] = rho_at(r, slot, tid + PAD);
-    if (do_left) ring[b] = rho_at(r, slot, PAD - 1);
-    if (do_right) ring[b + nact + 1] = rho_at(r, slot, nact + PAD);
+    if (edge) ring[b + ej] = rho_at(r, slot, ej + PAD - 1);
   };
   auto ghost_row = [&](int zg, int za) {
     const int bg = ring_slot(zg) * W, ba = ring_slot(za) * W;
@@ -1040,15 +1041,37 @@ __device__ __forceinline__ bool process_item_bulk(const StepArgs<real>& a, const
       }
     };
     if (active) copy1(tid + 1);
-    if (do_left) copy1(0);
-    if (do_right) copy1(nact + 1);
+    if (edge) copy1(ej);
   };
   // prologue: rows z0-1 .. z0+NSI-2 in flight
   auto slot_of = [](int r) { return (int)((unsigned)(r + NSI) % NSI); };  // r >= -1
   for (int r = z0 - 1; r <= z0 + NSI - 2; ++r) stage_row(r, slot_of(r));
-  if (z0 > 0) put_rho(z0 - 1, slot_of(z0 - 1));
-  put_rho(z0, slot_of(z0));
-  if (z0 == 0) ghost_row(-1, 0);
+  {
+    // The densities of the first three rows side by side (nothing else hides the latency of a sum here),
+    // and their six halo columns in one pass of the last warp's last threads; row by row, each halo column
+    // a pass of its own, this took 7800 of the 24000 clocks of a step of 64 x 32 in FP64, now 3800.  Persistent,
+    // us per step: 64 x 32 FP64 14.0 -> 12.2, 512 x 256 FP64 47.5 -> 45.1, FP32 6.85 -> 6.69; 8192 x 2048
+    // FP64 4961 -> 4743.
+    const bool lo = z0 > 0, hi = z0 + 1 < Lz;
+    if (lo) wait_row(slot_of(z0 - 1));
+    wait_row(slot_of(z0));
+    if (hi) wait_row(slot_of(z0 + 1));
+    if (active) {
+      const int rl = lo ? z0 - 1 : z0, rh = hi ? z0 + 1 : z0;
+      const Pr<real> dl = rho_at(rl, slot_of(rl), tid + PAD), dc = rho_at(z0, slot_of(z0), tid + PAD),
+                     dh = rho_at(rh, slot_of(rh), tid + PAD);
+      if (lo) ring[ring_slot(rl) * W + tid + 1] = dl;
+      ring[ring_slot(z0) * W + tid + 1] = dc;
+      if (hi) ring[ring_slot(rh) * W + tid + 1] = dh;
+    }
+    const int q = tid - (TX - 6);
+    if (q >= 0) {
+      const int r = z0 - 1 + (q >> 1), i = (q & 1) ? nact + 1 : 0;
+      if (r >= 0 && r < Lz) ring[ring_slot(r) * W + i] = rho_at(r, slot_of(r), i + PAD - 1);
+    }
+    __syncwarp();  // a ghost row's halo columns are copied by other threads of that warp
+    if (z0 == 0) ghost_row(-1, 0);
+  }
   int sp = slot_of(z0 - 1), sc = slot_of(z0), sn = slot_of(z0 + 1);  // slots of rows z-1, z, z+1
 
   const SiteK<real> K = site_constants<real, NOISE>(L);
@@ -1056,8 +1079,8 @@ __device__ __forceinline__ bool process_item_bulk(const StepArgs<real>& a, const
   bool ok = true;
 
   for (int z = z0; z < z1; ++z) {
-    if (z + 1 < Lz) put_rho(z + 1, sn);
-    else ghost_row(Lz, Lz - 1);
+    if (z + 1 == Lz) ghost_row(Lz, Lz - 1);
+    else if (z > z0) put_rho(z + 1, sn);
     __syncthreads();
     if (*abort_flag) {
       ok = false;
