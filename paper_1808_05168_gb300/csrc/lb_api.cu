@@ -772,7 +772,9 @@ int autotune(lb_ctx* c) {
       // state is untouched: every trial reads f[cur] and writes f[cur ^ 1]; the persistent
       // launch is timed as it schedules (tickets, per-item waits) in its trial mode, in which
       // every step reads f[cur]
-      const int reps = persistent ? 6 : 4;
+      // small batches: more steps, as a run's start and end weigh most there (512 x 256 in FP64, six steps:
+      // a shape of 50.4 us per step was taken for the best of 45.1)
+      const int reps = (persistent ? 6 : 4) * (int)std::clamp<int64_t>((1 << 20) / c->n_sites, 1, 4);
       const int grid =
           persistent ? std::min<int>(persistent_grid<real>(tx, c->noise_mode, c->bulk_ok), (int)c->items.size()) : 0;
       auto trial = [&](int steps) {
