@@ -634,20 +634,31 @@ cudaError_t enqueue_sample(lb_ctx* c) {
   p.prof_sum = c->prof_sum;
   p.prof_comp = c->prof_comp;
   p.n_rows = c->n_rows;
+  p.overlap = !c->device_t;
   cudaError_t e = launch_sf<real>(p, (const real*)c->fields, c->tmp, c->acc_sum, c->acc_comp, c->stream);
   if (e != cudaSuccess) return e;
-  e = launch_profiles<real>(c->d_diag, c->d_row_lat, c->n_rows, (const real*)c->fields, (const real*)c->pfield,
-                            c->prof_sum, c->prof_comp, c->stream);
-  if (e != cudaSuccess) return e;
-  c->launches += 4;
+  SampleTail t = {};
+  t.lat = c->d_diag;
   if (c->corr_mask) {
-    CorrPlan cp{c->d_diag, c->d_corr_real, c->n_corr_real, c->d_corr_mode, c->n_corr_mode, c->d_corr_modes,
-                (int)c->corr_modes.size()};
-    e = launch_corr<real>(cp, (const real*)c->fields, c->tmp, c->corr_R, c->corr_C, c->stream);
-    if (e != cudaSuccess) return e;
-    c->launches += (c->n_corr_real > 0) + (c->n_corr_mode > 0);
+    t.real_tasks = c->d_corr_real;
+    t.n_real_tasks = c->n_corr_real;
+    t.mode_tasks = c->d_corr_mode;
+    t.n_mode_tasks = c->n_corr_mode;
+    t.modes = c->d_corr_modes;
+    t.n_modes = (int)c->corr_modes.size();
+    t.R = c->corr_R;
+    t.C = c->corr_C;
   }
-  return launch_finalize(c->d_diag, c->n_lat, c->partials, c->stats, c->stream);
+  t.row_lat = c->d_row_lat;
+  t.n_rows = c->n_rows;
+  t.prof_sum = c->prof_sum;
+  t.prof_comp = c->prof_comp;
+  t.n_lat = c->n_lat;
+  t.partials = c->partials;
+  t.stats = c->stats;
+  t.overlap = !c->device_t;
+  c->launches += 3;
+  return launch_sample_tail<real>(t, (const real*)c->fields, (const real*)c->pfield, c->tmp, c->stream);
 }
 
 // Launches that a graph replays leave the device's step counter to a kernel of its own; others have it

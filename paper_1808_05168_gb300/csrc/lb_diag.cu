@@ -270,6 +270,7 @@ template <class real>
 __global__ void __launch_bounds__(512) sf_rows_kernel(const DiagLattice* lat, const int2* tasks, const real* fields, Cplx<real>* tmp,
                                double* prof_sum, double* prof_comp, int n_rows, int cap) {
   extern __shared__ __align__(16) unsigned char smem[];
+  wait_for_previous_grid();
   const int2 task = tasks[blockIdx.x];
   const DiagLattice L = lat[task.x];
   const int n = L.Lx, SS = sf_seq_stride(n), R = sf_row_group(n, L.Lz, cap);
@@ -346,6 +347,7 @@ template <class real>
 __global__ void __launch_bounds__(512) sf_cols_kernel(const DiagLattice* lat, const int2* tasks, const Cplx<real>* tmp, double* acc_sum,
                                double* acc_comp, int cap) {
   extern __shared__ __align__(16) unsigned char smem[];
+  wait_for_previous_grid();
   const int2 task = tasks[blockIdx.x];
   const DiagLattice L = lat[task.x];
   const int n = L.Lz, Lx = L.Lx, H = sf_half(Lx), SS = sf_seq_stride(n);
@@ -427,8 +429,9 @@ __device__ __forceinline__ double warp_total(double v) {
   return v;
 }
 
-__global__ void finalize_kernel(const DiagLattice* lat, int n_lat, const double* partials, DiagStats* stats) {
-  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+__device__ __forceinline__ void finalize_lattices(int block, const DiagLattice* lat, int n_lat, const double* partials,
+                                                  DiagStats* stats) {
+  const int i = (int)((block * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (i >= n_lat) return;  // the whole warp
   const DiagLattice L = lat[i];
   double p = 0, ma = 0, mb = 0;
@@ -449,6 +452,9 @@ __global__ void finalize_kernel(const DiagLattice* lat, int n_lat, const double*
   st.massB_last = L.mass_bg[1] + mb;
   if (!isfinite(P) || !isfinite(st.massA_last) || !isfinite(st.massB_last)) st.nonfinite = 1;
   stats[i] = st;
+}
+__global__ void finalize_kernel(const DiagLattice* lat, int n_lat, const double* partials, DiagStats* stats) {
+  finalize_lattices((int)blockIdx.x, lat, n_lat, partials, stats);
 }
 
 // Mass of the stored state of one lattice, both species at once.  Bound by memory in FP64 and by the
@@ -759,10 +765,10 @@ cudaError_t prepare_sf(size_t smem_rows, size_t smem_cols) {
 template <class real>
 cudaError_t launch_sf(const SfPlan& p, const real* fields, void* tmp, double* acc_sum, double* acc_comp,
                       cudaStream_t s) {
-  sf_rows_kernel<real><<<p.n_row_tasks, p.threads, p.smem_rows, s>>>(p.lat, p.row_tasks, fields, (Cplx<real>*)tmp,
-                                                                     p.prof_sum, p.prof_comp, p.n_rows, p.cap);
-  sf_cols_kernel<real><<<p.n_col_tasks, p.threads, p.smem_cols, s>>>(p.lat, p.col_tasks, (const Cplx<real>*)tmp,
-                                                                     acc_sum, acc_comp, p.cap);
+  launch_overlapped(p.overlap, sf_rows_kernel<real>, dim3(p.n_row_tasks), p.threads, p.smem_rows, s, p.lat, p.row_tasks,
+                    fields, (Cplx<real>*)tmp, p.prof_sum, p.prof_comp, p.n_rows, p.cap);
+  launch_overlapped(p.overlap, sf_cols_kernel<real>, dim3(p.n_col_tasks), p.threads, p.smem_cols, s, p.lat, p.col_tasks,
+                    (const Cplx<real>*)tmp, acc_sum, acc_comp, p.cap);
   return cudaGetLastError();
 }
 
@@ -866,10 +872,11 @@ cudaError_t launch_power_spectrum(const double* field, int Lx, int Lz, double* o
 // pressure over x in a fixed order (lane-strided partial sums in the working precision, four
 // values at a time, then in double and a butterfly) and adds the row mean to the compensated sum.
 template <class real>
-__global__ void profile_kernel(const DiagLattice* __restrict__ lat, const int* __restrict__ row_lat, int n_rows,
-                               const real* __restrict__ pfield, double* __restrict__ prof_sum,
-                               double* __restrict__ prof_comp) {
-  const int r = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+__device__ __forceinline__ void profile_rows(int block, const DiagLattice* __restrict__ lat,
+                                             const int* __restrict__ row_lat, int n_rows,
+                                             const real* __restrict__ pfield, double* __restrict__ prof_sum,
+                                             double* __restrict__ prof_comp) {
+  const int r = (int)(((int64_t)block * blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= n_rows) return;  // whole warps
   const DiagLattice& L = lat[row_lat[r]];
@@ -886,25 +893,14 @@ __global__ void profile_kernel(const DiagLattice* __restrict__ lat, const int* _
   if (lane == 0) neumaier_add(prof_sum[4 * (int64_t)n_rows + r], prof_comp[4 * (int64_t)n_rows + r], acc / (double)Lx);
 }
 
-template <class real>
-cudaError_t launch_profiles(const DiagLattice* lat, const int* row_lat, int n_rows, const real* fields,
-                            const real* pfield, double* prof_sum, double* prof_comp, cudaStream_t s) {
-  if (n_rows <= 0) return cudaSuccess;
-  const int64_t blocks = ((int64_t)n_rows * 32 + 255) / 256;
-  profile_kernel<real><<<(unsigned)blocks, 256, 0, s>>>(lat, row_lat, n_rows, pfield, prof_sum, prof_comp);
-  (void)fields;
-  return cudaGetLastError();
-}
-
 // Real-space correlation of one sample: block (CORR_TILE^2 threads) per (lattice, field, z tile,
 // z' tile); x runs in chunks of 32 staged in shared memory, each chunk's products summed in the
 // working precision and the chunk sums in double.
 template <class real>
-__global__ void corr_real_kernel(const DiagLattice* __restrict__ lat, const int4* __restrict__ tasks,
-                                 const real* __restrict__ fields, double* __restrict__ R) {
+__device__ __forceinline__ void corr_real_tile(int4 t, const DiagLattice* __restrict__ lat,
+                                               const real* __restrict__ fields, double* __restrict__ R) {
   constexpr int T = CORR_TILE;
   __shared__ real a[32][T + 1], b[32][T + 1];
-  const int4 t = tasks[blockIdx.x];
   const DiagLattice& L = lat[t.x];
   const int Lx = L.Lx, Lz = L.Lz, fld = t.y, z0 = t.z * T, zp0 = t.w * T;
   const int tz = threadIdx.x % T, tzp = threadIdx.x / T;
@@ -930,11 +926,10 @@ __global__ void corr_real_kernel(const DiagLattice* __restrict__ lat, const int4
 // Mode correlation of one sample: thread per (z, z') of a tile, from the row transforms
 // X(q, z) = sum_x dphi(x, z) exp(-i q x) (unnormalised): C += conj(X(q, z)) X(q, z') / Lx.
 template <class real>
-__global__ void corr_mode_kernel(const DiagLattice* __restrict__ lat, const int4* __restrict__ tasks,
-                                 const int* __restrict__ modes, int n_modes, const Cplx<real>* __restrict__ tmp,
-                                 double* __restrict__ C) {
+__device__ __forceinline__ void corr_mode_tile(int4 t, const DiagLattice* __restrict__ lat,
+                                               const int* __restrict__ modes, int n_modes,
+                                               const Cplx<real>* __restrict__ tmp, double* __restrict__ C) {
   constexpr int T = CORR_TILE;
-  const int4 t = tasks[blockIdx.x];
   const DiagLattice& L = lat[t.x];
   const int Lx = L.Lx, Lz = L.Lz, fld = t.y / n_modes, m = t.y - fld * n_modes, k = modes[m];
   const int z = t.z * T + (int)threadIdx.x % T, zp = t.w * T + (int)threadIdx.x / T;
@@ -951,13 +946,32 @@ __global__ void corr_mode_kernel(const DiagLattice* __restrict__ lat, const int4
   c[1] += (ur * vi - ui * vr) * inv;
 }
 
+// What is left of a sample after the transforms, one launch: blocks of correlation tiles, of pressure
+// rows and of lattices' statistics, which do not depend on one another (a launch each, they ran one after
+// another).  The three launches of a sample overlap at their ends where the steps do.  400 steps of 32
+// lattices of 128 x 32 in FP32 with 40 samples and their readouts: 11.9 -> 10.7 ms.
+constexpr int TAIL_THREADS = CORR_TILE * CORR_TILE;
 template <class real>
-cudaError_t launch_corr(const CorrPlan& p, const real* fields, const void* tmp, double* R, double* C, cudaStream_t s) {
-  if (p.n_real_tasks > 0)
-    corr_real_kernel<real><<<p.n_real_tasks, CORR_TILE * CORR_TILE, 0, s>>>(p.lat, p.real_tasks, fields, R);
-  if (p.n_mode_tasks > 0)
-    corr_mode_kernel<real><<<p.n_mode_tasks, CORR_TILE * CORR_TILE, 0, s>>>(
-        p.lat, p.mode_tasks, p.modes, p.n_modes, (const Cplx<real>*)tmp, C);
+__global__ void __launch_bounds__(TAIL_THREADS) sample_tail_kernel(SampleTail p, const real* __restrict__ fields,
+                                                                   const real* __restrict__ pfield,
+                                                                   const Cplx<real>* __restrict__ tmp) {
+  wait_for_previous_grid();
+  int b = (int)blockIdx.x;
+  if (b < p.n_real_tasks) return corr_real_tile<real>(p.real_tasks[b], p.lat, fields, p.R);
+  b -= p.n_real_tasks;
+  if (b < p.n_mode_tasks) return corr_mode_tile<real>(p.mode_tasks[b], p.lat, p.modes, p.n_modes, tmp, p.C);
+  b -= p.n_mode_tasks;
+  if (b < p.row_blocks) return profile_rows<real>(b, p.lat, p.row_lat, p.n_rows, pfield, p.prof_sum, p.prof_comp);
+  finalize_lattices(b - p.row_blocks, p.lat, p.n_lat, p.partials, p.stats);
+}
+
+template <class real>
+cudaError_t launch_sample_tail(SampleTail p, const real* fields, const real* pfield, const void* tmp, cudaStream_t s) {
+  constexpr int W = TAIL_THREADS / 32;  // rows and lattices per block
+  p.row_blocks = (p.n_rows + W - 1) / W;
+  const int blocks = p.n_real_tasks + p.n_mode_tasks + p.row_blocks + (p.n_lat + W - 1) / W;
+  launch_overlapped(p.overlap, sample_tail_kernel<real>, dim3(blocks), TAIL_THREADS, 0, s, p, fields, pfield,
+                    (const Cplx<real>*)tmp);
   return cudaGetLastError();
 }
 
@@ -969,9 +983,7 @@ cudaError_t launch_corr(const CorrPlan& p, const real* fields, const void* tmp, 
   template cudaError_t launch_from_absolute<real>(const double*, const BgParams&, real*, cudaStream_t);      \
   template cudaError_t launch_init_rest<real>(real*, const BgParams&, cudaStream_t);                         \
   template cudaError_t launch_columns<real>(real*, int, int, int, int, real*, bool, cudaStream_t);           \
-  template cudaError_t launch_profiles<real>(const DiagLattice*, const int*, int, const real*, const real*,    \
-                                             double*, double*, cudaStream_t);                                \
-  template cudaError_t launch_corr<real>(const CorrPlan&, const real*, const void*, double*, double*, cudaStream_t);
+  template cudaError_t launch_sample_tail<real>(SampleTail, const real*, const real*, const void*, cudaStream_t);
 LB_INST(float)
 LB_INST(double)
 

@@ -448,6 +448,7 @@ struct SfPlan {
   double* prof_sum;
   double* prof_comp;
   int n_rows;
+  bool overlap;  // with the launch before (launch_overlapped)
 };
 
 // The row transforms of a sample in tmp: the fields are real, so only q_x = 0 .. Lx/2 is kept,
@@ -489,30 +490,35 @@ template <class real>
 cudaError_t launch_sf(const SfPlan& p, const real* fields, void* tmp, double* acc_sum, double* acc_comp,
                       cudaStream_t s);
 
-// Two-point correlations of one sample (Sec. III.A-B, Appendix A), in tiles of CORR_TILE x
-// CORR_TILE rows (z, z'): real_tasks = (lattice, field, z tile, z' tile) add
-// (1/Lx) sum_x dphi(x, z) dphi(x, z') to R; mode_tasks = (lattice, field * n_modes + m, z tile,
-// z' tile) add dphi(q_m, z)^* dphi(q_m, z') (unitary partial transform in x) to C, from the row
-// transforms the structure-factor pass leaves in tmp.
+// What follows the transforms of a sample, in one launch.
+// Two-point correlations (Sec. III.A-B, Appendix A), in tiles of CORR_TILE x CORR_TILE rows (z, z'):
+// real_tasks = (lattice, field, z tile, z' tile) add (1/Lx) sum_x dphi(x, z) dphi(x, z') to R;
+// mode_tasks = (lattice, field * n_modes + m, z tile, z' tile) add dphi(q_m, z)^* dphi(q_m, z')
+// (unitary partial transform in x) to C, from the row transforms the structure-factor pass leaves in tmp.
+// z-profiles (Sec. III.C): the row pass of launch_sf adds the row means of delta rho, delta c, Ux and Uz
+// to the per-row compensated sums [5][n_rows]; this adds those of the sampled pressure (deviation), slot
+// 4; row_lat[r] is the lattice of global row r.  Last the lattices' statistics (launch_finalize).
 constexpr int CORR_TILE = 16;
-struct CorrPlan {
+
+struct SampleTail {
   const DiagLattice* lat;
   const int4* real_tasks;
-  int n_real_tasks;
   const int4* mode_tasks;
-  int n_mode_tasks;
+  int n_real_tasks, n_mode_tasks;  // 0: no correlations
   const int* modes;
   int n_modes;
+  double *R, *C;
+  const int* row_lat;
+  int n_rows;
+  int row_blocks;  // set by the launch
+  double *prof_sum, *prof_comp;
+  int n_lat;
+  const double* partials;
+  DiagStats* stats;
+  bool overlap;  // with the launch before (launch_overlapped)
 };
 template <class real>
-cudaError_t launch_corr(const CorrPlan& p, const real* fields, const void* tmp, double* R, double* C, cudaStream_t s);
-
-// z-profiles (Sec. III.C): the row pass of launch_sf adds the row means of delta rho, delta c, Ux
-// and Uz to the per-row compensated sums [5][n_rows]; this adds those of the sampled pressure
-// (deviation), slot 4; row_lat[r] is the lattice of global row r.
-template <class real>
-cudaError_t launch_profiles(const DiagLattice* lat, const int* row_lat, int n_rows, const real* fields,
-                            const real* pfield, double* prof_sum, double* prof_comp, cudaStream_t s);
+cudaError_t launch_sample_tail(SampleTail p, const real* fields, const real* pfield, const void* tmp, cudaStream_t s);
 
 cudaError_t launch_finalize(const DiagLattice* d_lat, int n_lat, const double* partials, DiagStats* stats,
                             cudaStream_t s);
