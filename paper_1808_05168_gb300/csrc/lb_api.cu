@@ -105,7 +105,8 @@ struct lb_ctx {
   int sf_threads = 256, sf_cap = 4096;  // sample-step transforms (sf_threads, SfPlan)
   size_t sf_smem_rows = 0, sf_smem_cols = 0;
   int64_t* d_t = nullptr;
-  bool device_t = false;  // the launches being enqueued go into a graph: they count steps on the device
+  bool device_t = false;  // the launches being enqueued count steps on the device, as graphs do that replay
+  bool captured = false;  // a caller has captured steps: its replays count on the device, unseen by the host
   unsigned* d_barrier = nullptr;  // the persistent launch's ticket counter (64-bit)
   unsigned* d_done = nullptr;     // persistent launch: steps completed per item
   int* d_nbr_off = nullptr;       // persistent launch: dependency lists of the items (CSR)
@@ -855,7 +856,8 @@ int step_impl(lb_ctx* c, int64_t n) {
   // captured by the library's own graphs, or by a caller's capture of the stream
   cudaStreamCaptureStatus cap_status = cudaStreamCaptureStatusNone;
   if (!graph && cudaStreamIsCapturing(c->stream, &cap_status) != cudaSuccess) cudaGetLastError();
-  c->device_t = graph || cap_status != cudaStreamCaptureStatusNone;
+  c->captured = c->captured || cap_status != cudaStreamCaptureStatusNone;
+  c->device_t = graph || c->captured;
   int64_t done = 0;
   while (done < n) {
     // segment: everything left (direct launches), or what one graph holds: up to 64 per-step

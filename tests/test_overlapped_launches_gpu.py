@@ -83,3 +83,26 @@ def test_captured_by_the_caller():
         torch.cuda.synchronize()
         got = sim.populations()
     assert np.array_equal(got, _run("dev32", (8,), lattices=[P[0]], every=0)[0])
+
+
+@pytest.mark.parametrize("kw", [{}, {"persistent": True}])
+def test_steps_after_replays_of_the_callers_graph(kw):
+    """Steps called directly between and after such replays go on from what the replays have run."""
+    with Simulation(P[0], precision="dev32", **kw) as sim:
+        st = torch.cuda.Stream()
+        sim.set_stream(st)
+        sim.step(2)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=st):
+            sim.step(2)
+        with torch.cuda.stream(st):
+            for _ in range(3):
+                g.replay()
+        sim.step(2)
+        with torch.cuda.stream(st):
+            g.replay()
+        sim.step(3)
+        torch.cuda.synchronize()
+        got = sim.populations()
+    assert np.array_equal(got, _run("dev32", (15,), lattices=[P[0]], every=0)[0])
