@@ -688,11 +688,13 @@ __global__ void adj_sum_pressure(const double* __restrict__ part, const AdjMap m
   if (threadIdx.x == 0) out[(int64_t)k * map.n_lat + li] = a;
 }
 
+// fbar (and mom and sb below) may still be written by the grid before this one while this one starts: no
+// __restrict__, which with const would let them be read as constant for the whole grid.
 // 16 warps per SM (128 registers): eight lattices of 256 x 128 246 us per step, 255 with the 12 that the
 // compiler's own 168 registers leave.
 template <class real, bool NOISE, bool UNIT>
 __global__ void __launch_bounds__(kAdjBlock, 16)
-    adj_local_default(const real* __restrict__ f, const double* __restrict__ fbar, const LatticeDev<real>* lat,
+    adj_local_default(const real* __restrict__ f, const double* fbar, const LatticeDev<real>* lat,
                       const AdjConst* __restrict__ kcs, const AdjMap map, const double* __restrict__ rho, uint32_t step,
                       double sign, double* __restrict__ mom, double* __restrict__ sb, double* __restrict__ shares,
                       const NormalTables* tab) {
@@ -874,8 +876,7 @@ __global__ void __launch_bounds__(kAdjBlock, 16)
 template <class real, bool UNIT>
 __global__ void __launch_bounds__(2 * kAdjBlock)
     adj_push_default(const LatticeDev<real>* lat, const AdjConst* __restrict__ kcs, const AdjMap map,
-                     const double* __restrict__ mom, const double* __restrict__ sb, double sign,
-                     double* __restrict__ fbar_prev) {
+                     const double* mom, const double* sb, double sign, double* __restrict__ fbar_prev) {
   constexpr int NM = UNIT ? 3 : 9;
   const int li = adj_lattice(map);
   const LatticeDev<real>& L = lat[li];
