@@ -265,7 +265,7 @@ def run_ours(args):
 # Double-precision arithmetic instructions (DFMA + DADD + DMUL, each one issue of the FP64 pipe)
 # per lattice update of the FP64 step kernel, from ncu's sm__sass_thread_inst_executed_op_d*
 # counters (profiles/step_kernel_bulk_f64_small.md).
-FP64_INSTR_PER_LU = 428.4
+FP64_INSTR_PER_LU = 132.8
 
 
 def fp64_roofline(glups):
