@@ -914,23 +914,46 @@ int step_impl(lb_ctx* c, int64_t n) {
 // FP32 20.2 / 22.4 / 28.4, 1024 x 1024 35.6 / 40.5 / 41.5 and in FP64 367 / 378 / 394, 2048 x 1024 63 / 66 /
 // 73, 4096 x 1024 122 / 120 / 136 and in FP64 1522 / 1309 / 1436, 8192 x 2048 460 / 434 / 510; 256 x 128 in
 // FP64 19.7 (items of one row) against 22.3.
+int64_t count_items(const lb_ctx* c, int tile_x, int rows) {
+  int64_t items = 0;
+  for (const lb_params& p : c->params) items += (int64_t)((p.Lx + tile_x - 1) / tile_x) * ((p.Lz + rows - 1) / rows);
+  return items;
+}
+int shortest_rows(const lb_ctx* c, int tile_x, int64_t most) {
+  int lo = 1, hi = c->max_Lz;  // the shortest that fits, or whole lattices
+  while (lo < hi) {
+    const int mid = lo + (hi - lo) / 2;
+    if (count_items(c, tile_x, mid) <= most) hi = mid;
+    else lo = mid + 1;
+  }
+  return lo;
+}
 int default_rows(const lb_ctx* c, int slots) {
-  auto fits = [&](int rows, int64_t most) {
-    int64_t items = 0;
-    for (const lb_params& p : c->params) items += (int64_t)((p.Lx + 127) / 128) * ((p.Lz + rows - 1) / rows);
-    return items <= most;
+  const int one = shortest_rows(c, 128, slots);
+  return one <= 32 ? one : shortest_rows(c, 128, 3 * (int64_t)slots);
+}
+
+// Whether the default items of a double-precision batch are 64 columns wide, and then their rows.  A step
+// takes as long as the SM with the most sites, the FP64 pipe being the bound: blocks on the fullest SM
+// times columns times rows, half a row added for the densities an item begins with.  Where items of 128
+// columns put a second block on some SMs only, those of 64 can even that out; they cost more per site (a
+// pass of a warp per row for two halo columns, two in the per-thread staging), so they have to win by a
+// quarter in this count, by 28% with per-thread staging (211 x 105, a count of 0.75: 20.2 / 22.0).  Us per
+// step, 128 / 64 columns, one launch per step and persistent: 160 x 96 18.0 / 12.4 and 19.0 / 13.6, four of
+// them 44.3 / 31.3 and 45.3 / 28.8, two of 130 x 64 18.1 / 18.1 and 19.0 / 15.3, 259 x 208 47.6 / 36.5 and
+// 44.8 / 37.8; eight of 256 x 128, a count of 0.88, 97 / 110.  FP32 steps are not bound by a pipe: 128 is the
+// best at all of these.
+bool default_narrow(const lb_ctx* c, int rows128, int slots64, int* rows) {
+  int dev = 0, sms = 0;
+  if (c->dev32 || rows128 > 32 || slots64 <= 0 || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+    return false;
+  auto count = [&](int tile_x, int r) {
+    return (count_items(c, tile_x, r) + sms - 1) / sms * std::min(tile_x, c->max_Lx) * (2 * r + 1);
   };
-  auto shortest = [&](int64_t most) {
-    int lo = 1, hi = c->max_Lz;  // the shortest that fits, or whole lattices
-    while (lo < hi) {
-      const int mid = lo + (hi - lo) / 2;
-      if (fits(mid, most)) hi = mid;
-      else lo = mid + 1;
-    }
-    return lo;
-  };
-  const int one = shortest(slots);
-  return one <= 32 ? one : shortest(3 * (int64_t)slots);
+  *rows = shortest_rows(c, 64, slots64);
+  return count_items(c, 128, rows128) > sms &&
+         100 * count(64, *rows) <= (c->bulk_ok ? 75 : 72) * count(128, rows128);
 }
 
 int create_impl(lb_ctx** out, int n, const lb_params* ps, int flags, lb_alloc_fn alloc_fn = nullptr,
@@ -1007,7 +1030,10 @@ int create_impl(lb_ctx** out, int n, const lb_params* ps, int flags, lb_alloc_fn
     const int slots = c->dev32 ? persistent_grid<float>(128, c->noise_mode, c->bulk_ok)
                                : persistent_grid<double>(128, c->noise_mode, c->bulk_ok);
     const int rows = default_rows(c, slots > 0 ? slots : 4 * 152);
-    rc = build_items(c, 128, rows);
+    int narrow_rows = 0;
+    const bool narrow =
+        default_narrow(c, rows, c->dev32 ? 0 : persistent_grid<double>(64, c->noise_mode, c->bulk_ok), &narrow_rows);
+    rc = narrow ? build_items(c, 64, narrow_rows) : build_items(c, 128, rows);
   }
   if (!rc) {
     for (int i = 0; i < n && !rc; ++i) {
