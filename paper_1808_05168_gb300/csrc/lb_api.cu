@@ -943,15 +943,16 @@ int default_rows(const lb_ctx* c, int slots) {
 // them 44.3 / 31.3 and 45.3 / 28.8, two of 130 x 64 18.1 / 18.1 and 19.0 / 15.3, 259 x 208 47.6 / 36.5 and
 // 44.8 / 37.8; eight of 256 x 128, a count of 0.88, 97 / 110.  FP32 steps are not bound by a pipe: 128 is the
 // best at all of these.
-bool default_narrow(const lb_ctx* c, int rows128, int slots64, int* rows) {
+// Twice as many blocks of 64 threads are resident as of 128 (slots128).
+bool default_narrow(const lb_ctx* c, int rows128, int slots128, int* rows) {
   int dev = 0, sms = 0;
-  if (c->dev32 || rows128 > 32 || slots64 <= 0 || cudaGetDevice(&dev) != cudaSuccess ||
+  if (c->dev32 || rows128 > 32 || slots128 <= 0 || cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     return false;
   auto count = [&](int tile_x, int r) {
     return (count_items(c, tile_x, r) + sms - 1) / sms * std::min(tile_x, c->max_Lx) * (2 * r + 1);
   };
-  *rows = shortest_rows(c, 64, slots64);
+  *rows = shortest_rows(c, 64, 2 * (int64_t)slots128);
   return count_items(c, 128, rows128) > sms &&
          100 * count(64, *rows) <= (c->bulk_ok ? 75 : 72) * count(128, rows128);
 }
@@ -1031,8 +1032,7 @@ int create_impl(lb_ctx** out, int n, const lb_params* ps, int flags, lb_alloc_fn
                                : persistent_grid<double>(128, c->noise_mode, c->bulk_ok);
     const int rows = default_rows(c, slots > 0 ? slots : 4 * 152);
     int narrow_rows = 0;
-    const bool narrow =
-        default_narrow(c, rows, c->dev32 ? 0 : persistent_grid<double>(64, c->noise_mode, c->bulk_ok), &narrow_rows);
+    const bool narrow = default_narrow(c, rows, slots, &narrow_rows);
     rc = narrow ? build_items(c, 64, narrow_rows) : build_items(c, 128, rows);
   }
   if (!rc) {
