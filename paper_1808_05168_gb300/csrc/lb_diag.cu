@@ -28,38 +28,79 @@ struct PairType {
 
 namespace {
 
-template <class real>
-__device__ __forceinline__ void twiddle(int k, int n, real& c, real& s);
-template <>
-__device__ __forceinline__ void twiddle<float>(int k, int n, float& c, float& s) {
-  // exp(-2 pi i k / n); k / n is exact in binary for power-of-two n
-  sincospif(-2.0f * (float)k / (float)n, &s, &c);
-}
-template <>
-__device__ __forceinline__ void twiddle<double>(int k, int n, double& c, double& s) {
-  sincospi(-2.0 * (double)k / (double)n, &s, &c);
-}
-
-// Twiddle tables of the sample-step transforms, exp(-2 pi i k / n) for k < n/2, every power of
-// two n = 2 .. 8192 at offset n/2 - 1; filled by prepare_sf and prepare_power_spectrum.
+// Twiddle tables of the transforms, exp(-2 pi i k / n) for k < n/2, every power of two n = 2 .. 8192 at
+// offset n/2 - 1.  Single precision: filled by prepare_sf, which only contexts call.  Double precision: part
+// of the module, since lb_power_spectrum reads it without a context, from its first call on, in a stream
+// capture or not; a fill by a kernel (then a wait for the device) would break a capture, and a note that it
+// was done would outlive the table when the device is reset.
 constexpr int TW_TABLE = 8192;
-__device__ Cplx<float> g_tw_f[TW_TABLE];
-__device__ Cplx<double> g_tw_d[TW_TABLE];
-template <class real>
-__device__ __forceinline__ Cplx<real>* tw_table();
-template <>
-__device__ __forceinline__ Cplx<float>* tw_table<float>() { return g_tw_f; }
-template <>
-__device__ __forceinline__ Cplx<double>* tw_table<double>() { return g_tw_d; }
 
+// The unevaluated sum of two doubles, and the product of two of them to about 2^-104 (Dekker 1971), for the
+// compiler's evaluation of the table.
+struct TwoDoubles {
+  double hi, lo;
+};
+constexpr TwoDoubles two_sum(double a, double b) {
+  const double s = a + b, t = s - a;
+  return {s, (a - (s - t)) + (b - t)};
+}
+constexpr TwoDoubles two_product(double a, double b) {
+  const double ca = 134217729.0 * a, cb = 134217729.0 * b;  // 2^27 + 1
+  const double ah = ca - (ca - a), bh = cb - (cb - b), al = a - ah, bl = b - bh;
+  const double p = a * b;
+  return {p, ((ah * bh - p) + ah * bl + al * bh) + al * bl};
+}
+constexpr TwoDoubles add(TwoDoubles a, TwoDoubles b) {
+  const TwoDoubles s = two_sum(a.hi, b.hi);
+  return two_sum(s.hi, s.lo + (a.lo + b.lo));
+}
+constexpr TwoDoubles multiply(TwoDoubles a, TwoDoubles b) {
+  const TwoDoubles p = two_product(a.hi, b.hi);
+  return two_sum(p.hi, p.lo + (a.hi * b.lo + a.lo * b.hi));
+}
+
+struct TwiddleTable {
+  Cplx<double> v[TW_TABLE];
+};
+constexpr TwiddleTable make_twiddles() {
+  // cos and sin of 2 pi j / 8192 in the first octant: the powers of exp(2 pi i / 8192), each the product of
+  // the last and the first; the rest by symmetry
+  const TwoDoubles c1{0x1.fffff62161a34p-1, -0x1.136dcb1f9b9c4p-57}, s1{0x1.921fb2aecb360p-11, 0x1.876157e566b4cp-65};
+  double co[1025] = {}, si[1025] = {};
+  TwoDoubles c{1.0, 0.0}, s{0.0, 0.0};
+  for (int j = 0; j <= 1024; ++j) {
+    co[j] = c.hi;
+    si[j] = s.hi;
+    const TwoDoubles ss = multiply(s, s1), cn = add(multiply(c, c1), TwoDoubles{-ss.hi, -ss.lo});
+    s = add(multiply(s, c1), multiply(c, s1));
+    c = cn;
+  }
+  TwiddleTable t{};
+  for (int n = 2; n <= TW_TABLE; n *= 2)
+    for (int k = 0; k < n / 2; ++k) {
+      const int j = k * (TW_TABLE / n), m = j <= 2048 ? j : 4096 - j;  // angle, and its mirror image below pi/2
+      const double cm = m <= 1024 ? co[m] : si[2048 - m], sm = m <= 1024 ? si[m] : co[2048 - m];
+      t.v[n / 2 - 1 + k] = Cplx<double>{j <= 2048 ? cm : -cm, -sm};
+    }
+  return t;
+}
+
+__device__ Cplx<float> g_tw_f[TW_TABLE];
+__device__ const TwiddleTable g_tw_d = make_twiddles();
 template <class real>
-__global__ void fill_tw_tables_kernel() {
+__device__ __forceinline__ const Cplx<real>* tw_table();
+template <>
+__device__ __forceinline__ const Cplx<float>* tw_table<float>() { return g_tw_f; }
+template <>
+__device__ __forceinline__ const Cplx<double>* tw_table<double>() { return g_tw_d.v; }
+
+__global__ void fill_tw_table_kernel() {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < TW_TABLE - 1; i += gridDim.x * blockDim.x) {
     const int n = 2 << (31 - __clz(i + 1));  // the table holding entry i: n/2 - 1 <= i < n - 1
     const int k = i - (n / 2 - 1);
-    real c, sn;
-    twiddle<real>(k, n, c, sn);
-    tw_table<real>()[i] = Cplx<real>{c, sn};
+    float c, sn;
+    sincospif(-2.0f * (float)k / (float)n, &sn, &c);  // k / n is exact in binary
+    g_tw_f[i] = Cplx<float>{c, sn};
   }
 }
 
@@ -754,8 +795,11 @@ cudaError_t launch_columns(real* f, int Lx, int Lz, int x_first, int n, real* bu
 
 template <class real>
 cudaError_t prepare_sf(size_t smem_rows, size_t smem_cols) {
-  fill_tw_tables_kernel<real><<<(TW_TABLE + 255) / 256, 256>>>();
-  cudaError_t e = cudaDeviceSynchronize();
+  cudaError_t e = cudaSuccess;
+  if (sizeof(real) == 4) {
+    fill_tw_table_kernel<<<(TW_TABLE + 255) / 256, 256>>>();
+    e = cudaDeviceSynchronize();
+  }
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(sf_rows_kernel<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_rows);
   if (e != cudaSuccess) return e;
@@ -838,10 +882,8 @@ static cudaError_t prepare_ps() {
   return cudaFuncSetAttribute(ps_cols_kernel<PTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPsSmemMax);
 }
 
-cudaError_t prepare_power_spectrum() {
-  fill_tw_tables_kernel<double><<<(TW_TABLE + 255) / 256, 256>>>();
-  cudaError_t e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) e = prepare_ps<4>();
+cudaError_t prepare_power_spectrum() {  // attributes only: legal while a stream is captured
+  cudaError_t e = prepare_ps<4>();
   if (e == cudaSuccess) e = prepare_ps<8>();
   if (e == cudaSuccess) e = prepare_ps<16>();
   return e;
