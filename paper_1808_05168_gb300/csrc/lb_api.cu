@@ -115,7 +115,7 @@ struct lb_ctx {
   CUtensorMap* d_tmaps = nullptr;  // bulk staging: 3-d tensor maps [buffer][lattice][run of 1, 2 links]
   bool tma = false;                // d_tmaps holds maps for the current tile
   int* d_err = nullptr;
-  const NormalTables* normals = nullptr;  // FP64 noise: the device's tables (normal_tables)
+  const NormalTables* normals = nullptr;  // FP64 noise: the tables (normal_tables)
   double* d_scratch = nullptr;  // 18 * max_lattice_sites doubles (populations I/O)
   double* d_mass = nullptr;     // lb_mass (MASS_BUF doubles)
   size_t bytes = 0;
@@ -1021,7 +1021,7 @@ int create_impl(lb_ctx** out, int n, const lb_params* ps, int flags, lb_alloc_fn
   c->stream = c->own_stream;
   if (!rc) rc = c->dev32 ? upload_tables<float>(c) : upload_tables<double>(c);
   if (!rc && (c->dev32 ? prepare_step<float>(256) : prepare_step<double>(256)) != cudaSuccess) rc = LB_ERR_CUDA;
-  if (!rc && !c->dev32 && normal_tables(&c->normals) != cudaSuccess) rc = LB_ERR_CUDA;
+  if (!rc && !c->dev32 && c->noise_mode != NOISE_OFF && normal_tables(&c->normals) != cudaSuccess) rc = LB_ERR_CUDA;
   if (!rc && (cudaMemset(c->stats, 0, n * sizeof(DiagStats)) != cudaSuccess ||
               cudaMemset(c->d_t, 0, sizeof(int64_t)) != cudaSuccess ||
               cudaMemset(c->d_err, 0, sizeof(int)) != cudaSuccess ||

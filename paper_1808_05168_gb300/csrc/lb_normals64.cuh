@@ -17,7 +17,7 @@
 // Against quadruple precision on 2^18 random pairs and the ends of the range: at most 7.4e-16 off, 6.9e-17
 // rms (the table-driven pair in double: 1.2e-15 and 1.2e-16).  FP64 instructions of a lattice update
 // 428 -> 208; four steps of 8192 x 2048 and the state read back 56.4 -> 28.4 ms.  327 KB of segments, 48 KB of
-// angles, filled once per device: nothing is formed per block any more (the tables in shared memory cost
+// angles, filled once per context: nothing is formed per block any more (the tables in shared memory cost
 // each launch of a small lattice about 20 us).
 #pragma once
 
@@ -80,8 +80,8 @@ __device__ __forceinline__ void normal_pair_fixed(uint32_t a, uint32_t b, double
   n1 = fixed59(x1, quad << 30 & 0x80000000u);         // negative in quadrants 2 and 3
 }
 
-// The tables of the current device, filled on first use (lb_step_f64.cu); the address is good for the
-// life of the process.  Synchronous on first use per device.
+// The tables of the current context, filled on its first use of them (lb_step_f64.cu); the address is good
+// for the life of that context, so every lb_ctx asks for its own.
 cudaError_t normal_tables(const NormalTables** tab);
 
 }  // namespace lbk

@@ -22,6 +22,7 @@ LB_STEP_INST(double)
 namespace {
 
 __device__ NormalTables g_normals;
+__device__ int g_normals_filled;  // zero until the tables are: in the module, like them
 
 // ln 2 in two parts, the first with 24 bits, so that its product with an exponent is exact
 constexpr double kLn2Hi = 0.693147182464599609375, kLn2Lo = -1.904654299957768e-09;
@@ -106,26 +107,25 @@ __global__ void fill_normals_kernel() {
 
 }  // namespace
 
+// The note that the tables are filled lies beside them on the device, so that it holds for the current
+// context's tables and for no others: after a device reset, or in a second context of the device, both are
+// new.  Fill and note are on the legacy stream, as is what the caller does next (lb_create_batch waits for
+// that stream before it returns).
 cudaError_t normal_tables(const NormalTables** tab) {
-  constexpr int kMaxDevices = 64;
   static std::mutex mu;
-  static void* addr[kMaxDevices] = {};
-  int dev = -1;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> g(mu);
-  if (!addr[dev]) {
-    void* p = nullptr;
-    e = cudaGetSymbolAddress(&p, g_normals);
-    if (e != cudaSuccess) return e;
+  void* p = nullptr;
+  cudaError_t e = cudaGetSymbolAddress(&p, g_normals);
+  int filled = 0;
+  if (e == cudaSuccess) e = cudaMemcpyFromSymbol(&filled, g_normals_filled, sizeof(filled));
+  if (e == cudaSuccess && !filled) {
     fill_normals_kernel<<<(2 * 4096 + 1024 + 2048 + 127) / 128, 128>>>();
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) return e;
-    addr[dev] = p;
+    filled = 1;
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_normals_filled, &filled, sizeof(filled));
   }
-  *tab = static_cast<const NormalTables*>(addr[dev]);
+  if (e != cudaSuccess) return e;
+  *tab = static_cast<const NormalTables*>(p);
   return cudaSuccess;
 }
 
