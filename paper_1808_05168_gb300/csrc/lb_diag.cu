@@ -432,8 +432,14 @@ __global__ void __launch_bounds__(512) sf_cols_kernel(const DiagLattice* lat, co
 // instructions per point and dimension): two real rows per complex transform, so that only
 // q_x = 0 .. Lx/2 goes through tmp and the column pass, which writes S(-q) = S(q) beside S(q).
 // 2048 x 1024: 158 us (448 us with radix-2 passes over all Lx complex columns), 64 x 64: 6.8 us (8.2).
+// The most threads ps_pass launches with PTS points each: a sequence of 4096 points (PTS 4) or 8192.
 template <int PTS>
-__global__ void __launch_bounds__(8192 / PTS) ps_rows_kernel(const double* __restrict__ phi, int Lx, int R,
+struct PsThreads {
+  static constexpr int most = (PTS == 4 ? 4096 : 8192) / PTS;
+  static_assert(most <= 1024, "a block cannot have more, and the compiler divides the registers by the bound");
+};
+template <int PTS>
+__global__ void __launch_bounds__(PsThreads<PTS>::most) ps_rows_kernel(const double* __restrict__ phi, int Lx, int R,
                                                       Cplx<double>* __restrict__ tmp) {
   extern __shared__ __align__(16) unsigned char smem[];
   Cplx<double>* tw = reinterpret_cast<Cplx<double>*>(smem);
@@ -442,7 +448,7 @@ __global__ void __launch_bounds__(8192 / PTS) ps_rows_kernel(const double* __res
 }
 
 template <int PTS>
-__global__ void __launch_bounds__(8192 / PTS) ps_cols_kernel(const Cplx<double>* __restrict__ tmp, int Lx, int Lz, int cq,
+__global__ void __launch_bounds__(PsThreads<PTS>::most) ps_cols_kernel(const Cplx<double>* __restrict__ tmp, int Lx, int Lz, int cq,
                                                       double* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int n = Lz, H = sf_half(Lx), SS = sf_seq_stride(n), q0 = blockIdx.x * cq, w = min(cq, H - q0);
@@ -854,8 +860,8 @@ cudaError_t launch_init_rest(real* f, const BgParams& bp, cudaStream_t s) {
 // One pass of the snapshot transforms over `seqs` sequences of n points.  A warp's FP64 instruction
 // holds the SM's pipe for 16 clocks however few of its lanes work, so a small pass wants many threads
 // of few points each (radix 4), a large one few passes through shared memory (radix 16).  Both passes,
-// in us with 4 / 8 / 16 points per thread: 512 x 256 24.6 / 31.9 / 51.3, 1024 x 256 35 / 35 / 53,
-// 1024 x 512 60 / 57 / 62, 2048 x 1024 220 / 211 / 207, 2048 x 4096 876 / 790 / 758; the lines lie at
+// in us with 4 / 8 / 16 points per thread: 64 x 64 16.6 / 24.7 / 38.9, 512 x 256 24.7 / 32.9 / 51.4, 1024 x 256
+// 35 / 35 / 53, 1024 x 512 61 / 55 / 62, 2048 x 1024 215 / 210 / 206, 2048 x 4096 918 / 788 / 757; the lines lie at
 // 2^17 and 2^19 complex points of a pass.  Blocks are of 64 or 128 threads (the best at each size), a
 // sequence that needs more takes a block of its own.
 struct PsPass {
