@@ -92,6 +92,8 @@ struct lb_ctx {
   int n_corr_real = 0, n_corr_mode = 0;
   int64_t corr_samples = 0;
   void* tmp = nullptr;      // 4 * n_sites complex
+  double* d_read = nullptr;     // a result on its way to the host (read_result), read_cap doubles
+  size_t read_cap = 0;
   double* acc_sum = nullptr;
   double* acc_comp = nullptr;
   double* partials = nullptr;
@@ -548,6 +550,8 @@ int alloc_diag(lb_ctx* c) {
   if (!rc) rc = dev_alloc(c, &c->prof_comp, 5 * (size_t)c->n_rows * sizeof(double));
   if (!rc) rc = dev_alloc(c, &c->d_row_lat, (size_t)c->n_rows * sizeof(int));
   if (!rc) rc = dev_alloc(c, (char**)&c->tmp, 4 * (size_t)c->n_sites * 2 * rs);
+  c->read_cap = (size_t)c->max_lattice_sites + 64;  // a spectrum and the flag, or a lattice's statistics
+  if (!rc) rc = dev_alloc(c, &c->d_read, c->read_cap * sizeof(double));
   if (!rc) rc = dev_alloc(c, &c->acc_sum, 4 * (size_t)c->n_sites * sizeof(double));
   if (!rc) rc = dev_alloc(c, &c->acc_comp, 4 * (size_t)c->n_sites * sizeof(double));
   if (rc) return rc;
@@ -1065,14 +1069,12 @@ int sync_and_check(lb_ctx* c) {
 }
 
 // A result of n doubles that `launch(out)` puts on the device, the error flag behind it: one copy, after
-// the context's pending work.  The transforms' buffer holds it meanwhile (free between samples; the
-// stream orders it), if it is large enough.
-bool read_fits(const lb_ctx* c, size_t n) {
-  return c->diag_ready && (n + 1) * sizeof(double) <= 4 * (size_t)c->n_sites * 2 * (c->dev32 ? sizeof(float) : sizeof(double));
-}
+// the context's pending work.  It passes through a buffer that nothing else uses: a read changes nothing
+// that a sample step works with, also one that the caller replays on another stream meanwhile.
+bool read_fits(const lb_ctx* c, size_t n) { return c->diag_ready && n + 1 <= c->read_cap; }
 template <class Launch>
 int read_result(lb_ctx* c, double* host, size_t n, Launch launch) {
-  double* out = static_cast<double*>(c->tmp);
+  double* out = c->d_read;
   if (launch(out) != cudaSuccess) return LB_ERR_CUDA;
   constexpr size_t kOneCopy = 32768;  // longer results go straight to the caller, the flag after them
   double small[64], flag = 0.0;
@@ -2166,7 +2168,7 @@ void lb_destroy(lb_ctx* c) {
                   c->tmp,     c->acc_sum,    c->acc_comp,   c->partials,  c->stats,      c->d_diag,
                   c->d_row_tasks, c->d_col_tasks, c->d_t, c->d_barrier, c->d_err, c->d_scratch, c->d_mass,
                   c->pfield, c->prof_sum, c->prof_comp, c->d_row_lat, c->corr_R, c->corr_C, c->d_corr_real,
-                  c->d_corr_mode, c->d_corr_modes, c->d_done, c->d_nbr_off, c->d_nbr, c->d_tmaps};
+                  c->d_corr_mode, c->d_corr_modes, c->d_read, c->d_done, c->d_nbr_off, c->d_nbr, c->d_tmaps};
   for (void* p : ptrs) dev_free(c, p);
   delete c;
 }
