@@ -1076,7 +1076,7 @@ template <class Launch>
 int read_result(lb_ctx* c, double* host, size_t n, Launch launch) {
   double* out = c->d_read;
   if (launch(out) != cudaSuccess) return LB_ERR_CUDA;
-  constexpr size_t kOneCopy = 32768;  // longer results go straight to the caller, the flag after them
+  constexpr size_t kOneCopy = 32768;  // longer results go straight to the caller, after the flag is known
   double small[64], flag = 0.0;
   std::vector<double> buf;
   double* h = small;
@@ -1088,16 +1088,19 @@ int read_result(lb_ctx* c, double* host, size_t n, Launch launch) {
     }
     e = cudaMemcpyAsync(h, out, (n + 1) * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   } else {
-    e = cudaMemcpyAsync(host, out, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, out + n, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+    e = cudaMemcpyAsync(&flag, out + n, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   }
   if (e != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) return LB_ERR_CUDA;
-  if ((n <= kOneCopy ? h[n] : flag) != 0.0) {
+  if ((n <= kOneCopy ? h[n] : flag) != 0.0) {  // the caller's buffer is as it was
     cudaMemset(c->d_err, 0, sizeof(int));
     return LB_ERR_TIMEOUT;
   }
-  if (n <= kOneCopy) std::copy(h, h + n, host);
-  return LB_OK;
+  if (n <= kOneCopy) {
+    std::copy(h, h + n, host);
+    return LB_OK;
+  }
+  e = cudaMemcpyAsync(host, out, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+  return e == cudaSuccess && cudaStreamSynchronize(c->stream) == cudaSuccess ? LB_OK : LB_ERR_CUDA;
 }
 
 int lattice_ok(lb_ctx* c, int lattice) { return c && lattice >= 0 && lattice < c->n_lat; }
