@@ -87,6 +87,7 @@ class Simulation:
         if getattr(self, "h", None):
             capi.lb_destroy(self.h)
             self.h = None
+            self._shapes.clear()  # a closed context has none
 
     def __del__(self):
         try:
@@ -136,12 +137,11 @@ class Simulation:
 
     # ---- results
     def shape(self, lattice: int = 0):
-        # a context's shapes never change: asked for once (an index out of range always asks)
-        s = self._shapes.get(lattice)
-        if s is None:
-            s = capi.lb_lattice_shape(self.h, lattice)
-            self._shapes[lattice] = s
-        return s
+        # a context's shapes never change: asked for once each (an index out of range always asks)
+        lattice = int(lattice)
+        if lattice not in self._shapes:
+            self._shapes[lattice] = capi.lb_lattice_shape(self.h, lattice)
+        return self._shapes[lattice]
 
     def structure_factor(self, field: str = "c", lattice: int = 0, qz0_only: bool = False):
         Lx, Lz = self.shape(lattice)
