@@ -1046,7 +1046,9 @@ int create_impl(lb_ctx** out, int n, const lb_params* ps, int flags, lb_alloc_fn
                                : launch_init_rest<double>((double*)c->f[0] + c->f_off[i], bp, nullptr);
       if (e != cudaSuccess) rc = cuda_err(e);
     }
-    if (!rc && cudaDeviceSynchronize() != cudaSuccess) rc = LB_ERR_CUDA;
+    // everything above is on the legacy stream; the device's other streams are not waited for (a gradient call
+    // makes a context too)
+    if (!rc && cudaStreamSynchronize(nullptr) != cudaSuccess) rc = LB_ERR_CUDA;
   }
   if (rc) {
     lb_destroy(c);
