@@ -696,10 +696,20 @@ cudaError_t enqueue_direct(lb_ctx* c, int cur, int64_t n, const std::vector<int6
   return advance(c, n);
 }
 
-// Whether the persistent launch gives every block an item of its own (PersistArgs::owner): as many
-// blocks as items, and every lattice cut into chunks of the same number of rows.
-int owner_mode(const lb_ctx* c, int grid) {
-  if (grid != (int)c->items.size()) return 0;
+// Whether the persistent launch gives every block an item of its own (PersistArgs::owner): items of one
+// length, at most one per SM and at most half of the blocks that fit (slots).  With more of them some SMs hold
+// two blocks and others one, and tickets even that out.  Us per step, owner / tickets: FP64 rows of 64 columns,
+// 32 of them 12.1 / 12.6, 152 12.4 / 12.7, 160 13.4 / 12.8, 256 13.6 / 13.7, of 128 columns, 152 13.5 / 13.7,
+// 192 18.7 / 17.1; FP32 32 x 64 columns 4.2 / 4.5, 152 4.3 / 4.5, 160 4.6 / 4.5, 512 x 192 (768) 8.1 / 6.3, 16
+// lattices of 128 x 32 (512) 6.3 / 5.3.
+// Half of the blocks that fit, since an owner's block waits for given blocks and so needs the whole grid
+// resident: two such grids at a time (a gradient call's, two contexts') are, whichever blocks come first.
+int owner_mode(const lb_ctx* c, int slots) {
+  const int n = (int)c->items.size();
+  int dev = 0, sms = 0;
+  if (n > slots / 2 || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n > sms)
+    return 0;
   for (const lb_params& p : c->params)
     if (std::min(p.Lz, c->rows_per_item) != std::min(c->params[0].Lz, c->rows_per_item)) return 0;
   return 1;
@@ -730,7 +740,7 @@ cudaError_t enqueue_persistent(lb_ctx* c, int cur, int64_t n, const std::vector<
       if (e == cudaSuccess) e = cudaMemsetAsync(c->d_done, 0, c->items.size() * sizeof(unsigned), c->stream);
       if (e != cudaSuccess) return e;
       const PersistArgs pa{reinterpret_cast<unsigned long long*>(c->d_barrier), c->d_done, c->d_nbr_off, c->d_nbr,
-                           c->d_err, 2000, owner_mode(c, grid), 0};
+                           c->d_err, 2000, owner_mode(c, c->coop_grid), 0};
       e = launch_step_persistent<real>(step_args<real>(c, cur, k, t_after(c, k + plain, n)), c->tile_x, (int)plain, c->noise_mode,
                                        c->bulk_ok, pa, grid, c->stream);
       if (e != cudaSuccess) return e;
@@ -791,8 +801,8 @@ int autotune(lb_ctx* c) {
       // small batches: more steps, as a run's start and end weigh most there (512 x 256 in FP64, six steps:
       // a shape of 50.4 us per step was taken for the best of 45.1)
       const int reps = (persistent ? 6 : 4) * (int)std::clamp<int64_t>((1 << 20) / c->n_sites, 1, 4);
-      const int grid =
-          persistent ? std::min<int>(persistent_grid<real>(tx, c->noise_mode, c->bulk_ok), (int)c->items.size()) : 0;
+      const int slots = persistent ? persistent_grid<real>(tx, c->noise_mode, c->bulk_ok) : 0;
+      const int grid = std::min<int>(slots, (int)c->items.size());
       auto trial = [&](int steps) {
         if (!persistent) {
           for (int k = 0; k < steps; ++k)
@@ -802,7 +812,7 @@ int autotune(lb_ctx* c) {
         cudaMemsetAsync(c->d_barrier, 0, sizeof(unsigned long long), c->stream);
         cudaMemsetAsync(c->d_done, 0, c->items.size() * sizeof(unsigned), c->stream);
         const PersistArgs pa{reinterpret_cast<unsigned long long*>(c->d_barrier), c->d_done, c->d_nbr_off, c->d_nbr,
-                             c->d_err, 2000, owner_mode(c, grid), 1};
+                             c->d_err, 2000, owner_mode(c, slots), 1};
         launch_step_persistent<real>(step_args<real>(c, c->cur, 0), tx, steps, c->noise_mode, c->bulk_ok, pa, grid,
                                      c->stream);
       };
@@ -1362,7 +1372,7 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
       ok(cudaMemsetAsync(x->d_barrier, 0, sizeof(unsigned long long), R.s));
       ok(cudaMemsetAsync(x->d_done, 0, x->items.size() * sizeof(unsigned), R.s));
       const PersistArgs pa{reinterpret_cast<unsigned long long*>(x->d_barrier), x->d_done, x->d_nbr_off, x->d_nbr,
-                           c->d_err, 2000, owner_mode(x, grid), 0, ring ? (int64_t)R.S : 0};
+                           c->d_err, 2000, owner_mode(x, x->coop_grid), 0, ring ? (int64_t)R.S : 0};
       ok(launch_step_persistent<real>(args(R, src, dst, k), x->tile_x, (int)nsteps, R.noise, x->bulk_ok, pa, grid, R.s));
       return;
     }

@@ -399,7 +399,7 @@ struct PersistArgs {
   const int* nbr;
   int* err;
   int limit_ms;
-  int owner;  // a block per item and items of one length: block b runs item b of every step
+  int owner;  // every block of the grid is resident and has an item: block b runs item b of every step
   int trial;  // autotuner's trial mode: every step reads src and writes dst (the state is untouched)
   int64_t ring = 0;  // elements per step: step k reads src + k ring and writes dst + k ring, no state
                      // is overwritten (0: the two buffers alternate)

@@ -1199,10 +1199,15 @@ __global__ void __launch_bounds__(TX, BulkBlocks<real>::value * 128 / TX) step_k
 // it reads is written, and no one still reads the region it overwrites.  The relation is
 // symmetric and the tickets an item waits on were all handed out before its own, so with every
 // block resident (cooperative launch) each wait ends; it is bounded all the same.
-// With a resident block for every item and items of one length (PersistArgs::owner) block b keeps item
-// b for all steps: no ticket to draw, and the item's constants stay in shared memory.  512 x 256 in
-// FP32: 6.75 us per step (128 x 1 items), 9.6 with tickets and the constants reloaded.  Items of different lengths are left to the tickets: the ensemble of 16 seeds, whose 128
-// x 256 items would each have a block of their own, runs 0.56 ms per step with tickets and 0.66 with owners.
+// With PersistArgs::owner (a block per item, the items of one length, a block per SM at most) block b keeps
+// item b for all steps: no ticket to draw, and the item's constants stay in shared memory.  64 x 32, us per
+// step with owners / with tickets: FP64 12.1 / 12.6, FP32 4.2 / 4.5.  An owner's block waits for given blocks, not
+// for what was handed out before, so that argument does not hold here and another has to: all blocks of the
+// grid are resident at the same time.  A cooperative launch is asked for that (a barrier of the whole grid needs
+// no less), and the host chooses owners only where the grid takes at most half of the blocks that fit, so that
+// two such grids are resident side by side even if each only got what the other leaves.  More of them at a time
+// rest on the cooperative launch alone, and on the bound of the waits.  Items of different lengths are left to
+// the tickets, with which a block that is done early takes the next.
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
