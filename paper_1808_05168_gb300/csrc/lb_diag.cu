@@ -998,11 +998,12 @@ __device__ __forceinline__ void corr_mode_tile(int4 t, const DiagLattice* __rest
 // rows and of lattices' statistics, which do not depend on one another (a launch each, they ran one after
 // another).  The three launches of a sample overlap at their ends where the steps do.  400 steps of 32
 // lattices of 128 x 32 in FP32 with 40 samples and their readouts: 11.9 -> 10.7 ms.
+// What the launches before hand on comes without __restrict__, as everywhere where launches overlap: with const
+// it would let the compiler read them as constant for the whole kernel, before the wait too.
 constexpr int TAIL_THREADS = CORR_TILE * CORR_TILE;
 template <class real>
-__global__ void __launch_bounds__(TAIL_THREADS) sample_tail_kernel(SampleTail p, const real* __restrict__ fields,
-                                                                   const real* __restrict__ pfield,
-                                                                   const Cplx<real>* __restrict__ tmp) {
+__global__ void __launch_bounds__(TAIL_THREADS) sample_tail_kernel(SampleTail p, const real* fields, const real* pfield,
+                                                                   const Cplx<real>* tmp) {
   wait_for_previous_grid();
   int b = (int)blockIdx.x;
   if (b < p.n_real_tasks) return corr_real_tile<real>(p.real_tasks[b], p.lat, fields, p.R);
