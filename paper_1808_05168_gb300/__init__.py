@@ -138,10 +138,10 @@ class Simulation:
     # ---- results
     def shape(self, lattice: int = 0):
         # a context's shapes never change: asked for once each (an index out of range always asks)
-        lattice = int(lattice)
-        if lattice not in self._shapes:
-            self._shapes[lattice] = capi.lb_lattice_shape(self.h, lattice)
-        return self._shapes[lattice]
+        s = self._shapes.get(int(lattice))
+        if s is None:
+            s = self._shapes[int(lattice)] = capi.lb_lattice_shape(self.h, lattice)
+        return s
 
     def structure_factor(self, field: str = "c", lattice: int = 0, qz0_only: bool = False):
         Lx, Lz = self.shape(lattice)
