@@ -401,7 +401,7 @@ struct PersistArgs {
   int limit_ms;
   int owner;  // every block of the grid is resident and has an item: block b runs item b of every step
   int trial;  // autotuner's trial mode: every step reads src and writes dst (the state is untouched)
-  int64_t ring = 0;  // elements per step: step k reads src + k ring and writes dst + k ring, no state
+  int64_t ring = 0;  // elements per step (negative: back): step k reads src + k ring and writes dst + k ring, no state
                      // is overwritten (0: the two buffers alternate)
 };
 
