@@ -1631,6 +1631,8 @@ int lb_set_tile(lb_ctx* c, int tile_x, int rows_per_item) {
   if (!c) return LB_ERR_BAD_PARAM;
   if (!(tile_x == 32 || tile_x == 64 || tile_x == 128 || tile_x == 256) || rows_per_item < 1)
     return LB_ERR_BAD_PARAM;
+  // steps in flight read the items and their schedule
+  if (cudaStreamSynchronize(c->stream) != cudaSuccess) return LB_ERR_CUDA;
   int rc = build_items(c, tile_x, std::min(rows_per_item, c->max_Lz));
   if (rc) return rc;
   c->tile_fixed = true;
