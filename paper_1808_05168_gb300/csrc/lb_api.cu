@@ -1493,38 +1493,44 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
   ok(cudaEventRecord(ev[1], s1));
   ok(cudaStreamWaitEvent(st, ev[1], 0));
   std::vector<DiagStats> hs(2 * (size_t)n);
-  std::vector<double> hg(6 * (size_t)n, 0.0), hp[2];
-  for (int q = 0; q < 2; ++q) {
-    if (fused) {
-      hp[q].resize((size_t)T * n);
-      ok(cudaMemcpyAsync(hp[q].data(), runs[q].psum, hp[q].size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-    } else {
+  std::vector<double> hg(6 * (size_t)n, 0.0);
+  if (!fused)
+    for (int q = 0; q < 2; ++q)
       ok(cudaMemcpyAsync(hs.data() + (size_t)q * n, runs[q].stats, (size_t)n * sizeof(DiagStats), cudaMemcpyDeviceToHost,
                          st));
-    }
-  }
   if (want_grad) ok(cudaMemcpyAsync(hg.data(), d_grad, hg.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   ok(cudaStreamSynchronize(st));
-  // time averages of the mean pressure, per run and lattice (compensated sums over the steps)
-  std::vector<double> mean(2 * (size_t)n);
+  // time averages of the mean pressure, per run and lattice: compensated sums over the steps.  The steps' values
+  // come in pieces of 512 kB (or one step): host memory is no matter of the number of steps.
+  std::vector<double> mean(2 * (size_t)n), sum(n), comp(n);
+  const int64_t most = std::min(T, std::max<int64_t>(1, 65536 / n));
+  std::vector<double> hp(fused ? (size_t)most * n : 0);
   bool nonfinite = false;
-  for (int q = 0; q < 2; ++q)
+  for (int q = 0; q < 2; ++q) {
     for (int i = 0; i < n; ++i) {
-      double sum = hs[(size_t)q * n + i].P_sum, comp = hs[(size_t)q * n + i].P_comp;
-      if (fused) {
-        const DiagLattice& d = runs[q].x->diag[i];
-        sum = comp = 0.0;
-        for (int64_t t = 0; t < T; ++t) {
-          const double v = d.P_bg_mean + hp[q][(size_t)t * n + i] / d.n_sites, r = sum + v;
-          comp += std::fabs(sum) >= std::fabs(v) ? (sum - r) + v : (v - r) + sum;
-          sum = r;
-        }
-        nonfinite = nonfinite || !std::isfinite(sum);
-      } else {
-        nonfinite = nonfinite || hs[(size_t)q * n + i].nonfinite != 0;
-      }
-      mean[(size_t)q * n + i] = (sum + comp) / (double)T;
+      const DiagStats& x = hs[(size_t)q * n + i];
+      sum[i] = fused ? 0.0 : x.P_sum;
+      comp[i] = fused ? 0.0 : x.P_comp;
+      nonfinite = nonfinite || (!fused && x.nonfinite != 0);
     }
+    for (int64_t t0 = 0; fused && t0 < T && e == cudaSuccess; t0 += most) {
+      const int64_t len = std::min(most, T - t0);
+      ok(cudaMemcpyAsync(hp.data(), runs[q].psum + t0 * n, (size_t)(len * n) * sizeof(double), cudaMemcpyDeviceToHost, st));
+      ok(cudaStreamSynchronize(st));
+      for (int i = 0; i < n; ++i) {
+        const DiagLattice& d = runs[q].x->diag[i];
+        for (int64_t t = 0; t < len; ++t) {
+          const double v = d.P_bg_mean + hp[(size_t)t * n + i] / d.n_sites, r = sum[i] + v;
+          comp[i] += std::fabs(sum[i]) >= std::fabs(v) ? (sum[i] - r) + v : (v - r) + sum[i];
+          sum[i] = r;
+        }
+      }
+    }
+    for (int i = 0; i < n; ++i) {
+      nonfinite = nonfinite || (fused && !std::isfinite(sum[i]));
+      mean[(size_t)q * n + i] = (sum[i] + comp[i]) / (double)T;
+    }
+  }
   release();
   if (e != cudaSuccess) return cuda_err(e);
   if (nonfinite) return LB_ERR_NONFINITE;
