@@ -247,9 +247,9 @@ int lb_power_spectrum(const double* field, int Lx, int Lz, double* out, void* st
  * ordering as lb_power_spectrum, and in addition Lx * Lz <= LB_NOALLOC_MAX_POINTS (larger
  * products return LB_ERR_SIZE);
  * the intermediate transform lives in a fixed 4 MiB array compiled into the library, which
- * every GPU that loads the library holds until the process exits.  The first call on a device
- * (with that device current) looks up the array's device address and sets the kernels'
- * attributes, so make that first call before any stream capture.  Every call shares the one
+ * every GPU that loads the library holds until the process exits.  The first call in a CUDA
+ * context sets the kernels' attributes, so make it where the library may be loaded onto the device
+ * (inside a stream capture it is captured like any other call).  Every call in a context shares the one
  * array: calls whose work overlaps on the GPU (different streams, or different host threads)
  * race on it and give wrong results; the array needs no clearing, since each call overwrites
  * what it reads. */

@@ -1153,20 +1153,51 @@ int power_spectrum_args_ok(const double* field, int Lx, int Lz, const double* ou
   return LB_OK;
 }
 
+namespace {
+// The current context's id, which no later context of the process gets again: what is kept per context goes
+// by it, since the device's ordinal stays when the device is reset and is shared by several contexts.
+bool current_context_id(unsigned long long* id) {
+  using GetCurrent = CUresult (*)(CUcontext*);
+  using GetId = CUresult (*)(CUcontext, unsigned long long*);
+  struct Entries {
+    GetCurrent current = nullptr;
+    GetId id = nullptr;
+  };
+  static const Entries fn = [] {
+    Entries f;
+    void *a = nullptr, *b = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &a, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess &&
+        cudaGetDriverEntryPointByVersion("cuCtxGetId", &b, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+        q == cudaDriverEntryPointSuccess) {
+      f.current = reinterpret_cast<GetCurrent>(a);
+      f.id = reinterpret_cast<GetId>(b);
+    }
+    cudaGetLastError();
+    return f;
+  }();
+  CUcontext ctx = nullptr;
+  return fn.id && fn.current(&ctx) == CUDA_SUCCESS && ctx && fn.id(ctx, id) == CUDA_SUCCESS;
+}
+}  // namespace
+
+// The kernels' attributes, once per context (in every call where the context cannot be told or too many have
+// been seen: the same values again).
 int prepare_power_spectrum_current_device() {
-  constexpr int kMaxDevices = 64;
+  constexpr int kMost = 64;
   static std::mutex mu;
-  static bool done[kMaxDevices] = {};
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+  static unsigned long long ready[kMost];
+  static int n_ready = 0;
+  unsigned long long id = 0;
+  const bool known = current_context_id(&id);
+  std::lock_guard<std::mutex> g(mu);
+  if (known && std::find(ready, ready + n_ready, id) != ready + n_ready) return LB_OK;
+  if (prepare_power_spectrum() != cudaSuccess) {
     cudaGetLastError();
     return LB_ERR_CUDA;
   }
-  std::lock_guard<std::mutex> g(mu);
-  if (!done[dev]) {
-    if (prepare_power_spectrum() != cudaSuccess) return LB_ERR_CUDA;
-    done[dev] = true;
-  }
+  if (known && n_ready < kMost) ready[n_ready++] = id;
   return LB_OK;
 }
 

@@ -555,7 +555,7 @@ cudaError_t launch_power_spectrum(const double* field, int Lx, int Lz, double* o
 // Lx and Lz are powers of two in 2..8192 and field and out are device (or managed) memory of the
 // current device; LB_OK otherwise.
 int power_spectrum_args_ok(const double* field, int Lx, int Lz, const double* out);
-// prepare_power_spectrum once per device, with that device current (LB_OK or LB_ERR_CUDA).
+// prepare_power_spectrum once per CUDA context, in the current one (LB_OK or LB_ERR_CUDA).
 int prepare_power_spectrum_current_device();
 
 // Measured fused multiply-add rate of the current device (FP64 or FP32 scalar FMA, 2 flops each),

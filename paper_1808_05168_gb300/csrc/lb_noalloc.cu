@@ -9,8 +9,6 @@
 // (4 MiB), which every GPU that loads the library holds until the process exits.
 #include <cuda_runtime.h>
 
-#include <mutex>
-
 #include "lb_internal.cuh"
 
 namespace {
@@ -23,27 +21,14 @@ static_assert(kNoAllocMaxPoints == LB_NOALLOC_MAX_POINTS, "limit out of sync wit
 // (two streams, or two host threads) race on it.
 static __device__ __align__(256) double2 g_noalloc_scratch[kNoAllocMaxPoints];
 
-constexpr int kMaxDevices = 64;
-std::mutex g_mu;
-void* g_scratch_addr[kMaxDevices] = {};  // device address of g_noalloc_scratch, per device
-
-// Once per device, with that device current: the array's device address (the host-side name of
-// g_noalloc_scratch is only a stand-in and must never reach a kernel) and the kernels'
-// shared-memory attributes.
+// The array's address in the current context (the host-side name of g_noalloc_scratch is only a stand-in and
+// must never reach a kernel), asked for in every call: it belongs to the context, not to the device's ordinal.
+// Once per context the kernels' shared-memory attributes.
 int setup_current_device(void** scratch) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return LB_ERR_CUDA;
-  {
-    std::lock_guard<std::mutex> g(g_mu);
-    if (!g_scratch_addr[dev]) {
-      void* p = nullptr;
-      if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) {
-        cudaGetLastError();
-        return LB_ERR_CUDA;
-      }
-      g_scratch_addr[dev] = p;
-    }
-    *scratch = g_scratch_addr[dev];
+  *scratch = nullptr;
+  if (cudaGetSymbolAddress(scratch, g_noalloc_scratch) != cudaSuccess || !*scratch) {
+    cudaGetLastError();
+    return LB_ERR_CUDA;
   }
   return lbk::prepare_power_spectrum_current_device();
 }
