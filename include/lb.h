@@ -235,8 +235,10 @@ int lb_import_columns(lb_ctx* ctx, int lattice, int x_first, int n_cols, const v
  * alias field), in memory of the current device (or managed memory); Lx and Lz are powers of two
  * in 2..8192.  Host pointers, another device's memory or other sizes return LB_ERR_BAD_PARAM
  * before anything is launched.  Stream-ordered on `stream` (NULL: legacy default stream), which also
- * orders a device scratch of (Lx/2 + 1) * Lz * 16 bytes allocated and freed with cudaMallocAsync /
- * cudaFreeAsync; returns before the result is ready. */
+ * orders a device scratch of (Lx/2 + 1) * Lz * 16 bytes, allocated and freed in stream order
+ * (cudaMallocFromPoolAsync / cudaFreeAsync) from a memory pool of the library's own, one per CUDA
+ * context, which keeps unused memory as the device's current pool does, up to 64 MiB; inside a
+ * stream capture the scratch is the graph's.  Returns before the result is ready. */
 int lb_power_spectrum(const double* field, int Lx, int Lz, double* out, void* stream);
 
 /* lb_power_spectrum for callers that must not allocate device memory (the paper has no

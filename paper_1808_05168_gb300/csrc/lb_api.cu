@@ -1180,7 +1180,72 @@ bool current_context_id(unsigned long long* id) {
   CUcontext ctx = nullptr;
   return fn.id && fn.current(&ctx) == CUDA_SUCCESS && ctx && fn.id(ctx, id) == CUDA_SUCCESS;
 }
+
+// The snapshot spectrum's scratch, in stream order.  With the device's own pool a call waits in cudaMallocAsync
+// while other streams' scratch is in flight: looking for memory that those streams have just done with
+// (opportunistic reuse) took 20 to 100 us of host time, more than the transforms of up to 2^18 points.  So each
+// context has a pool without it; a stream reuses its own memory.  Three streams in turn, us per call: 64 x 64
+// 54 -> 7, 64 x 256 108 -> 8, 512 x 256 83 -> 14, 2048 x 1024 158 -> 158; one stream the same.  The pool gives back
+// at the same points as the device's: it follows that pool's threshold (zero unless the program raised it), up
+// to kKeep.  Null: the device's pool.
+cudaMemPool_t scratch_pool() {
+  struct Entry {
+    unsigned long long context;
+    cudaMemPool_t pool;
+    uint64_t threshold;
+  };
+  constexpr int kMost = 64;
+  constexpr uint64_t kKeep = 64ull << 20;
+  static std::mutex mu;
+  static Entry entries[kMost];
+  static int n = 0;
+  unsigned long long id = 0;
+  int dev = -1;
+  if (!current_context_id(&id) || cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+  cudaMemPool_t devices = nullptr;
+  uint64_t threshold = 0;
+  if (cudaDeviceGetMemPool(&devices, dev) != cudaSuccess ||
+      cudaMemPoolGetAttribute(devices, cudaMemPoolAttrReleaseThreshold, &threshold) != cudaSuccess)
+    return nullptr;
+  threshold = std::min(threshold, kKeep);
+  std::lock_guard<std::mutex> g(mu);
+  Entry* e = std::find_if(entries, entries + n, [&](const Entry& x) { return x.context == id; });
+  if (e == entries + n) {
+    if (n == kMost) return nullptr;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    int off = 0;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+      pool = nullptr;
+    } else if (cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowOpportunistic, &off) != cudaSuccess) {
+      cudaMemPoolDestroy(pool);
+      pool = nullptr;
+    }
+    cudaGetLastError();
+    *e = Entry{id, pool, 0};
+    ++n;
+  }
+  if (e->pool && e->threshold != threshold &&
+      cudaMemPoolSetAttribute(e->pool, cudaMemPoolAttrReleaseThreshold, &threshold) == cudaSuccess)
+    e->threshold = threshold;
+  return e->pool;
+}
 }  // namespace
+
+// From scratch_pool, else from the device's pool (also where the first cannot get the memory, which the other may
+// hold); freed with cudaFreeAsync.  A stream that is being captured takes its scratch from the graph: there the
+// pools, which a capture does not let be made or asked, play no part.
+cudaError_t scratch_malloc(void** p, size_t bytes, cudaStream_t s) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  const bool free_stream = cudaStreamIsCapturing(s, &status) == cudaSuccess && status == cudaStreamCaptureStatusNone;
+  cudaMemPool_t pool = free_stream ? scratch_pool() : nullptr;
+  if (pool && cudaMallocFromPoolAsync(p, bytes, pool, s) == cudaSuccess) return cudaSuccess;
+  cudaGetLastError();
+  return cudaMallocAsync(p, bytes, s);
+}
 
 // The kernels' attributes, once per context (in every call where the context cannot be told or too many have
 // been seen: the same values again).
@@ -2236,7 +2301,7 @@ int lb_power_spectrum(const double* field, int Lx, int Lz, double* out, void* st
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   void* tmp = nullptr;
-  if (cudaMallocAsync(&tmp, (size_t)sf_half(Lx) * Lz * 2 * sizeof(double), s) != cudaSuccess) {
+  if (scratch_malloc(&tmp, (size_t)sf_half(Lx) * Lz * 2 * sizeof(double), s) != cudaSuccess) {
     cudaGetLastError();
     return LB_ERR_OOM;
   }
