@@ -496,8 +496,8 @@ __global__ void adj_gather_push_kernel(const LatticeDev<real>* lat, const RowCon
 
 // ---- the default options (a*, copy-rule ghosts, hom noise) ----------------------------------------
 // The transposed step is bound by the FP64 pipe (two lanes per clock and SM), so these kernels are
-// arranged for the fewest FP64 instructions: about 355 per site and step against about 1000 of the
-// kernels above, which remain for the other options.
+// arranged for the fewest FP64 instructions: about 320 per site and step (280 in the local pass, 43 in the
+// gather) against about 1000 of the kernels above, which remain for the other options.
 //  - what both species share is formed once from their density-weighted sums T_a = sum_s rho^S t^S_a;
 //  - with a* the sensitivities of m^eq and of the source act on the same combinations of the moments,
 //    so one dot product per species (K_1 .. K_5) gives both shares of rho^S;

@@ -6,10 +6,11 @@
 
 namespace lbk {
 
-// One warp per block: the transposed step runs at about 166 registers, so a lattice of a few
-// ten thousand sites is fewer threads than the GPU holds, and the smallest blocks spread them
-// most evenly over the SMs (measured on 256 x 128: 32 threads 0.476 s per gradient, 128
-// threads 0.504 s).
+// One warp per block: the transposed step takes many registers (128 a thread for the default options,
+// bound there, with 16 to 80 bytes spilled; 152 to 184 for the others), so a lattice of a few ten thousand
+// sites is fewer threads than the GPU holds, and the smallest blocks spread them most evenly over the SMs
+// (measured on 256 x 128 with the kernels of every option: 32 threads 0.476 s per gradient, 128 threads
+// 0.504 s).
 constexpr int kAdjBlock = 32;
 inline int adjoint_blocks(int n_sites) { return (n_sites + kAdjBlock - 1) / kAdjBlock; }
 

@@ -5,7 +5,9 @@
 // them to integers of one scale, combine those exactly, and round once on the way back.  The scale puts
 // the largest magnitude's leading bit at bit 57, so a sum of up to 32 of them fits, and values are
 // rounded at 2^-58 of the largest: far below the roundings of the same sums in double (2^-53 of each
-// partial sum) whatever the values.  (Cut instead of rounded, and at 2^-55, the error after 100 steps
+// partial sum) for every sum that contains the largest value.  Here that is the density, which every link
+// contains, unless the flow is far from anything the method describes; a link that lacked the largest value
+// could be rounded coarser than in double.  (Cut instead of rounded, and at 2^-55, the error after 100 steps
 // was six times that of the double sums: a bias of a fraction of a bit adds up from step to step.)
 // Groups with an infinity or a NaN, above 2^1008 or below 2^-950 are left to the caller's double
 // arithmetic.
