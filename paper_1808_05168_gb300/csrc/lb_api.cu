@@ -168,6 +168,18 @@ int cuda_err(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? LB_ERR_OOM : LB_ERR_CUDA;
 }
 
+// Copies and clears outside lb_step go through the legacy stream, and calls for them may return before the device
+// has done them (clears, and copies from pageable memory).  The context's stream does not wait for the legacy
+// one, so whoever set something up waits here.
+int set_up_done() { return cudaStreamSynchronize(nullptr) == cudaSuccess ? LB_OK : LB_ERR_CUDA; }
+
+// The error flag, once it has been seen.
+int clear_flag(int* d_err) {
+  const cudaError_t e = cudaMemset(d_err, 0, sizeof(int));
+  const int rc = set_up_done();
+  return e == cudaSuccess ? rc : LB_ERR_CUDA;
+}
+
 int check_params(const lb_params& p) {
   auto rate_ok = [](double l) { return std::isfinite(l) && l > 0.0 && l < 2.0; };
   if (p.Lx < 1 || p.Lz < 2) return LB_ERR_BAD_PARAM;
@@ -538,7 +550,8 @@ int build_items(lb_ctx* c, int tile_x, int rows) {
   c->rows_per_item = rows;
   c->coop_grid = -1;
   drop_graphs(c);
-  return build_tmaps(c, tile_x);
+  rc = build_tmaps(c, tile_x);
+  return rc ? rc : set_up_done();
 }
 
 int alloc_diag(lb_ctx* c) {
@@ -589,6 +602,8 @@ int alloc_diag(lb_ctx* c) {
   if (cudaMemset(c->acc_sum, 0, 4 * (size_t)c->n_sites * sizeof(double)) != cudaSuccess ||
       cudaMemset(c->acc_comp, 0, 4 * (size_t)c->n_sites * sizeof(double)) != cudaSuccess)
     return LB_ERR_CUDA;
+  rc = set_up_done();
+  if (rc) return rc;
   c->diag_ready = true;
   return LB_OK;
 }
@@ -1058,7 +1073,7 @@ int create_impl(lb_ctx** out, int n, const lb_params* ps, int flags, lb_alloc_fn
     }
     // everything above is on the legacy stream; the device's other streams are not waited for (a gradient call
     // makes a context too)
-    if (!rc && cudaStreamSynchronize(nullptr) != cudaSuccess) rc = LB_ERR_CUDA;
+    if (!rc) rc = set_up_done();
   }
   if (rc) {
     lb_destroy(c);
@@ -1074,7 +1089,7 @@ int sync_and_check(lb_ctx* c) {
   int err = 0;
   if (cudaMemcpy(&err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return LB_ERR_CUDA;
   if (err) {
-    cudaMemset(c->d_err, 0, sizeof(int));
+    clear_flag(c->d_err);
     return LB_ERR_TIMEOUT;
   }
   return LB_OK;
@@ -1104,7 +1119,7 @@ int read_result(lb_ctx* c, double* host, size_t n, Launch launch) {
   }
   if (e != cudaSuccess || cudaStreamSynchronize(c->stream) != cudaSuccess) return LB_ERR_CUDA;
   if ((n <= kOneCopy ? h[n] : flag) != 0.0) {  // the caller's buffer is as it was
-    cudaMemset(c->d_err, 0, sizeof(int));
+    clear_flag(c->d_err);
     return LB_ERR_TIMEOUT;
   }
   if (n <= kOneCopy) {
@@ -1439,6 +1454,7 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
     }
     if (want_grad) ok(cudaMemcpy(R.kcs, R.hkcs.data(), (size_t)n * sizeof(AdjConst), cudaMemcpyHostToDevice));
   }
+  if (set_up_done() != LB_OK) ok(cudaErrorUnknown);  // the tables of both runs
   ok(cudaMemsetAsync(d_grad, 0, (size_t)6 * n * sizeof(double), st));
   ok(cudaEventRecord(ev[0], st));  // the second run's stream starts after the set-up
   ok(cudaStreamWaitEvent(s1, ev[0], 0));
@@ -1639,7 +1655,7 @@ int pressure_shift_impl(lb_ctx* c, int64_t T, int64_t C, double* grads, double* 
   }
   int err = 0;
   if (cudaMemcpy(&err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess && err) {
-    cudaMemset(c->d_err, 0, sizeof(int));
+    clear_flag(c->d_err);
     return LB_ERR_TIMEOUT;
   }
   return LB_OK;
@@ -1879,6 +1895,11 @@ int lb_set_correlations(lb_ctx* c, int field_mask, int n_modes, const int* modes
     corr_free(c);
     return LB_ERR_CUDA;
   }
+  rc = set_up_done();
+  if (rc) {
+    corr_free(c);
+    return rc;
+  }
   c->corr_mask = field_mask;
   return LB_OK;
 }
@@ -2055,7 +2076,7 @@ int lb_set_site_map(lb_ctx* c, int lattice, int x0, int Lx_global) {
     if (cudaMemcpy((LatticeDev<double>*)c->d_lat + lattice, &L, sizeof(L), cudaMemcpyHostToDevice) != cudaSuccess)
       return LB_ERR_CUDA;
   }
-  return LB_OK;
+  return set_up_done();
 }
 
 namespace {
@@ -2225,7 +2246,7 @@ int lb_load_checkpoint(lb_ctx* c, const void* host_buf, size_t bytes) {
                               (c->corr_C_n == 0 || to_device(c->corr_C, c->corr_C_n * sizeof(double)));
   // the step count, on the host and in the device counter
   if (ok) ok = cudaMemcpy(c->d_t, &h.t, sizeof(int64_t), cudaMemcpyHostToDevice) == cudaSuccess;
-  if (!ok) return LB_ERR_CUDA;
+  if (!ok || set_up_done() != LB_OK) return LB_ERR_CUDA;
   c->t = h.t;
   c->nsamples = h.nsamples;
   c->corr_samples = h.corr_samples;
@@ -2250,7 +2271,7 @@ int lb_reset_statistics(lb_ctx* c) {
   if ((c->corr_R && cudaMemset(c->corr_R, 0, c->corr_R_n * sizeof(double)) != cudaSuccess) ||
       (c->corr_C && cudaMemset(c->corr_C, 0, c->corr_C_n * sizeof(double)) != cudaSuccess))
     return LB_ERR_CUDA;
-  return LB_OK;
+  return set_up_done();
 }
 
 int lb_kernel_launches(lb_ctx* c, int64_t* n) {
