@@ -129,7 +129,8 @@ int lb_set_stream(lb_ctx* ctx, void* cuda_stream);
 int lb_set_sampling(lb_ctx* ctx, int64_t discard, int64_t every);
 
 /* Fix the tile shape: tile_x columns per block (32, 64, 128 or 256) and rows_per_item rows
- * per work item (>= 1; larger values are clipped to Lz).  Overrides LB_AUTOTUNE. */
+ * per work item (>= 1; larger values are clipped to Lz).  Overrides LB_AUTOTUNE.  Waits for the
+ * context's stream. */
 int lb_set_tile(lb_ctx* ctx, int tile_x, int rows_per_item);
 int lb_get_tile(lb_ctx* ctx, int* tile_x, int* rows_per_item);
 
@@ -274,7 +275,9 @@ int lb_power_spectrum_noalloc(const double* field, int Lx, int Lz, double* out, 
  * streams (the context's and one of the call's own), each with its own buffers; the noiseless one,
  * uniform in x, on two columns.  Device memory: about steps/ckpt_every + 1.4 ckpt_every + 8 states
  * (default options without the gradient: 33 states, 1 GB at most where two are less), allocated for
- * the call and freed before it returns.  Synchronous. */
+ * the call and freed before it returns.  Synchronous: it waits for its own work and for the legacy
+ * stream, and for the whole device only where the library allocates itself (cudaFree waits for it;
+ * not with lb_create_batch_with_allocator). */
 int lb_pressure_shift_gradient(lb_ctx* ctx, int64_t steps, int64_t ckpt_every, double grad[3], double* loss);
 
 /* lb_pressure_shift_gradient for every lattice of a batch in one sweep: each lattice's own loss
